@@ -224,9 +224,7 @@ int ensure_query(cfpq_ctx *ctx, bool restricted = false) {
 }
 
 int bits_to_host(cfpq_ctx *ctx, const uint64_t *dev_rows, uint32_t n, uint32_t W, uint64_t *bits) {
-    const size_t wn = (n + 63) / 64;
-    CK(ctx, cudaMemcpy2DAsync(bits, wn * 8, dev_rows, (size_t)W * 8, wn * 8, n, cudaMemcpyDeviceToHost, ctx->stream));
-    CK(ctx, cudaStreamSynchronize(ctx->stream));
+    CK(ctx, rows_to_host(&ctx->A, dev_rows, n, W, bits, ctx->stream));
     return CFPQ_OK;
 }
 

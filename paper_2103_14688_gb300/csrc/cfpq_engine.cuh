@@ -76,6 +76,8 @@ cudaError_t launch_stage_compact(const uint32_t *off, const uint32_t *col, const
 cudaError_t launch_popcount(const uint64_t *p, size_t nwords, unsigned long long *out, cudaStream_t st);
 cudaError_t launch_nonempty_bits(const uint32_t *off, uint32_t n, uint32_t n_term, uint32_t W, uint64_t *bits,
                                  cudaStream_t st);
+cudaError_t launch_pack_rows(const uint64_t *src, uint32_t W, uint32_t wn, uint32_t r0, uint32_t rows, uint64_t *out,
+                             cudaStream_t st);
 cudaError_t launch_copy_rows(const uint64_t *const *ptrs, const uint32_t *rows, uint32_t njobs, uint32_t W,
                              uint64_t *out, cudaStream_t st);
 
@@ -390,6 +392,10 @@ struct PathsDev {
                      uint32_t T, uint32_t L, std::vector<uint64_t> *out, std::string *err);
 };
 
+// Copy an n x n bit matrix (rows of W words) to host rows of ceil(n / 64)
+// words and wait for it.
+cudaError_t rows_to_host(Allocator *A, const uint64_t *dev_rows, uint32_t n, uint32_t W, uint64_t *bits,
+                         cudaStream_t st);
 int stage_graph(GraphDev *g, Allocator *A, cudaStream_t st, uint32_t n, uint32_t n_term, size_t m, const uint32_t *src,
                 const uint32_t *lbl, const uint32_t *dst, bool device_ptrs, std::string *err);
 

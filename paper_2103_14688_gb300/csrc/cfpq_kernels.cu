@@ -1265,6 +1265,17 @@ __global__ void k_copy_rows(const uint64_t *const *__restrict__ ptrs, const uint
     }
 }
 
+// Rows [r0, r0 + rows) of a bit matrix without their padding word: wn < W words
+// each, back to back (a linear write, 8 bytes a thread; bound by HBM, and two
+// orders below the host copy that follows).
+__global__ void k_pack_rows(const uint64_t *__restrict__ src, uint32_t W, uint32_t wn, uint32_t r0, size_t words,
+                            uint64_t *__restrict__ out) {
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += (size_t)gridDim.x * blockDim.x) {
+        const size_t r = i / wn;
+        out[i] = src[(r0 + r) * W + (i - r * wn)];
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Host launchers.
 // ---------------------------------------------------------------------------
@@ -1449,6 +1460,13 @@ cudaError_t launch_nonempty_bits(const uint32_t *off, uint32_t n, uint32_t n_ter
 cudaError_t launch_popcount(const uint64_t *p, size_t nwords, unsigned long long *out, cudaStream_t st) {
     if (nwords == 0) return cudaSuccess;
     k_popcount<<<grid_for(nwords, 256, 2048), 256, 0, st>>>(p, nwords, out);
+    return cudaGetLastError();
+}
+cudaError_t launch_pack_rows(const uint64_t *src, uint32_t W, uint32_t wn, uint32_t r0, uint32_t rows, uint64_t *out,
+                             cudaStream_t st) {
+    const size_t words = (size_t)rows * wn;
+    if (words == 0) return cudaSuccess;
+    k_pack_rows<<<grid_for(words, 256, 2048), 256, 0, st>>>(src, W, wn, r0, words, out);
     return cudaGetLastError();
 }
 cudaError_t launch_copy_rows(const uint64_t *const *ptrs, const uint32_t *rows, uint32_t njobs, uint32_t W,

@@ -233,10 +233,7 @@ int cfpq_result_reachable_bits(cfpq_server *s, uint64_t ticket, uint32_t box, ui
     if (j.state != kDone) return sfail(s, CFPQ_ERR_NOT_READY, "query not finished");
     if (box >= j.q->B) return sfail(s, CFPQ_ERR_INVALID_ARG, "box out of range");
     SCK(s, cudaSetDevice(s->opt.device));
-    const size_t wn = (j.q->n + 63) / 64;
-    SCK(s, cudaMemcpy2DAsync(bits, wn * 8, j.q->m2_ptr(box), (size_t)j.q->W * 8, wn * 8, j.q->n,
-                             cudaMemcpyDeviceToHost, s->stream));
-    SCK(s, cudaStreamSynchronize(s->stream));
+    SCK(s, rows_to_host(&s->A, j.q->m2_ptr(box), j.q->n, j.q->W, bits, s->stream));
     return j.status;
 }
 

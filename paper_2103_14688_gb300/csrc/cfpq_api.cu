@@ -374,7 +374,10 @@ int cfpq_run(cfpq_ctx *ctx, cfpq_run_stats *stats) {
     ClosureProfile prof;
     if (ctx->query.small_ok && ctx->opt.loop_mode == CFPQ_LOOP_DEVICE) {
         // the whole fixpoint in one CTA (state in shared memory)
-        CK(ctx, launch_small_fixpoint(ctx->query.small_desc.p, 1, ctx->query.small_smem, ctx->stream));
+        const QueryDev &q = ctx->query;
+        CK(ctx, launch_small_fixpoint(q.small_desc.p, q.W, q.small_smem, q.small_meta,
+                                      (uint64_t)ctx->graph.n_term * ctx->graph.n, ctx->graph.m_unique, q.small_items,
+                                      ctx->stream));
         ctls.resize(1);
         CK(ctx, cudaMemcpyAsync(ctls.data(), ctx->query.ctl(), sizeof(QCtl), cudaMemcpyDeviceToHost, ctx->stream));
         CK(ctx, cudaStreamSynchronize(ctx->stream));

@@ -90,19 +90,16 @@ cudaError_t launch_shard_apply(const uint64_t *full, uint64_t *m2, uint64_t *a2,
                                uint32_t *box_new_it, cudaStream_t st);
 
 // ---- single-CTA fixpoint (cfpq_small.cu) ----
-struct SmallSrc;
+struct QueryDev;
 size_t small_smem_bytes(uint32_t n, uint32_t W, uint32_t B, uint32_t nblk);
 size_t small_desc_size();
-size_t small_src_size();
 size_t small_smem_limit();
-cudaError_t launch_small_fixpoint(const void *descs, uint32_t count, size_t smem, cudaStream_t st);
-void build_small_desc(void *desc_out, uint32_t n, uint32_t W, uint32_t B, uint32_t nblk, uint32_t n_levels,
-                      unsigned long long cyclic_mask, uint32_t max_iter, uint32_t max_passes,
-                      const uint32_t *dev_arrays, const SmallSrc *dev_srcs, size_t off_level, size_t off_src0,
-                      size_t off_nsrc, size_t off_f0, size_t off_nf, size_t off_fb, size_t off_null,
-                      const uint32_t *csr_off, const uint32_t *csr_col, uint64_t *blk_out, uint64_t *m2_out,
-                      QCtl *ctl);
-void fill_small_src(void *dst, uint32_t kind, uint32_t label, uint32_t ident, uint32_t same_level, int32_t rblk);
+cudaError_t launch_small_fixpoint(const void *desc, uint32_t W, size_t state_smem, size_t meta_bytes, uint64_t csr_rows,
+                                  uint64_t csr_m, uint32_t max_items, cudaStream_t st);
+std::vector<uint32_t> build_small_plan(const QueryDev &q, void *desc_out);
+void finish_small_desc(void *desc, const uint32_t *meta, uint32_t max_iter, uint32_t max_passes,
+                       const uint32_t *csr_off, const uint32_t *csr_col, uint64_t *blk_out, uint64_t *m2_out,
+                       QCtl *ctl);
 
 // ---- device memory ----
 struct Allocator {
@@ -277,7 +274,8 @@ struct QueryDev {
     int enqueue_init(cudaStream_t st, uint32_t max_iter, uint32_t max_rounds, uint32_t max_passes);
     // single-CTA path: eligible when rows are <= 512 bits and the state fits one SM
     DBuf small_arrays, small_desc;
-    size_t small_smem = 0;
+    size_t small_smem = 0, small_meta = 0;  // bytes of the state, of the plan's tables
+    uint32_t small_items = 0;               // rows of the largest level
     bool small_ok = false;
     int prepare_small(Allocator *A, cudaStream_t st, uint32_t max_iter, uint32_t max_passes, std::string *err);
     QCtl *ctl() const { return ctl_mem.as<QCtl>(); }

@@ -4,7 +4,7 @@
 // shared memory of one SM, the index-creation loop of Listing 1 (arXiv
 // 2103.14688, Sec. 3.1) runs inside a single CTA: the same level schedule,
 // edge channels and dirty stamps as the multi-kernel path (cfpq_kernels.cu),
-// with __syncthreads between passes instead of kernel launches.  Rows are at
+// with a barrier between passes instead of kernel launches.  Rows are at
 // most 512 bits wide (W <= 8 words), so each thread owns one output row per
 // step and keeps it in registers.  At the end the closure blocks and M2 are
 // copied to the query's global buffers, where every result call reads them.
@@ -12,25 +12,39 @@
 #include <stdint.h>
 #include <string.h>
 
-#include "cfpq_dev.cuh"
+#include <vector>
+
+#include "cfpq_engine.cuh"
 
 namespace cfpq {
 
 constexpr uint32_t kSmallMaxW = 8;
-constexpr int kSmallThreads = 512;
+constexpr int kSmallMaxThreads = 512;  // 128 registers a thread: 1024 threads would spill
 
-struct SmallSrc {
-    uint32_t kind, label, ident, same_level;
+// One source of a block (SrcDesc without the pointers), read as one 16-byte
+// shared-memory load.
+struct alignas(16) SmallSrc {
+    uint32_t kind, label;
+    uint32_t flags;  // bit 0: ident, bit 1: same level
     int32_t rblk;
-    uint32_t pad;
+};
+
+// One level: its blocks lvl_blk[blk0 .. blk0 + nblk), and what its first pass
+// of an iteration reads: the boxes of its nonterminal sources, the levels
+// below that its sources read blocks of, whether it has terminal sources.
+struct alignas(16) SmallLevel {
+    uint32_t blk0, nblk, has_term, any_box;  // any_box: a nonterminal source of a box >= 64
+    unsigned long long boxes, reads;
 };
 
 struct SmallDesc {
-    uint32_t n, W, B, nblk, n_levels, max_iter, max_passes, pad;
+    uint32_t n, W, B, nblk, n_levels, max_iter, max_passes;
+    uint32_t magic;           // ceil(2^32 / n): item / n = umulhi(item, magic) while item * n < 2^32; 0 for n = 1
+    uint32_t meta_words;      // words of the plan's tables at `meta` (a multiple of 4)
+    uint32_t o_srcs, o_blk, o_src0, o_nsrc, o_f0, o_nf, o_null, o_fb;  // word offsets in `meta` (levels at 0)
+    uint32_t pad;
     unsigned long long cyclic_mask;
-    const uint32_t *blk_level, *blk_src0, *blk_nsrc;
-    const SmallSrc *srcs;
-    const uint32_t *box_f0, *box_nf, *fblocks, *box_nullable;
+    const uint32_t *meta;
     const uint32_t *csr_off;  // label l, vertex x: csr_off[l * n + x] .. csr_off[l * n + x + 1]
     const uint32_t *csr_col;
     uint64_t *blk_out;        // nblk * n * W
@@ -38,10 +52,28 @@ struct SmallDesc {
     QCtl *ctl;                // statistics written at the end
 };
 
-__global__ void __launch_bounds__(kSmallThreads) k_small_fixpoint(const SmallDesc *__restrict__ descs) {
-    const SmallDesc D = descs[blockIdx.x];
-    const uint32_t n = D.n, W = D.W, B = D.B, nblk = D.nblk;
-    extern __shared__ uint64_t sm[];
+// Latency-bound: a query of this size holds a few thousand row words, and its
+// fixpoint is a chain of thousands of dependent passes (two coprime cycles of
+// 63 and 64 vertices: 4033 iterations, 12099 passes).  So what a pass costs
+// is counted in barriers and in dependent shared-memory loads:
+//   - the plan's tables and the graph's CSR are copied to shared memory when
+//     they fit beside the state (`meta_smem`, `csr_smem`);
+//   - a level whose first pass has nothing to read in this iteration (no new
+//     terminal or box edge, no lower level that changed) is counted and passed
+//     over without a barrier: what decides it is the same in every thread
+//     (register masks of the boxes and levels that changed);
+//   - a pass has one barrier, which also carries the "some row changed" flag;
+//     counters stay in registers until the end.
+// Two cycles 63 / 64: 23.1 -> 11.3 ms (1.9 us a pass before, with four barriers,
+// divisions and table loads from global memory); the regular query
+// (ab)*c|a*b* at n = 200: 620 -> 165 us.
+template <uint32_t W>
+__global__ void __launch_bounds__(kSmallMaxThreads, 1)
+    k_small_fixpoint(const SmallDesc *__restrict__ desc, uint32_t meta_smem, uint32_t csr_smem, uint32_t csr_rows,
+                     uint32_t csr_m) {
+    const SmallDesc &D = *desc;
+    const uint32_t n = D.n, B = D.B, nblk = D.nblk;
+    extern __shared__ __align__(16) uint64_t sm[];
     uint64_t *C = sm;
     uint64_t *M2 = C + (size_t)nblk * n * W;
     uint64_t *A2 = M2 + (size_t)B * n * W;
@@ -49,27 +81,51 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_fixpoint(const SmallDes
     uint32_t *last = stamp + (size_t)nblk * n;
     uint32_t *a2it = last + nblk;
     uint32_t *boxit = a2it + (size_t)B * n;
-    __shared__ uint32_t s_changed;
+    const uint32_t words32 = nblk * n + nblk + B * n + B;
     __shared__ unsigned long long s_new, s_ors, s_rows;
     const uint32_t tid = threadIdx.x, T = blockDim.x;
 
-    const size_t words64 = (size_t)(nblk + 2 * B) * n * W;
-    for (size_t i = tid; i < words64; i += T) sm[i] = 0ull;
-    const size_t words32 = (size_t)nblk * n + nblk + (size_t)B * n + B;
-    for (size_t i = tid; i < words32; i += T) stamp[i] = 0u;
-    if (tid == 0) { s_ors = 0; s_rows = 0; }
+    const uint32_t words64 = (nblk + 2u * B) * n * W;
+    for (uint32_t i = tid; i < words64; i += T) sm[i] = 0ull;
+    for (uint32_t i = tid; i < words32; i += T) stamp[i] = 0u;
+    uint32_t *extra = stamp + ((words32 + 3u) & ~3u);  // 16-byte aligned: the tables, then the CSR
+    const uint32_t *meta = D.meta;
+    if (meta_smem) {
+        for (uint32_t i = tid; i < D.meta_words; i += T) extra[i] = D.meta[i];
+        meta = extra;
+        extra += D.meta_words;
+    }
+    const uint32_t *csr_off = D.csr_off, *csr_col = D.csr_col;
+    if (csr_smem) {
+        for (uint32_t i = tid; i <= csr_rows; i += T) extra[i] = D.csr_off[i];
+        for (uint32_t i = tid; i < csr_m; i += T) extra[csr_rows + 1u + i] = D.csr_col[i];
+        csr_off = extra;
+        csr_col = extra + csr_rows + 1u;
+    }
+    if (tid == 0) { s_new = 0; s_ors = 0; s_rows = 0; }
     __syncthreads();
-    unsigned long long edges_total = 0;
+    const SmallLevel *levels = reinterpret_cast<const SmallLevel *>(meta);
+    const SmallSrc *srcs = reinterpret_cast<const SmallSrc *>(meta + D.o_srcs);
+    const uint32_t *lvl_blk = meta + D.o_blk, *blk_src0 = meta + D.o_src0, *blk_nsrc = meta + D.o_nsrc;
+    const uint32_t *box_f0 = meta + D.o_f0, *box_nf = meta + D.o_nf, *nullable = meta + D.o_null;
+    const uint32_t *fblocks = meta + D.o_fb;
+
+    unsigned long long edges_eps = 0, my_new = 0;
+    unsigned long long new_boxes = 0;  // boxes (< 64) with edges new in this iteration
+    bool new_any = false;              // some box has
+    uint32_t my_ors = 0, my_rows = 0;
     // epsilon rows: M2^b[i,i] = A2^b[i,i] = 1 for boxes whose start state is final
     for (uint32_t b = 0; b < B; ++b) {
-        if (!D.box_nullable[b]) continue;
+        if (!nullable[b]) continue;
         for (uint32_t x = tid; x < n; x += T) {
-            M2[((size_t)b * n + x) * W + (x >> 6)] |= 1ull << (x & 63);
-            A2[((size_t)b * n + x) * W + (x >> 6)] = 1ull << (x & 63);
-            a2it[(size_t)b * n + x] = 1;
+            M2[(b * n + x) * W + (x >> 6)] = 1ull << (x & 63);
+            A2[(b * n + x) * W + (x >> 6)] = 1ull << (x & 63);
+            a2it[b * n + x] = 1;
         }
         if (tid == 0) boxit[b] = 1;
-        edges_total += n;
+        edges_eps += n;
+        new_any = true;
+        if (b < 64u) new_boxes |= 1ull << b;
     }
     __syncthreads();
 
@@ -77,59 +133,69 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_fixpoint(const SmallDes
     bool done = false;
     while (!done) {
         const uint32_t g0 = g;
+        unsigned long long lvl_changed = 0;  // levels that changed in this iteration
         for (uint32_t L = 0; L < D.n_levels && !done; ++L) {
+            const SmallLevel lv = levels[L];
+            const bool cyc = (D.cyclic_mask >> L) & 1ull;
+            bool active = (iter == 1u && lv.has_term) || (lv.boxes & new_boxes) != 0ull || (lv.any_box && new_any) ||
+                          (lv.reads & lvl_changed) != 0ull;
             uint32_t mode = kModeNew;
             while (true) {
-                if (tid == 0) s_changed = 0;
-                __syncthreads();
-                uint32_t my_ors = 0, my_rows = 0;
-                for (uint32_t item = tid; item < nblk * n; item += T) {
-                    const uint32_t b = item / n, x = item - b * n;
-                    if (D.blk_level[b] != L) continue;
-                    uint64_t acc[kSmallMaxW];
+                bool ch_any = false;
+                const uint32_t items = active ? lv.nblk * n : 0u;
+                for (uint32_t item = tid; item < items; item += T) {
+                    const uint32_t bi = D.magic ? __umulhi(item, D.magic) : item, x = item - bi * n;
+                    const uint32_t b = lvl_blk[lv.blk0 + bi];
+                    uint64_t acc[W];
 #pragma unroll
-                    for (uint32_t w = 0; w < kSmallMaxW; ++w) acc[w] = 0ull;
-                    for (uint32_t k = 0; k < D.blk_nsrc[b]; ++k) {
-                        const SmallSrc s = D.srcs[D.blk_src0[b] + k];
+                    for (uint32_t w = 0; w < W; ++w) acc[w] = 0ull;
+                    bool any = false;
+                    const uint32_t k0 = blk_src0[b], k1 = k0 + blk_nsrc[b];
+                    for (uint32_t k = k0; k < k1; ++k) {
+                        const SmallSrc s = srcs[k];
                         uint32_t chans = 0;
                         if (mode == kModeNew) {
                             const bool term1 = s.kind == 0 && iter == 1;
                             if (term1 || (s.kind == 1 && boxit[s.label] == iter)) chans |= 1u;
-                            if (s.rblk >= 0 && !s.same_level && !term1 && last[s.rblk] >= g0) chans |= 2u;
-                        } else if (s.rblk >= 0 && s.same_level && last[s.rblk] + 1u >= g) {
+                            if (s.rblk >= 0 && !(s.flags & 2u) && !term1 && last[s.rblk] >= g0) chans |= 2u;
+                        } else if (s.rblk >= 0 && (s.flags & 2u) && last[s.rblk] + 1u >= g) {
                             chans |= 4u;
                         }
-                        for (uint32_t cb = 1u; cb <= 4u; cb <<= 1) {
+                        for (uint32_t cb = 1u; cb <= chans; cb <<= 1) {
                             if (!(chans & cb)) continue;
                             const bool new_edges = cb == 1u;
-                            const bool ident = new_edges && s.ident;
+                            const bool ident = new_edges && (s.flags & 1u);
                             if (!ident && s.rblk < 0) continue;
                             const uint32_t thr = new_edges ? 0u : (cb == 2u ? g0 : g - 1u);
+                            const uint32_t *rstamp = stamp + (s.rblk >= 0 ? (uint32_t)s.rblk * n : 0u);
+                            const uint64_t *rrow = C + (s.rblk >= 0 ? (uint32_t)s.rblk * n * W : 0u);
                             auto take = [&](uint32_t y) {
                                 if (ident) {
 #pragma unroll
-                                    for (uint32_t w = 0; w < kSmallMaxW; ++w)
+                                    for (uint32_t w = 0; w < W; ++w)
                                         if (w == (y >> 6)) acc[w] |= 1ull << (y & 63);
+                                    any = true;
                                 }
-                                if (s.rblk >= 0 && (thr == 0u || stamp[(size_t)s.rblk * n + y] >= thr)) {
-                                    const uint64_t *r = C + ((size_t)s.rblk * n + y) * W;
+                                if (s.rblk >= 0 && (thr == 0u || rstamp[y] >= thr)) {
+                                    const ulonglong2 *r = reinterpret_cast<const ulonglong2 *>(rrow + y * W);
 #pragma unroll
-                                    for (uint32_t w = 0; w < kSmallMaxW; ++w)
-                                        if (w < W) acc[w] |= r[w];
+                                    for (uint32_t w = 0; w < W / 2; ++w) {
+                                        const ulonglong2 v = r[w];
+                                        acc[2 * w] |= v.x;
+                                        acc[2 * w + 1] |= v.y;
+                                    }
+                                    any = true;
                                     ++my_ors;
                                 }
                             };
                             if (s.kind == 0) {
-                                const uint32_t *off = D.csr_off + (size_t)s.label * n;
-                                for (uint32_t e = off[x]; e < off[x + 1]; ++e) take(D.csr_col[e]);
+                                const uint32_t *off = csr_off + s.label * n + x;
+                                const uint32_t e1 = off[1];
+                                for (uint32_t e = off[0]; e < e1; ++e) take(csr_col[e]);
                             } else {
-                                const uint64_t *adj;
-                                if (new_edges) {
-                                    if (a2it[(size_t)s.label * n + x] != iter) continue;
-                                    adj = A2 + ((size_t)s.label * n + x) * W;
-                                } else {
-                                    adj = M2 + ((size_t)s.label * n + x) * W;
-                                }
+                                if (new_edges && a2it[s.label * n + x] != iter) continue;
+                                const uint64_t *adj = (new_edges ? A2 : M2) + (s.label * n + x) * W;
+#pragma unroll 1
                                 for (uint32_t w = 0; w < W; ++w) {
                                     uint64_t bits = adj[w];
                                     while (bits) {
@@ -141,27 +207,26 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_fixpoint(const SmallDes
                             }
                         }
                     }
-                    uint64_t *o = C + ((size_t)b * n + x) * W;
+                    if (!any) continue;
+                    uint64_t *o = C + (b * n + x) * W;
                     bool ch = false;
 #pragma unroll
-                    for (uint32_t w = 0; w < kSmallMaxW; ++w) {
-                        if (w < W && (acc[w] & ~o[w])) {
-                            o[w] |= acc[w];
+                    for (uint32_t w = 0; w < W; ++w) {
+                        const uint64_t old = o[w];
+                        if (acc[w] & ~old) {
+                            o[w] = old | acc[w];
                             ch = true;
                         }
                     }
                     if (ch) {
-                        stamp[(size_t)b * n + x] = g;
+                        stamp[b * n + x] = g;
                         last[b] = g;
-                        s_changed = 1;
+                        ch_any = true;
                         ++my_rows;
                     }
                 }
-                if (my_ors) atomicAdd(&s_ors, (unsigned long long)my_ors);
-                if (my_rows) atomicAdd(&s_rows, (unsigned long long)my_rows);
-                __syncthreads();
-                const bool changed = s_changed != 0;
-                __syncthreads();  // every thread has read the flag before it is reset
+                const bool changed = active && __syncthreads_or(ch_any) != 0;
+                if (changed) lvl_changed |= 1ull << L;
                 ++passes;
                 g += 1;
                 if (passes >= D.max_passes) {
@@ -169,7 +234,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_fixpoint(const SmallDes
                     done = true;
                     break;
                 }
-                if (((D.cyclic_mask >> L) & 1ull) && changed) {
+                if (cyc && changed) {
                     mode = kModeProp;
                     continue;
                 }
@@ -178,65 +243,61 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_fixpoint(const SmallDes
         }
         if (done) break;
         // extraction: new = OR_f C[q0, f] & ~M2 on rows changed this iteration
-        if (tid == 0) s_new = 0;
-        __syncthreads();
-        unsigned long long my_new = 0;
+        bool has_new = false;
         for (uint32_t item = tid; item < B * n; item += T) {
-            const uint32_t b = item / n, x = item - b * n;
-            if (D.box_nf[b] == 0) continue;
-            uint64_t cand[kSmallMaxW];
+            const uint32_t b = D.magic ? __umulhi(item, D.magic) : item, x = item - b * n;
+            const uint32_t f0 = box_f0[b], f1 = f0 + box_nf[b];
+            uint64_t cand[W];
 #pragma unroll
-            for (uint32_t w = 0; w < kSmallMaxW; ++w) cand[w] = 0ull;
+            for (uint32_t w = 0; w < W; ++w) cand[w] = 0ull;
             bool any = false;
-            for (uint32_t f = 0; f < D.box_nf[b]; ++f) {
-                const uint32_t fb = D.fblocks[D.box_f0[b] + f];
-                if (stamp[(size_t)fb * n + x] < g0) continue;
+            for (uint32_t f = f0; f < f1; ++f) {
+                const uint32_t fb = fblocks[f];
+                if (stamp[fb * n + x] < g0) continue;
                 any = true;
-                const uint64_t *r = C + ((size_t)fb * n + x) * W;
+                const uint64_t *r = C + (fb * n + x) * W;
 #pragma unroll
-                for (uint32_t w = 0; w < kSmallMaxW; ++w)
-                    if (w < W) cand[w] |= r[w];
+                for (uint32_t w = 0; w < W; ++w) cand[w] |= r[w];
             }
             if (!any) continue;
-            uint64_t *m = M2 + ((size_t)b * n + x) * W;
-            uint64_t *a = A2 + ((size_t)b * n + x) * W;
+            uint64_t *m = M2 + item * W;
+            uint64_t *a = A2 + item * W;
             bool has = false;
 #pragma unroll
-            for (uint32_t w = 0; w < kSmallMaxW; ++w) {
-                if (w < W) {
-                    cand[w] &= ~m[w];
-                    has |= cand[w] != 0ull;
-                }
+            for (uint32_t w = 0; w < W; ++w) {
+                cand[w] &= ~m[w];
+                has |= cand[w] != 0ull;
             }
             if (!has) continue;
 #pragma unroll
-            for (uint32_t w = 0; w < kSmallMaxW; ++w) {
-                if (w < W) {
-                    a[w] = cand[w];
-                    m[w] |= cand[w];
-                    my_new += (unsigned long long)__popcll(cand[w]);
-                }
+            for (uint32_t w = 0; w < W; ++w) {
+                a[w] = cand[w];
+                m[w] |= cand[w];
+                my_new += (unsigned long long)__popcll(cand[w]);
             }
-            a2it[(size_t)b * n + x] = iter + 1;
+            a2it[item] = iter + 1;
             boxit[b] = iter + 1;
+            has_new = true;
         }
-        if (my_new) atomicAdd(&s_new, my_new);
-        __syncthreads();
-        const unsigned long long added = s_new;
-        __syncthreads();
+        const bool added = __syncthreads_or(has_new) != 0;
         iters_done = iter;
-        edges_total += added;
-        if (added == 0ull) break;
+        if (!added) break;
         if (D.max_iter && iter >= D.max_iter) {
             status = kStatusIterCap;
             break;
         }
         ++iter;
-        __syncthreads();
+        new_any = true;
+        new_boxes = 0ull;
+        for (uint32_t b = 0; b < B && b < 64u; ++b)
+            if (boxit[b] == iter) new_boxes |= 1ull << b;
     }
+    if (my_new) atomicAdd(&s_new, my_new);
+    if (my_ors) atomicAdd(&s_ors, (unsigned long long)my_ors);
+    if (my_rows) atomicAdd(&s_rows, (unsigned long long)my_rows);
     __syncthreads();
-    for (size_t i = tid; i < (size_t)nblk * n * W; i += T) D.blk_out[i] = C[i];
-    for (size_t i = tid; i < (size_t)B * n * W; i += T) D.m2_out[i] = M2[i];
+    for (uint32_t i = tid; i < nblk * n * W; i += T) D.blk_out[i] = C[i];
+    for (uint32_t i = tid; i < B * n * W; i += T) D.m2_out[i] = M2[i];
     if (tid == 0) {
         QCtl c;
         memset(&c, 0, sizeof(c));
@@ -246,7 +307,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_fixpoint(const SmallDes
         c.status = status;
         c.iters_done = iters_done;
         c.passes = passes;
-        c.edges_total = edges_total;
+        c.edges_total = edges_eps + s_new;
         c.row_ors = s_ors;
         c.rounds_total = passes;
         c.rows_changed_total = s_rows;
@@ -261,7 +322,6 @@ size_t small_smem_bytes(uint32_t n, uint32_t W, uint32_t B, uint32_t nblk) {
 }
 
 size_t small_desc_size() { return sizeof(SmallDesc); }
-size_t small_src_size() { return sizeof(SmallSrc); }
 
 // Largest dynamic shared memory a CTA may use on the current device.
 size_t small_smem_limit() {
@@ -271,51 +331,107 @@ size_t small_smem_limit() {
     return (size_t)v > 2048 ? (size_t)v - 2048 : 0;  // room for the static shared variables
 }
 
-cudaError_t launch_small_fixpoint(const void *descs, uint32_t count, size_t smem, cudaStream_t st) {
-    if (count == 0) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_small_fixpoint, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_small_fixpoint<<<count, kSmallThreads, smem, st>>>(static_cast<const SmallDesc *>(descs));
-    return cudaGetLastError();
+// The query's tables go to shared memory when they fit beside the state, and
+// then the graph's CSR (csr_rows offsets and csr_m columns).  threads: the
+// items of the largest level (one row each), at most 512 -- a barrier over
+// fewer warps is cheaper.
+cudaError_t launch_small_fixpoint(const void *desc, uint32_t W, size_t state_smem, size_t meta_bytes, uint64_t csr_rows,
+                                  uint64_t csr_m, uint32_t max_items, cudaStream_t st) {
+    size_t smem = (state_smem + 15) & ~(size_t)15;
+    const size_t limit = small_smem_limit();
+    const uint32_t meta_smem = smem + meta_bytes <= limit ? 1u : 0u;
+    if (meta_smem) smem += meta_bytes;
+    const uint64_t csr_bytes = (csr_rows + 1 + csr_m) * 4;
+    const uint32_t csr_smem = smem + csr_bytes <= limit ? 1u : 0u;
+    if (csr_smem) smem += csr_bytes;
+    const uint32_t threads = max_items >= (uint32_t)kSmallMaxThreads ? (uint32_t)kSmallMaxThreads
+                                                                     : (max_items < 64u ? 64u : (max_items + 31u) & ~31u);
+    auto run = [&](auto kernel) -> cudaError_t {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        kernel<<<1, threads, smem, st>>>(static_cast<const SmallDesc *>(desc), meta_smem, csr_smem, (uint32_t)csr_rows,
+                                         (uint32_t)csr_m);
+        return cudaGetLastError();
+    };
+    switch (W) {
+        case 2: return run(k_small_fixpoint<2>);
+        case 4: return run(k_small_fixpoint<4>);
+        case 6: return run(k_small_fixpoint<6>);
+        case 8: return run(k_small_fixpoint<8>);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
-// Host-side packing of one query's plan for the kernel: `blob` receives the
-// arrays, `desc` the descriptor with device addresses inside `dev_blob`.
-void build_small_desc(void *desc_out, uint32_t n, uint32_t W, uint32_t B, uint32_t nblk,
-                      uint32_t n_levels, unsigned long long cyclic_mask, uint32_t max_iter,
-                      uint32_t max_passes, const uint32_t *dev_arrays, const SmallSrc *dev_srcs,
-                      size_t off_level, size_t off_src0, size_t off_nsrc, size_t off_f0, size_t off_nf, size_t off_fb,
-                      size_t off_null, const uint32_t *csr_off, const uint32_t *csr_col, uint64_t *blk_out,
-                      uint64_t *m2_out, QCtl *ctl) {
+// Host-side packing of one query's plan: the tables the kernel reads (levels,
+// sources, blocks by level, boxes) as words, and the descriptor.
+std::vector<uint32_t> build_small_plan(const QueryDev &q, void *desc_out) {
+    const uint32_t nblk = (uint32_t)q.blocks.size();
+    std::vector<SmallLevel> lv(q.n_levels);
+    std::vector<SmallSrc> src;
+    std::vector<uint32_t> by_level;
+    for (uint32_t L = 0; L < q.n_levels; ++L) {
+        memset(&lv[L], 0, sizeof(SmallLevel));
+        lv[L].blk0 = (uint32_t)by_level.size();
+        for (uint32_t b = 0; b < nblk; ++b) {
+            if (q.blk_level[b] != L) continue;
+            by_level.push_back(b);
+            for (uint32_t k = 0; k < q.blk_nsrc[b]; ++k) {
+                const auto &s = q.srcs[q.blk_src0[b] + k];
+                if (s.label_kind == 0) lv[L].has_term = 1u;
+                else if (s.label < 64u) lv[L].boxes |= 1ull << s.label;
+                else lv[L].any_box = 1u;
+                if (s.rblk >= 0 && !s.same_level) lv[L].reads |= 1ull << q.blk_level[(size_t)s.rblk];
+            }
+        }
+        lv[L].nblk = (uint32_t)by_level.size() - lv[L].blk0;
+    }
+    for (const auto &s : q.srcs)
+        src.push_back(SmallSrc{s.label_kind, s.label, (s.ident ? 1u : 0u) | (s.same_level ? 2u : 0u), s.rblk});
+    std::vector<uint32_t> m;
+    auto put = [&](const void *p, size_t bytes) {
+        const uint32_t at = (uint32_t)m.size();
+        m.resize(at + bytes / 4);
+        if (bytes) memcpy(m.data() + at, p, bytes);
+        return at;
+    };
     SmallDesc d;
     memset(&d, 0, sizeof(d));
-    d.n = n;
-    d.W = W;
-    d.B = B;
+    put(lv.data(), lv.size() * sizeof(SmallLevel));
+    d.o_srcs = put(src.data(), src.size() * sizeof(SmallSrc));  // (16-byte records up to here)
+    d.o_blk = put(by_level.data(), by_level.size() * 4);
+    d.o_src0 = put(q.blk_src0.data(), q.blk_src0.size() * 4);
+    d.o_nsrc = put(q.blk_nsrc.data(), q.blk_nsrc.size() * 4);
+    d.o_f0 = put(q.box_f0.data(), q.box_f0.size() * 4);
+    d.o_nf = put(q.box_nf.data(), q.box_nf.size() * 4);
+    std::vector<uint32_t> null_box(q.B);
+    for (uint32_t b = 0; b < q.B; ++b) null_box[b] = q.rsm.final_[q.rsm.box_start[b]] ? 1u : 0u;
+    d.o_null = put(null_box.data(), null_box.size() * 4);
+    d.o_fb = put(q.fblocks.data(), q.fblocks.size() * 4);
+    while (m.size() % 4) m.push_back(0u);
+    d.n = q.n;
+    d.W = q.W;
+    d.B = q.B;
     d.nblk = nblk;
-    d.n_levels = n_levels;
-    d.max_iter = max_iter;
-    d.max_passes = max_passes;
-    d.cyclic_mask = cyclic_mask;
-    d.blk_level = dev_arrays + off_level;
-    d.blk_src0 = dev_arrays + off_src0;
-    d.blk_nsrc = dev_arrays + off_nsrc;
-    d.srcs = dev_srcs;
-    d.box_f0 = dev_arrays + off_f0;
-    d.box_nf = dev_arrays + off_nf;
-    d.fblocks = dev_arrays + off_fb;
-    d.box_nullable = dev_arrays + off_null;
-    d.csr_off = csr_off;
-    d.csr_col = csr_col;
-    d.blk_out = blk_out;
-    d.m2_out = m2_out;
-    d.ctl = ctl;
+    d.n_levels = q.n_levels;
+    d.magic = (uint32_t)((0x100000000ull + q.n - 1) / q.n);  // (n = 1: wraps to 0)
+    d.meta_words = (uint32_t)m.size();
+    d.cyclic_mask = q.cyclic_mask;
     memcpy(desc_out, &d, sizeof(d));
+    return m;
 }
 
-void fill_small_src(void *dst, uint32_t kind, uint32_t label, uint32_t ident, uint32_t same_level, int32_t rblk) {
-    SmallSrc s{kind, label, ident, same_level, rblk, 0u};
-    memcpy(dst, &s, sizeof(s));
+void finish_small_desc(void *desc, const uint32_t *meta, uint32_t max_iter, uint32_t max_passes,
+                       const uint32_t *csr_off, const uint32_t *csr_col, uint64_t *blk_out, uint64_t *m2_out,
+                       QCtl *ctl) {
+    SmallDesc *d = static_cast<SmallDesc *>(desc);
+    d->meta = meta;
+    d->max_iter = max_iter;
+    d->max_passes = max_passes;
+    d->csr_off = csr_off;
+    d->csr_col = csr_col;
+    d->blk_out = blk_out;
+    d->m2_out = m2_out;
+    d->ctl = ctl;
 }
 
 }  // namespace cfpq

@@ -185,7 +185,7 @@ struct TcJob {
     const uint64_t *A;
     const uint32_t *a_it;      // if set: A row x is used only when a_it[x] == iter
     const uint64_t *B;
-    const uint32_t *b_stamp;   // stamps of B rows (null: all rows)
+    const uint32_t *b_stamp;   // stamps of B rows (0: never written; null: all rows)
     QCtl *ctl;                 // null: standalone product (iter = 0, thr = 0, g = 0)
     uint32_t n, W;
     uint32_t ident;            // also OR the A rows themselves into out (product edge u == t)
@@ -216,17 +216,26 @@ struct TcJob {
     uint32_t kstride;
     uint32_t fp4;
     uint32_t tile_ratio;        // new_tiles_pay's ratio (channel-1 jobs)
+    // Row compaction of a compacted job: M holds only the rows x that can
+    // gain a bit -- A's row x has an edge to a listed row of B (kmask: the
+    // listed rows as W words), and the output row lacks a column that some
+    // listed row has (ucols: their OR, W words).  a8 row m is A's row xs[m],
+    // m < *mrows.  a_live (null: every row) is zero for rows of A without
+    // any edge.  ucols and mrows are zeroed before every pass.
+    const uint32_t *a_live;
+    uint64_t *kmask;
+    uint64_t *ucols;
+    uint32_t *xs;
+    unsigned long long *mrows;
     // Channel-1 job (covers_new): the iteration's new edges A2 (A = A2 rows,
-    // a_it = their iteration marks) times whole rows of B, compacted on both
-    // sides: M to the rows x with a new edge (xs, count *mcount), K to the
-    // columns y of some new edge (newcols, a bitmap of W words, then ys).
-    // *ecount = the number of new edges.  mcount, ecount and newcols are
-    // zeroed before every pass.  The job runs only when new_tiles_pay says
-    // the tiles beat the row gather on those counts; the gather then skips
-    // the channel's row ORs.
+    // a_it = their iteration marks) times whole rows of B; K = the columns y
+    // of some new edge (newcols, W words) whose row of B was ever written.
+    // *mcount = rows with a new edge, *ecount = the number of new edges;
+    // newcols and the counts are zeroed before every pass.  The job runs only
+    // when new_tiles_pay says the tiles beat the row gather on those counts;
+    // the gather then skips the channel's row ORs.
     uint32_t covers_new;
     uint64_t *newcols;
-    uint32_t *xs;
     unsigned long long *mcount;
     unsigned long long *ecount;
 };

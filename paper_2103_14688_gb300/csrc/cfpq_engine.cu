@@ -615,8 +615,19 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
         kind_set = true;
     }
     uint32_t n_maps = 0;
-    size_t n_newcols = 0;  // words of the channel-1 jobs' column bitmaps and counts
-    std::vector<size_t> newcols_of;
+    // Per-pass scratch of the tile jobs, zeroed before every pass: newcols,
+    // kmask and ucols (W words each), then mcount, ecount and mrows.
+    size_t n_scratch = 0;
+    auto scratch_words = [](uint32_t W) { return 3u * (size_t)W + 8u; };
+    auto set_scratch = [](TcJob &j, size_t off) {  // (offsets, made pointers below)
+        const size_t W = j.W;
+        j.newcols = reinterpret_cast<uint64_t *>(off);
+        j.kmask = reinterpret_cast<uint64_t *>(off + W);
+        j.ucols = reinterpret_cast<uint64_t *>(off + 2 * W);
+        j.mcount = reinterpret_cast<unsigned long long *>(off + 3 * W);
+        j.ecount = reinterpret_cast<unsigned long long *>(off + 3 * W + 1);
+        j.mrows = reinterpret_cast<unsigned long long *>(off + 3 * W + 2);
+    };
     uint32_t live_bound[kClasses] = {0};
     for (uint32_t qi = 0; qi < nq; ++qi) {
         QueryDev &q = *qs[qi];
@@ -658,16 +669,15 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
             d.box_switch = sd.box_switch;
             d.label_box = sd.label_kind == 1 ? sd.label : 0u;
             if (sd.tc_slot_new >= 0) {
-                // the channel-1 job's column bitmap and counts: W + 8 words of
-                // the executor's newcols buffer (offsets, made pointers below)
+                // the channel-1 job's counts, in the executor's scratch buffer
+                // (offsets, made pointers below)
                 d.tile_new = 1u;
                 d.tc_kcap = q.kcap;
                 d.tc_ratio = q.tile_ratio;
                 d.tc_kcount = q.tc_kcount((uint32_t)sd.tc_slot_new);
-                d.tc_mcount = reinterpret_cast<const unsigned long long *>((size_t)(n_newcols + q.W));
-                d.tc_ecount = reinterpret_cast<const unsigned long long *>((size_t)(n_newcols + q.W + 1));
-                newcols_of.push_back(n_newcols);
-                n_newcols += q.W + 8u;
+                d.tc_mcount = reinterpret_cast<const unsigned long long *>(n_scratch + 3u * (size_t)q.W);
+                d.tc_ecount = reinterpret_cast<const unsigned long long *>(n_scratch + 3u * (size_t)q.W + 1u);
+                n_scratch += scratch_words(q.W);
             }
             hs.push_back(d);
         }
@@ -764,6 +774,7 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
                         j.box_new_it = nullptr;
                     } else {
                         j.A = q.m2_ptr(sd.label);
+                        j.a_live = q.a2it_mem.as<uint32_t>() + (size_t)sd.label * q.n;
                         j.box_new_it = d.box_new_it;
                     }
                     j.a_it = nullptr;
@@ -785,7 +796,10 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
                     j.kstride = q.tc_kstride();
                     j.fp4 = q.tile_fp4 ? 1u : 0u;
                     j.tile_ratio = q.tile_ratio;
+                    j.xs = q.tc_xs((uint32_t)sd.tc_slot);
                     j.ys = q.tc_ys((uint32_t)sd.tc_slot);
+                    set_scratch(j, n_scratch);
+                    n_scratch += scratch_words(q.W);
                     j.kcount = q.tc_kcount((uint32_t)sd.tc_slot);
                     j.a8 = q.tc_a8((uint32_t)sd.tc_slot);
                     j.b8 = q.tc_b8((uint32_t)sd.tc_slot);
@@ -796,15 +810,11 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
                     max_tc_w = std::max(max_tc_w, q.W);
                     if (sd.tc_slot_new >= 0) {
                         // channel 1: A2 rows (new in the iteration) x whole rows of B
-                        const size_t off = reinterpret_cast<size_t>(d.tc_mcount) - q.W;
+                        set_scratch(j, reinterpret_cast<size_t>(d.tc_mcount) - 3u * (size_t)q.W);
                         j.chan = 1u;
                         j.A = q.a2_ptr(sd.label);
                         j.a_it = q.a2it_mem.as<uint32_t>() + (size_t)sd.label * q.n;
-                        j.b_stamp = nullptr;
                         j.covers_new = 1u;
-                        j.newcols = reinterpret_cast<uint64_t *>(off);
-                        j.mcount = reinterpret_cast<unsigned long long *>(off + q.W);
-                        j.ecount = reinterpret_cast<unsigned long long *>(off + q.W + 1);
                         j.xs = q.tc_xs((uint32_t)sd.tc_slot_new);
                         j.ys = q.tc_ys((uint32_t)sd.tc_slot_new);
                         j.kcount = q.tc_kcount((uint32_t)sd.tc_slot_new);
@@ -863,20 +873,22 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
         return CFPQ_OK;
     };
     int rc;
-    newcols_words = n_newcols;
-    if (n_newcols) {
-        if (!newcols.ensure(A, n_newcols * 8, err)) return CFPQ_ERR_OUT_OF_MEMORY;
-        uint64_t *nb = newcols.as<uint64_t>();
+    scratch_words_total = n_scratch;
+    if (n_scratch) {
+        if (!scratch.ensure(A, n_scratch * 8, err)) return CFPQ_ERR_OUT_OF_MEMORY;
+        uint64_t *nb = scratch.as<uint64_t>();
         auto fix = [nb](auto *&p) {
             using T = std::remove_pointer_t<std::remove_reference_t<decltype(p)>>;
             p = reinterpret_cast<T *>(nb + reinterpret_cast<size_t>(p));
         };
-        for (auto &j : hj)
-            if (j.covers_new) {
-                fix(j.newcols);
-                fix(j.mcount);
-                fix(j.ecount);
-            }
+        for (auto &j : hj) {
+            fix(j.newcols);
+            fix(j.kmask);
+            fix(j.ucols);
+            fix(j.mcount);
+            fix(j.ecount);
+            fix(j.mrows);
+        }
         for (auto &d : hs)
             if (d.tile_new) {
                 fix(d.tc_mcount);
@@ -978,7 +990,7 @@ int Executor::enqueue_pass(cudaStream_t st, cudaGraphConditionalHandle h, int us
     // gather whose source's new edges the tiles take needs the job's list.
     if (ev) ENG_CK(cudaEventRecord(ev[0], st));
     if (n_tcjobs) {
-        if (newcols_words) ENG_CK(cudaMemsetAsync(newcols.p, 0, newcols_words * 8, st));
+        if (scratch_words_total) ENG_CK(cudaMemsetAsync(scratch.p, 0, scratch_words_total * 8, st));
         ENG_CK(launch_tc_compact(tcjobs.as<TcJob>(), T, max_tc_w, tc_err.as<int>(), st));
     }
     if (ev) ENG_CK(cudaEventRecord(ev[1], st));

@@ -331,8 +331,8 @@ struct Executor {
     std::vector<QueryDev *> qs;
     DBuf ctl_ptrs, mirror, items[kClasses], xitems[kClasses], srcs, fds, running;
     DBuf tcjobs, tcmaps, tables, tc_err, done_counter;
-    DBuf newcols;              // new-edge column bitmaps of the jobs covering new edges (zeroed every pass)
-    size_t newcols_words = 0;
+    DBuf scratch;              // the tile jobs' column bitmaps and counts (zeroed every pass)
+    size_t scratch_words_total = 0;
     ExecTables T;
     uint32_t n_items[kClasses] = {0}, n_xitems[kClasses] = {0};
     uint32_t max_live[kClasses] = {0};  // bound on live items of a pass: sum over queries of the largest level

@@ -539,7 +539,6 @@ __global__ void __launch_bounds__(tc::kThreads, 2)
 // Dirty-row compaction of the product jobs (channels 2 and 4).
 // ---------------------------------------------------------------------------
 constexpr uint32_t kRowChunk = 2048;  // k_tc_rows: rows per unit
-constexpr uint32_t kColRows = 8;      // k_tc_cols: rows per unit (one per warp)
 constexpr uint32_t kColMaxW = 1024;   // largest row in words (n <= 65536)
 constexpr uint32_t kCasLimit = 1u << 20;
 
@@ -561,14 +560,13 @@ __device__ __forceinline__ uint32_t reserve_rows(unsigned long long *kc, uint32_
 // Units (job, chunk) of the pass's active jobs (the control kernel's list)
 // are numbered in list order; the CTA takes those congruent to its index.
 // `body(J, c)` runs for each.
-template <typename F>
-__device__ __forceinline__ void for_job_chunks(const TcJob *jobs, const ExecTables &T, uint32_t rows_per_chunk,
-                                               F body) {
+template <typename R, typename F>
+__device__ __forceinline__ void for_job_chunks(const TcJob *jobs, const ExecTables &T, R rows_per_chunk, F body) {
     uint32_t u0 = 0;
     const uint32_t na = *T.aj_n;
     for (uint32_t a = 0; a < na; ++a) {
         const TcJob &J = jobs[T.aj[a]];
-        const uint32_t chunks = (J.n + rows_per_chunk - 1) / rows_per_chunk;
+        const uint32_t per = rows_per_chunk(J), chunks = (J.n + per - 1) / per;
         const uint32_t first = (blockIdx.x + gridDim.x - (u0 % gridDim.x)) % gridDim.x;
         u0 += chunks;
         if (first >= chunks || !J.ys) continue;
@@ -578,7 +576,7 @@ __device__ __forceinline__ void for_job_chunks(const TcJob *jobs, const ExecTabl
 
 // Channel-1 jobs (TcJob::covers_new), before their row lists: for the A2
 // rows x new in the iteration, newcols (zeroed before the pass) |= row x,
-// x is appended to xs, and *ecount += the row's edges.  Bound by latency: a
+// *mcount += 1 and *ecount += the row's edges.  Bound by latency: a
 // pass has few new rows and a unit's rows are read one after another, so a
 // unit is small (64 rows: 47 CTAs at n = 3001, where units of 512 rows left 6
 // CTAs with 512 dependent loads each), its new rows are listed first, and the
@@ -589,9 +587,9 @@ __device__ __forceinline__ void for_job_chunks(const TcJob *jobs, const ExecTabl
 constexpr uint32_t kNewColRows = 64;
 __global__ void __launch_bounds__(256) k_tc_newcols(const TcJob *__restrict__ jobs, ExecTables T) {
     __shared__ unsigned long long s_edges;
-    __shared__ uint32_t s_rows[kNewColRows], s_cnt[2], s_base;
+    __shared__ uint32_t s_rows[kNewColRows], s_cnt[2];
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-    for_job_chunks(jobs, T, kNewColRows, [&](const TcJob &J, uint32_t c) {
+    for_job_chunks(jobs, T, [](const TcJob &) { return kNewColRows; }, [&](const TcJob &J, uint32_t c) {
         uint32_t thr, iter, g;
         if (!J.covers_new || !tc_job_active(J, &thr, &iter, &g)) return;
         const uint32_t W = J.W;
@@ -612,9 +610,8 @@ __global__ void __launch_bounds__(256) k_tc_newcols(const TcJob *__restrict__ jo
             return;
         }
         if (mine) s_rows[(warp ? s_cnt[0] : 0u) + (uint32_t)__popc(bal & ((1u << lane) - 1u))] = x;
-        if (tid == 0) s_base = (uint32_t)atomicAdd(J.mcount, (unsigned long long)cnt);
+        if (tid == 0) atomicAdd(J.mcount, (unsigned long long)cnt);
         __syncthreads();
-        if (tid < cnt) J.xs[s_base + tid] = s_rows[tid];
         const uint32_t groups = W < 256u ? 256u / W : 1u, grp = W < 256u ? tid / W : 0u;
         uint32_t edges = 0u;
         for (uint32_t w = W < 256u ? tid - grp * W : tid; w < W && grp < groups; w += 256u) {
@@ -647,7 +644,9 @@ __global__ void __launch_bounds__(256) k_tc_newcols(const TcJob *__restrict__ jo
 }
 
 // List the rows y of B with stamp >= thr; for a channel-1 job the columns
-// of its newcols (order irrelevant: the product sums over them).
+// of its newcols whose row of B was ever written (stamp != 0: on Dyck-4 two
+// thirds of the vertices start no path, so their rows are empty).  The order
+// is irrelevant (the product sums over them).  kmask = the listed rows.
 __global__ void __launch_bounds__(256) k_tc_rows(const TcJob *__restrict__ jobs, ExecTables T, int *err_flag) {
     // a unit's listed rows are counted over the CTA first, so that the unit
     // reserves its part of the list with one atomic (one per warp step kept
@@ -656,17 +655,21 @@ __global__ void __launch_bounds__(256) k_tc_rows(const TcJob *__restrict__ jobs,
     static_assert(kRowChunk % 256u == 0u && kPer <= 32u, "k_tc_rows: 256 threads, a bit per row");
     __shared__ uint32_t s_warp[8], s_base;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for_job_chunks(jobs, T, kRowChunk, [&](const TcJob &J, uint32_t c) {
+    for_job_chunks(jobs, T, [](const TcJob &) { return kRowChunk; }, [&](const TcJob &J, uint32_t c) {
         uint32_t thr, iter, g;
-        if (!tc_job_active(J, &thr, &iter, &g) || (!J.b_stamp && !J.covers_new)) return;
+        if (!tc_job_active(J, &thr, &iter, &g) || !J.b_stamp) return;
         const uint32_t y_beg = c * kRowChunk, y_end = min(J.n, y_beg + kRowChunk);
         uint32_t mask = 0u;
 #pragma unroll
         for (uint32_t i = 0; i < kPer; ++i) {
             const uint32_t y = y_beg + threadIdx.x + 256u * i;
-            const bool dirty = y < y_end && (J.covers_new ? ((J.newcols[y >> 6] >> (y & 63u)) & 1ull) != 0ull
+            const bool dirty = y < y_end && (J.covers_new ? ((J.newcols[y >> 6] >> (y & 63u)) & 1ull) != 0ull &&
+                                                                J.b_stamp[y] != 0u
                                                           : J.b_stamp[y] >= thr);
             if (dirty) mask |= 1u << i;
+            const unsigned bal = __ballot_sync(0xffffffffu, dirty);
+            // (y_beg and 256 i are multiples of 32: the warp's rows are one 32-bit word of kmask)
+            if (lane == 0 && y < y_end) reinterpret_cast<uint32_t *>(J.kmask)[y >> 5] = bal;
         }
         // exclusive prefix of the threads' counts over the CTA
         const uint32_t cnt = (uint32_t)__popc(mask);
@@ -697,69 +700,118 @@ __global__ void __launch_bounds__(256) k_tc_rows(const TcJob *__restrict__ jobs,
     });
 }
 
-// a8[x][k] = A[x][ys[k]] as a 0/1 FP8 byte for k < D, 0 up to the next
-// multiple of 128; one warp per row x, the row staged in shared memory, each
-// lane writing 4 consecutive bytes of a coalesced 128-byte step.  FP4 jobs
-// get E2M1 nibbles instead (see below).
+// Rows of A a compacted job multiplies, and their operand: a8[m][k] =
+// A[xs[m]][ys[k]] as a 0/1 FP8 byte (FP4 jobs: E2M1 nibble) for k < D, 0 up to
+// the next multiple of 128 (256).  A row takes part when it has an edge to a
+// listed row of B and its output row lacks a column of their OR.  (Runs after
+// k_tc_b8, which gathers that OR.)  On Dyck-4 the answer is close to a complete
+// bipartite graph between a third of the vertices and two thirds: without
+// the filter two of three multiplied rows are empty, and the late iterations
+// multiply rows that cannot change.  n = 65536: rows multiplied per pass 65536 -> about
+// 20000 while the answer grows and a few hundred after.
+// Unit of a warp: up to 8 rows (n / 4096, so that small graphs still spread over
+// the chip) -- their marks in one load, the tests row by row (kmask words that
+// are zero skip A's), one atomic for their places, then the expansion, the row
+// staged in shared memory, each lane writing 4 consecutive bytes of a coalesced
+// 128-byte step.
 __global__ void __launch_bounds__(256) k_tc_a8(const TcJob *__restrict__ jobs, ExecTables T, uint32_t max_w) {
     extern __shared__ uint64_t s_rowbuf[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint64_t *row = s_rowbuf + (size_t)warp * max_w;
-    for_job_chunks(jobs, T, kColRows, [&](const TcJob &J, uint32_t c) {
+    auto rows_of = [](const TcJob &J) { return min(8u, max(1u, J.n / 4096u)); };
+    for_job_chunks(jobs, T, [&](const TcJob &J) { return 8u * rows_of(J); }, [&](const TcJob &J, uint32_t c) {
         uint32_t thr, iter, g;
         if (!tc_job_active(J, &thr, &iter, &g)) return;
         const KDim K = job_kdim(J, g);
         if (!K.compact || K.kdim == 0u) return;
-        // row m of a8: A's row m, or for a channel-1 job A2's row xs[m]
-        const uint32_t m = c * kColRows + (uint32_t)warp;
-        if (m >= (J.covers_new ? (uint32_t)*J.mcount : J.n)) return;
-        const uint32_t x = J.covers_new ? J.xs[m] : m;
-        const uint32_t W = J.W, D = K.kdim, dpad = (D + 127u) & ~127u;
-        const uint4 *src = reinterpret_cast<const uint4 *>(J.A + (size_t)x * W);
-        bool nz = false;
-        for (uint32_t v = (uint32_t)lane; v < W / 2u; v += 32u) {
-            const uint4 t4 = src[v];
-            reinterpret_cast<uint4 *>(row)[v] = t4;
-            nz |= (t4.x | t4.y | t4.z | t4.w) != 0u;
-        }
-        nz = __any_sync(0xffffffffu, nz);
-        __syncwarp();
-        uint32_t *dst = reinterpret_cast<uint32_t *>(J.a8 + (size_t)m * J.kstride);
-        if (J.fp4) {
-            // E2M1 nibbles: 8 elements (4 bytes) per lane and 256-element step,
-            // zero up to the next multiple of 256 (a whole K stage) within kcap
-            const uint32_t kend = min((D + 255u) & ~255u, J.kcap);
-            for (uint32_t k0 = 0; k0 < kend; k0 += 256u) {
-                const uint32_t kb = k0 + 8u * (uint32_t)lane;
-                if (kb >= kend) continue;
-                uint32_t word = 0u;
-                if (nz && kb < D) {
-                    const uint4 y0 = *reinterpret_cast<const uint4 *>(J.ys + kb);
-                    const uint4 y1 = *reinterpret_cast<const uint4 *>(J.ys + kb + 4u);
-                    const uint32_t yv[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        if (kb + (uint32_t)i < D && ((row[yv[i] >> 6] >> (yv[i] & 63u)) & 1ull))
-                            word |= 0x2u << (4 * i);
+        const uint32_t R = rows_of(J), x0 = (c * 8u + (uint32_t)warp) * R, W = J.W, nvec = W / 2u;
+        bool cand = false;
+        if ((uint32_t)lane < R && x0 + (uint32_t)lane < J.n)
+            cand = J.a_it ? J.a_it[x0 + lane] == iter : (!J.a_live || J.a_live[x0 + lane] != 0u);
+        const unsigned cands = __ballot_sync(0xffffffffu, cand);
+        unsigned use = 0u;
+        const uint4 *km = reinterpret_cast<const uint4 *>(J.kmask), *uc = reinterpret_cast<const uint4 *>(J.ucols);
+        for (unsigned m = cands; m; m &= m - 1u) {
+            const uint32_t x = x0 + (uint32_t)(__ffs(m) - 1);
+            const uint4 *ar = reinterpret_cast<const uint4 *>(J.A + (size_t)x * W);
+            const uint4 *orow = reinterpret_cast<const uint4 *>(J.out + (size_t)x * W);
+            bool hit = false;
+            for (uint32_t v0 = 0; v0 < nvec && !hit; v0 += 32u) {
+                const uint32_t v = v0 + (uint32_t)lane;
+                bool h = false;
+                if (v < nvec) {
+                    const uint4 k4 = km[v];
+                    if (k4.x | k4.y | k4.z | k4.w) {
+                        const uint4 t4 = ar[v];
+                        h = ((t4.x & k4.x) | (t4.y & k4.y) | (t4.z & k4.z) | (t4.w & k4.w)) != 0u;
+                    }
                 }
-                dst[kb >> 3] = word;
+                hit = __any_sync(0xffffffffu, h);
             }
+            if (!hit) continue;
+            bool lacks = false;
+            for (uint32_t v0 = 0; v0 < nvec && !lacks; v0 += 32u) {
+                const uint32_t v = v0 + (uint32_t)lane;
+                bool h = false;
+                if (v < nvec) {
+                    const uint4 u4 = uc[v];
+                    if (u4.x | u4.y | u4.z | u4.w) {
+                        const uint4 o4 = orow[v];
+                        h = ((u4.x & ~o4.x) | (u4.y & ~o4.y) | (u4.z & ~o4.z) | (u4.w & ~o4.w)) != 0u;
+                    }
+                }
+                lacks = __any_sync(0xffffffffu, h);
+            }
+            if (lacks) use |= m & (0u - m);
+        }
+        if (!use) return;
+        const uint32_t D = K.kdim, dpad = (D + 127u) & ~127u, kend = min((D + 255u) & ~255u, J.kcap);
+        const uint32_t rows = (uint32_t)__popc(use);
+        uint32_t pos = 0u;
+        if (lane == 0) {
+            pos = (uint32_t)atomicAdd(J.mrows, (unsigned long long)rows);
+            if (J.ctl) atomicAdd(&J.ctl->tile_operand_bytes, (unsigned long long)rows * (J.fp4 ? kend / 2u : dpad));
+        }
+        pos = __shfl_sync(0xffffffffu, pos, 0);
+        for (; use; use &= use - 1u, ++pos) {
+            const uint32_t x = x0 + (uint32_t)(__ffs(use) - 1);
+            if (lane == 0) J.xs[pos] = x;
+            const uint4 *src = reinterpret_cast<const uint4 *>(J.A + (size_t)x * W);
+            for (uint32_t v = (uint32_t)lane; v < nvec; v += 32u) reinterpret_cast<uint4 *>(row)[v] = src[v];
             __syncwarp();
-            return;
-        }
-        for (uint32_t k0 = 0; k0 < dpad; k0 += 128u) {
-            const uint32_t kb = k0 + 4u * (uint32_t)lane;
-            uint32_t word = 0u;
-            if (nz && kb < D) {
-                const uint4 y4 = *reinterpret_cast<const uint4 *>(J.ys + kb);
-                const uint32_t yv[4] = {y4.x, y4.y, y4.z, y4.w};
+            uint32_t *dst = reinterpret_cast<uint32_t *>(J.a8 + (size_t)pos * J.kstride);
+            if (J.fp4) {
+                // E2M1 nibbles: 8 elements (4 bytes) per lane and 256-element step,
+                // zero up to the next multiple of 256 (a whole K stage) within kcap
+                for (uint32_t kb = 8u * (uint32_t)lane; kb < kend; kb += 256u) {
+                    uint32_t word = 0u;
+                    if (kb < D) {
+                        const uint4 y0 = *reinterpret_cast<const uint4 *>(J.ys + kb);
+                        const uint4 y1 = *reinterpret_cast<const uint4 *>(J.ys + kb + 4u);
+                        const uint32_t yv[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (kb + (uint32_t)i < D && ((row[yv[i] >> 6] >> (yv[i] & 63u)) & 1ull)) word |= 0x38u << (8 * i);
+                        for (int i = 0; i < 8; ++i)
+                            if (kb + (uint32_t)i < D && ((row[yv[i] >> 6] >> (yv[i] & 63u)) & 1ull))
+                                word |= 0x2u << (4 * i);
+                    }
+                    dst[kb >> 3] = word;
+                }
+            } else {
+                for (uint32_t kb = 4u * (uint32_t)lane; kb < dpad; kb += 128u) {
+                    uint32_t word = 0u;
+                    if (kb < D) {
+                        const uint4 y4 = *reinterpret_cast<const uint4 *>(J.ys + kb);
+                        const uint32_t yv[4] = {y4.x, y4.y, y4.z, y4.w};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            if (kb + (uint32_t)i < D && ((row[yv[i] >> 6] >> (yv[i] & 63u)) & 1ull))
+                                word |= 0x38u << (8 * i);
+                    }
+                    dst[kb >> 2] = word;
+                }
             }
-            dst[kb >> 2] = word;
+            __syncwarp();  // the next row reuses the staging buffer
         }
-        __syncwarp();  // the next row reuses the staging buffer
     });
 }
 
@@ -794,13 +846,8 @@ __global__ void __launch_bounds__(256) k_tc_b8(const TcJob *__restrict__ jobs, E
         const uint32_t units = kchunks * zchunks;
         const uint32_t first = (gw + nw - (u0 % nw)) % nw;
         u0 += units;
-        if (first == 0u && lane == 0 && units && J.ctl) {
-            // operand bytes of the job in this pass: B's (this kernel) and A's (k_tc_a8)
-            const uint32_t ka = J.fp4 ? min((D + 255u) & ~255u, J.kcap) / 2u : (D + 127u) & ~127u;
-            const unsigned long long rows_a = J.covers_new ? *J.mcount : (unsigned long long)J.n;
-            atomicAdd(&J.ctl->tile_operand_bytes,
-                      (unsigned long long)(zend - zbeg) * (J.fp4 ? kpad / 2u : kpad) + rows_a * ka);
-        }
+        if (first == 0u && lane == 0 && units && J.ctl)  // operand bytes of B (A's: k_tc_a8)
+            atomicAdd(&J.ctl->tile_operand_bytes, (unsigned long long)(zend - zbeg) * (J.fp4 ? kpad / 2u : kpad));
         for (uint32_t u = first; u < units; u += nw) {
             const uint32_t k0 = (u / zchunks) * 64u, z0 = zbeg + (u % zchunks) * 256u;
             const uint32_t halves = min(2u, (zend - z0) / 128u);  // 128-column halves in the row
@@ -814,6 +861,20 @@ __global__ void __launch_bounds__(256) k_tc_b8(const TcJob *__restrict__ jobs, E
 #pragma unroll
                 for (int c = 0; c < 2; ++c)
                     row[h][c] = (src && (uint32_t)c < halves) ? src[c] : make_uint4(0u, 0u, 0u, 0u);
+            }
+            // the rows' OR: eight 32-bit words of the unit's columns, one a lane
+            {
+                uint32_t u = 0u;
+#pragma unroll
+                for (int w = 0; w < 8; ++w) {
+                    const uint4 &r0 = row[0][w >> 2], &r1 = row[1][w >> 2];
+                    const uint32_t v = (w & 3) == 0 ? r0.x | r1.x : (w & 3) == 1 ? r0.y | r1.y : (w & 3) == 2 ? r0.z | r1.z
+                                                                                                                : r0.w | r1.w;
+                    const uint32_t o = __reduce_or_sync(0xffffffffu, v);
+                    if (lane == w) u = o;
+                }
+                uint32_t *uw = reinterpret_cast<uint32_t *>(J.ucols) + (z0 >> 5) + (uint32_t)lane;
+                if (u && (u & ~__ldcg(uw))) atomicOr(uw, u);  // (u is zero in lanes 8 .. 31 and past the row)
             }
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
@@ -894,7 +955,7 @@ __device__ __forceinline__ void tma_load(void *dst, const void *map, int32_t c0,
 struct Tile {
     const TcJob *J;
     uint32_t m0, n0, ks, g;
-    uint32_t mlim;  // rows of a8 (a channel-1 job's row count; else n)
+    uint32_t mlim;  // rows of a8
 };
 struct JobCache {
     const TcJob *J = nullptr;
@@ -973,7 +1034,7 @@ __device__ __forceinline__ bool next_tile(const TcJob *jobs, const ExecTables &T
         jc.ok = ok;
         jc.ks = (K.kdim + KSTAGE - 1u) / KSTAGE;
         jc.g = g;
-        jc.mlim = ok && J.covers_new ? (uint32_t)*J.mcount : J.n;
+        jc.mlim = ok ? (uint32_t)*J.mrows : 0u;
         jc.ntn = COLS == 256u ? J.tiles_n : (J.n + COLS - 1u) / COLS;
         job_window(J, &jc.c0, &jc.c1);
         li -= gridDim.x;  // re-enter through the cache
@@ -1157,7 +1218,7 @@ __global__ void __launch_bounds__(tc2::kThreads, 1)
             __syncwarp();
             if (lane == 0) arrive(&tempty[0]);  // the accumulators may be overwritten
             const uint32_t r = quarter * 32u + (uint32_t)lane, mr = tl.m0 + 128u * hh + r;
-            const uint32_t x = mr >= tl.mlim ? J.n : (J.covers_new ? J.xs[mr] : mr);
+            const uint32_t x = mr >= tl.mlim ? J.n : J.xs[mr];
             bool ch = false;
             if (x < J.n) {
                 // read the three output words first and OR only those that
@@ -1224,9 +1285,9 @@ __global__ void __launch_bounds__(tc2::kThreads, 1)
             if (lane == 0) arrive(&tempty[acc]);  // the accumulators may be overwritten
 #pragma unroll
             for (int hh = 0; hh < kHalves; ++hh) {
-                // output row: tile row m0 + 128 hh + r, through xs for a channel-1 job
+                // output row: tile row m0 + 128 hh + r, through xs
                 const uint32_t r = quarter * 32u + (uint32_t)lane, mr = tl.m0 + 128u * (uint32_t)hh + r;
-                const uint32_t x = mr >= tl.mlim ? J.n : (J.covers_new ? J.xs[mr] : mr);
+                const uint32_t x = mr >= tl.mlim ? J.n : J.xs[mr];
                 bool ch = false;
                 if (x < J.n) {
                     const uint32_t w0 = (tl.n0 >> 6) + half * 2u;
@@ -1347,10 +1408,10 @@ cudaError_t launch_tc_compact(const TcJob *jobs, const ExecTables &T, uint32_t m
     k_tc_rows<<<(unsigned)sms * 4u, 256, 0, st>>>(jobs, T, err_flag);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_tc_a8<<<(unsigned)sms * 4u, 256, (size_t)max_w * 8u * 8u, st>>>(jobs, T, max_w);
+    k_tc_b8<<<(unsigned)sms * 8u, 256, 0, st>>>(jobs, T);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_tc_b8<<<(unsigned)sms * 8u, 256, 0, st>>>(jobs, T);
+    k_tc_a8<<<(unsigned)sms * 4u, 256, (size_t)max_w * 8u * 8u, st>>>(jobs, T, max_w);
     return cudaGetLastError();
 }
 

@@ -8,14 +8,14 @@
 // it: once per device and process it runs a probe query through the
 // library's own API -- Dyck-4 on a seeded graph of 8192 vertices with
 // Zipf(2.1) out-degrees (mean about 3), 8 labels -- with the bit-packed
-// closure and with every
-// tile kernel, in the host-driven loop with per-kernel CUDA events, times
-// reads of an L2-sized and an HBM-sized buffer, and keeps
-//   - the rate of each tile kernel (0/1 multiply-adds per second over its
-//     launches) and of the gather (source-row bytes ORed per second; the
-//     probe's 8 MiB closure blocks stay in L2, so for blocks beyond half the
-//     L2 the rate is scaled by the ratio of the device's read bandwidth
-//     from HBM to that from L2, both measured);
+// closure in the host-driven loop with per-kernel CUDA events, times a dense
+// 8192^3 product in every tile kernel and reads of an L2-sized and an
+// HBM-sized buffer, and keeps
+//   - the rate of each tile kernel (0/1 multiply-adds per second) and of the
+//     gather (source-row bytes ORed per second; the probe's 8 MiB closure
+//     blocks stay in L2, so for blocks beyond half the L2 the rate is scaled
+//     by the ratio of the device's read bandwidth from HBM to that from L2,
+//     both measured);
 //   - the fastest tile kernel, AUTO's default (the built-in FP4 one unless
 //     another is 3% faster);
 //   - per kernel and query size, the ratio of the cost model that decides
@@ -26,6 +26,7 @@
 // Every choice leaves the answer unchanged (the products are exact).
 #include <chrono>
 #include <cmath>
+#include <cstring>
 #include <mutex>
 #include <vector>
 
@@ -84,7 +85,6 @@ struct ProbeRsm {
 };
 
 constexpr uint32_t kProbeN = 8192, kProbeMaxDeg = 192, kProbeLabels = 8;
-constexpr double kTileFlopPerKstage = 2.0 * 128 * 256 * 128;
 
 // One probe run (the second of two: the first pays for set-up and module
 // loading); returns a CFPQ status.  profiled: the host-driven loop with
@@ -166,6 +166,88 @@ double read_gbs(Allocator &A, cudaStream_t st, int dev, size_t bytes, uint32_t r
     return best;
 }
 
+// Rate of a tile kernel (TFLOP/s): one dense product of two n x n 0/1
+// matrices, operands already expanded, best of 3 launches after an untimed
+// one; 0 on error.  (Not taken from the probe query: its products keep only
+// the rows that can change and are too small to show a kernel's rate -- they
+// put the FP8 kernel first, at half the E2M1 kernels' rate on a large product.)
+double tile_rate(Allocator &A, cudaStream_t st, uint32_t kind) {
+    constexpr uint32_t n = kProbeN, W = n / 64u;
+    const bool fp4 = tile_kind_fp4(kind);
+    const uint32_t kstride = fp4 ? n / 2u : n;
+    std::string err;
+    struct Head {  // descriptors and counts, one buffer
+        unsigned char maps[2 * 128];
+        TcJob job;
+        unsigned long long kcount, mrows;
+        uint32_t tab[4];
+        int err_flag;
+    };
+    DBuf head, out, xs, a8, b8;
+    if (tc_map_bytes() != 128 || !head.ensure(&A, sizeof(Head), &err) || !out.ensure(&A, (size_t)n * W * 8, &err) ||
+        !xs.ensure(&A, (size_t)n * 4, &err) || !a8.ensure(&A, (size_t)n * kstride, &err) ||
+        !b8.ensure(&A, (size_t)n * kstride, &err))
+        return 0;
+    std::vector<uint32_t> ids(n);
+    for (uint32_t i = 0; i < n; ++i) ids[i] = i;
+    alignas(64) Head h;
+    memset(&h, 0, sizeof(h));
+    Head *d = head.as<Head>();
+    TcJob &j = h.job;
+    j.out = out.as<uint64_t>();
+    j.n = n;
+    j.W = W;
+    j.tiles_m = n / 128u;
+    j.tiles_n = n / 256u;
+    j.kcap = n;
+    j.kstride = kstride;
+    j.fp4 = fp4 ? 1u : 0u;
+    j.xs = j.ys = xs.as<uint32_t>();
+    j.a8 = a8.as<uint8_t>();
+    j.b8 = b8.as<uint8_t>();
+    j.kcount = &d->kcount;
+    j.mrows = &d->mrows;
+    h.kcount = n;  // (pass stamp 0: a job without a query)
+    h.mrows = n;
+    h.tab[0] = j.tiles_m * j.tiles_n;
+    h.tab[3] = 1u;
+    ExecTables T;
+    memset(&T, 0, sizeof(T));
+    T.nq = 1;
+    T.t_total = d->tab;
+    T.t_pre = d->tab + 1;
+    T.t_job_beg = d->tab + 2;
+    T.t_job_end = d->tab + 3;
+    double best = 0;
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    const int one = fp4 ? 0x22 : 0x38;
+    if (prepare_tc_launch() == cudaSuccess && tc_encode_maps(&j, 1, h.maps) == cudaSuccess &&
+        cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess &&
+        cudaMemcpyAsync(head.p, &h, sizeof(h), cudaMemcpyHostToDevice, st) == cudaSuccess &&
+        cudaMemcpyAsync(xs.p, ids.data(), (size_t)n * 4, cudaMemcpyHostToDevice, st) == cudaSuccess &&
+        cudaMemsetAsync(out.p, 0, (size_t)n * W * 8, st) == cudaSuccess &&
+        cudaMemsetAsync(a8.p, one, (size_t)n * kstride, st) == cudaSuccess &&
+        cudaMemsetAsync(b8.p, one, (size_t)n * kstride, st) == cudaSuccess) {
+        for (int r = 0; r < 4; ++r) {
+            cudaEventRecord(e0, st);
+            if (launch_tc_product_tma(&d->job, d->maps, h.tab[0], T, &d->err_flag, st, kind) != cudaSuccess) break;
+            cudaEventRecord(e1, st);
+            float ms = 0;
+            if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) break;
+            if (r > 0 && ms > 0) best = std::max(best, 2.0 * n * (double)n * n / (ms * 1e9));
+        }
+        int flag = 0;
+        if (cudaMemcpyAsync(&flag, &d->err_flag, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+            cudaStreamSynchronize(st) != cudaSuccess || flag != 0)
+            best = 0;
+    }
+    cudaStreamSynchronize(st);
+    if (e0) cudaEventDestroy(e0);
+    if (e1) cudaEventDestroy(e1);
+    cudaGetLastError();
+    return best;
+}
+
 uint32_t ratio_for(double tflops, double gather_gbs) {
     // M * K < e * rate_tile / (16 * rate_gather): TFLOP/s over GB/s is 1e3
     const double r = tflops * 1e3 / (16.0 * gather_gbs);
@@ -208,10 +290,13 @@ Tuning run_probe(const cfpq_options &like, cudaStream_t st) {
     if (!rc && s.ms_gather > 0) t.gather_gbs = (double)s.row_ors * (double)s.row_bytes / (s.ms_gather * 1e6);
     const uint32_t fmts[kTileKinds] = {CFPQ_TILES_FP8, CFPQ_TILES_FP8_128, CFPQ_TILES_FP4, CFPQ_TILES_NVFP4};
     for (uint32_t k = 0; k < kTileKinds && !rc; ++k) {
-        const uint32_t mode = tile_kind_fp4(k) ? CFPQ_CLOSURE_TC_FP4 : CFPQ_CLOSURE_TC_FP8;
-        rc = probe_run(like, st, mode, fmts[k], 0, true, pr, src, lbl, dst, &s);
-        if (!rc && s.ms_tile_products > 0)
-            t.tflops[k] = (double)s.tile_kstages * kTileFlopPerKstage / (s.ms_tile_products * 1e9);
+        Allocator A;
+        A.alloc = like.alloc;
+        A.free = like.free;
+        A.user = like.alloc_user;
+        A.stream = st;
+        t.tflops[k] = tile_rate(A, st, k);
+        if (t.tflops[k] <= 0) rc = CFPQ_ERR_CUDA;
     }
     t.probe_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     t.status = rc;

@@ -108,10 +108,8 @@ int run_executor(cfpq_ctx *ctx, Executor &ex, std::vector<QCtl> *ctls, uint32_t 
     const cudaStream_t st = ctx->stream;
     const uint32_t mi = ctx->opt.max_iterations, mr = ctx->opt.max_rounds, mp = pass_cap(ctx->opt);
     uint32_t n_gather = 0, n_extract = 0;
-    for (int v = 0; v < kClasses; ++v) {
-        n_gather += ex.n_items[v] ? 1 : 0;
-        n_extract += ex.n_xitems[v] ? 1 : 0;
-    }
+    for (uint32_t k : ex.n_items) n_gather += k ? 1 : 0;
+    for (uint32_t k : ex.n_xitems) n_extract += k ? 1 : 0;
     // tile jobs: new-edge columns, row list, A and B operands, the two product kernels
     const uint32_t per_pass = n_gather + n_extract + (ex.n_tcjobs ? 6 : 0) + (n_extract ? 0 : 1);
     if (ctx->opt.loop_mode == CFPQ_LOOP_HOST) {

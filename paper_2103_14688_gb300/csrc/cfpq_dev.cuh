@@ -275,15 +275,20 @@ constexpr uint32_t kAutoTilesMinN = 2048;  // AUTO switches boxes to tile produc
 // level and an exclusive prefix over queries, so that persistent kernels walk
 // only the live items.
 constexpr int kVplClasses = 5;
-// Item classes: row width class (VPL 1, 2, 4, 8, 16) x kernel variant: the
-// general variant (nt = 1) serves blocks with sources over nonterminal
+// Item classes.  Gather: row width class (VPL 1, 2, 4, 8, 16) x kernel variant
+// -- the general variant (nt = 1) serves blocks with sources over nonterminal
 // (bit-row) adjacency or reading pure-terminal blocks; class = 2 * vpl_index + nt.
-constexpr int kClasses = 2 * kVplClasses;
+// Blocks whose sources read no closure row at all (kExpand: see k_expand), rows
+// of at most / of more than kExpandNarrowW words, have classes of their own.
+// Extraction: the row width class.
+constexpr int kExpandNarrow = 2 * kVplClasses, kExpandWide = kExpandNarrow + 1;
+constexpr int kClasses = kExpandWide + 1, kXClasses = kVplClasses;
+constexpr uint32_t kExpandNarrowW = 128;
 struct ExecTables {
     uint32_t nq;
     uint32_t maxL1;                          // max levels over queries + 1
     const uint32_t *g_lvl[kClasses];         // [nq * maxL1] gather items per (q, level)
-    const uint32_t *x_rng[kClasses];         // [nq + 1] extraction items per query
+    const uint32_t *x_rng[kXClasses];         // [nq + 1] extraction items per query
     const uint32_t *t_lvl;                   // [nq * maxL1] TC jobs per (q, level)
     const uint32_t *t_lvl_tiles;             // [nq * maxL1] TC tiles of the jobs at (q, level)
     // written by the control kernel for the next pass
@@ -291,9 +296,9 @@ struct ExecTables {
     uint32_t *g_next;                        // [kClasses] dynamic gather units taken in the pass
     uint32_t *g_pre[kClasses];               // [nq] exclusive prefix of live items
     uint32_t *g_beg[kClasses];               // [nq] first live item
-    uint32_t *x_total;                       // [kClasses]
-    uint32_t *x_pre[kClasses];
-    uint32_t *x_beg[kClasses];
+    uint32_t *x_total;                       // [kXClasses]
+    uint32_t *x_pre[kXClasses];
+    uint32_t *x_beg[kXClasses];
     uint32_t *t_total;                       // [1] live TC tiles
     uint32_t *t_pre;                         // [nq] prefix of live tiles
     uint32_t *t_job_beg;                     // [nq]

@@ -591,17 +591,16 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
     std::vector<SrcDesc> hs;
     std::vector<GItem> hi[kClasses];
     std::vector<FDesc> hf;
-    std::vector<XItem> hx[kClasses];
+    std::vector<XItem> hx[kXClasses];
     std::vector<TcJob> hj;
     // static tables
-    std::vector<uint32_t> g_lvl[kClasses], x_rng[kClasses];
-    for (int v = 0; v < kClasses; ++v) {
-        g_lvl[v].assign((size_t)nq * maxL1, 0);
-        x_rng[v].assign((size_t)nq + 1, 0);
-    }
+    std::vector<uint32_t> g_lvl[kClasses], x_rng[kXClasses];
+    for (auto &t : g_lvl) t.assign((size_t)nq * maxL1, 0);
+    for (auto &t : x_rng) t.assign((size_t)nq + 1, 0);
     std::vector<uint32_t> t_lvl((size_t)nq * maxL1, 0), t_lvl_tiles((size_t)nq * maxL1, 0);
     max_tc_tiles = 0;
     max_tc_w = 0;
+    max_expand_w = 0;
     // one tile kernel per executor: the product kernel is launched for it
     tile_kind = kTileFp8Pair;
     bool kind_set = false;
@@ -696,13 +695,19 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
             uint32_t lvl_tiles = 0;
             for (size_t b = 0; b < q.blocks.size(); ++b) {
                 if (q.blk_level[b] != L || q.blk_nsrc[b] == 0) continue;
-                bool has_nt = false;
+                bool has_nt = false, expand = true;
                 for (uint32_t k = 0; k < q.blk_nsrc[b]; ++k) {
                     const auto &sd = q.srcs[q.blk_src0[b] + k];
                     // the general kernel variant: nonterminal adjacency rows, pure-terminal blocks
                     has_nt |= (sd.label_kind != 0) || sd.pure_rb;
+                    // no closure row read: product edges alone, or CSR rows of a pure-terminal block
+                    expand &= sd.rblk < 0 || sd.pure_rb;
                 }
-                const int cls = 2 * vi + (has_nt ? 1 : 0);
+                // (blocks of terminal edges alone stay on the CSR gather: they
+                // have work in one pass of a run)
+                expand &= has_nt;
+                const int cls = !expand ? 2 * vi + (has_nt ? 1 : 0) : q.W <= kExpandNarrowW ? kExpandNarrow : kExpandWide;
+                if (expand) max_expand_w = std::max(max_expand_w, q.W);
                 // wide rows of nonterminal blocks: the adjacency columns are
                 // split over several items, so that rows with thousands of new
                 // edges (hubs) spread over several CTAs
@@ -729,7 +734,7 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
                 // nonterminal blocks of wide rows: 128-row items (measured on
                 // Dyck-4; the CSR blocks of the RPQ bench prefer 64)
                 const uint32_t rows_item =
-                    (has_nt && q.W >= 256u) ? std::min<uint32_t>(1024u, std::max<uint32_t>(rpi, 128u * item_scale)) : rpi;
+                    (has_nt && !expand && q.W >= 256u) ? std::min<uint32_t>(1024u, std::max<uint32_t>(rpi, 128u * item_scale)) : rpi;
                 // the gather keeps an item's row mask in 16 words of shared memory
                 if (rows_item > 1024u || rows_item % 64u != 0u) {
                     *err = "gather items: rows per item must be a multiple of 64 and at most 1024";
@@ -845,7 +850,7 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
         }
         const uint32_t fbase = (uint32_t)hf.size();
         for (uint32_t fb : q.fblocks) hf.push_back(FDesc{q.blk_ptr(fb), q.stamp_ptr(fb)});
-        for (int v = 0; v < kClasses; ++v) x_rng[v][qi] = (uint32_t)hx[v].size();
+        for (int v = 0; v < kXClasses; ++v) x_rng[v][qi] = (uint32_t)hx[v].size();
         for (uint32_t b = 0; b < q.B; ++b) {
             if (q.box_nf[b] == 0) continue;
             for (uint32_t r0 = 0; r0 < q.n; r0 += rpi) {
@@ -862,11 +867,11 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
                 x.row1 = std::min(q.n, r0 + rpi);
                 x.W = q.W;
                 x.lpr = q.lpr;
-                hx[2 * vi].push_back(x);
+                hx[vi].push_back(x);
             }
         }
     }
-    for (int v = 0; v < kClasses; ++v) x_rng[v][nq] = (uint32_t)hx[v].size();
+    for (int v = 0; v < kXClasses; ++v) x_rng[v][nq] = (uint32_t)hx[v].size();
     auto upload = [&](DBuf &buf, const void *h, size_t bytes) -> int {
         if (!buf.ensure(A, std::max<size_t>(bytes, 64), err)) return CFPQ_ERR_OUT_OF_MEMORY;
         if (bytes) ENG_CK(cudaMemcpyAsync(buf.p, h, bytes, cudaMemcpyHostToDevice, st));
@@ -909,15 +914,17 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
     for (int v = 0; v < kClasses; ++v) {
         max_live[v] = live_bound[v];
         n_items[v] = (uint32_t)hi[v].size();
-        n_xitems[v] = (uint32_t)hx[v].size();
         if ((rc = upload(items[v], hi[v].data(), hi[v].size() * sizeof(GItem)))) return rc;
+    }
+    for (int v = 0; v < kXClasses; ++v) {
+        n_xitems[v] = (uint32_t)hx[v].size();
         if ((rc = upload(xitems[v], hx[v].data(), hx[v].size() * sizeof(XItem)))) return rc;
     }
     // tables: one buffer, static part then the per-pass part
     const size_t nqa = std::max<uint32_t>(nq, 1), lv = nqa * maxL1;
-    const size_t words = kClasses * lv + kClasses * (nqa + 1) + 2 * lv  // static
+    const size_t words = kClasses * lv + kXClasses * (nqa + 1) + 2 * lv  // static
                          + 2 * kClasses + 2 * kClasses * nqa              // gather lists and unit counters
-                         + kClasses + 2 * kClasses * nqa                  // extraction lists
+                         + kXClasses + 2 * kXClasses * nqa                // extraction lists
                          + 1 + 3 * nqa                                    // tensor-core lists
                          + 1 + hj.size();                                 // active tile jobs
     std::vector<uint32_t> ht(words, 0);
@@ -937,7 +944,7 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
         std::copy(g_lvl[v].begin(), g_lvl[v].end(), ht.begin() + o);
         T.g_lvl[v] = take(lv);
     }
-    for (int v = 0; v < kClasses; ++v) {
+    for (int v = 0; v < kXClasses; ++v) {
         std::copy(x_rng[v].begin(), x_rng[v].end(), ht.begin() + o);
         T.x_rng[v] = take(nqa + 1);
     }
@@ -949,9 +956,9 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
     T.g_next = take(kClasses);
     for (int v = 0; v < kClasses; ++v) T.g_pre[v] = take(nqa);
     for (int v = 0; v < kClasses; ++v) T.g_beg[v] = take(nqa);
-    T.x_total = take(kClasses);
-    for (int v = 0; v < kClasses; ++v) T.x_pre[v] = take(nqa);
-    for (int v = 0; v < kClasses; ++v) T.x_beg[v] = take(nqa);
+    T.x_total = take(kXClasses);
+    for (int v = 0; v < kXClasses; ++v) T.x_pre[v] = take(nqa);
+    for (int v = 0; v < kXClasses; ++v) T.x_beg[v] = take(nqa);
     T.t_total = take(1);
     T.t_pre = take(nqa);
     T.t_job_beg = take(nqa);
@@ -994,7 +1001,10 @@ int Executor::enqueue_pass(cudaStream_t st, cudaGraphConditionalHandle h, int us
         ENG_CK(launch_tc_compact(tcjobs.as<TcJob>(), T, max_tc_w, tc_err.as<int>(), st));
     }
     if (ev) ENG_CK(cudaEventRecord(ev[1], st));
-    for (int c = 0; c < kClasses; ++c)
+    for (int c = kExpandNarrow; c <= kExpandWide; ++c)
+        ENG_CK(launch_expand(c == kExpandWide, items[c].as<GItem>(), max_live[c], srcs.as<SrcDesc>(), max_expand_w, T, c,
+                             st));
+    for (int c = 0; c < kExpandNarrow; ++c)
         ENG_CK(launch_gather(kVplOf[c / 2], (c & 1) != 0, items[c].as<GItem>(), max_live[c], srcs.as<SrcDesc>(), T, c,
                              st));
     if (ev) ENG_CK(cudaEventRecord(ev[2], st));
@@ -1005,11 +1015,11 @@ int Executor::enqueue_pass(cudaStream_t st, cudaGraphConditionalHandle h, int us
     if (ev) ENG_CK(cudaEventRecord(ev[3], st));
     // the last extraction launch of the pass also runs the loop control
     int last_x = -1;
-    for (int c = 0; c < kClasses; c += 2)
+    for (int c = 0; c < kXClasses; ++c)
         if (n_xitems[c]) last_x = c;
-    for (int c = 0; c < kClasses; c += 2) {
+    for (int c = 0; c < kXClasses; ++c) {
         const bool fuse = c == last_x;
-        ENG_CK(launch_extract(kVplOf[c / 2], xitems[c].as<XItem>(), n_xitems[c], fds.as<FDesc>(), T, c,
+        ENG_CK(launch_extract(kVplOf[c], xitems[c].as<XItem>(), n_xitems[c], fds.as<FDesc>(), T, c,
                               fuse ? ctl_ptrs.as<QCtl *>() : nullptr, (uint32_t)qs.size(), mirror.as<QCtl>(), h,
                               use_handle, running_out, done_counter.as<unsigned int>(), st));
     }

@@ -26,6 +26,8 @@ namespace cfpq {
 int vpl_for_words(uint32_t W);
 cudaError_t launch_gather(int vpl, bool nt, const GItem *items, uint32_t n_items, const SrcDesc *srcs,
                           const ExecTables &T, int cls, cudaStream_t st);
+cudaError_t launch_expand(bool wide, const GItem *items, uint32_t n_items, const SrcDesc *srcs, uint32_t max_w,
+                          const ExecTables &T, int cls, cudaStream_t st);
 cudaError_t launch_extract(int vpl, const XItem *items, uint32_t n_items, const FDesc *fds, const ExecTables &T,
                            int cls, QCtl *const *ctls, uint32_t nq, QCtl *mirror, cudaGraphConditionalHandle h,
                            int use_handle, int *running_out, unsigned int *done_counter, cudaStream_t st);
@@ -329,14 +331,14 @@ constexpr uint32_t kLoopUnroll = 2;
 // Runs the fixpoint of a set of queries with shared launches.
 struct Executor {
     std::vector<QueryDev *> qs;
-    DBuf ctl_ptrs, mirror, items[kClasses], xitems[kClasses], srcs, fds, running;
+    DBuf ctl_ptrs, mirror, items[kClasses], xitems[kXClasses], srcs, fds, running;
     DBuf tcjobs, tcmaps, tables, tc_err, done_counter;
     DBuf scratch;              // the tile jobs' column bitmaps and counts (zeroed every pass)
     size_t scratch_words_total = 0;
     ExecTables T;
-    uint32_t n_items[kClasses] = {0}, n_xitems[kClasses] = {0};
+    uint32_t n_items[kClasses] = {0}, n_xitems[kXClasses] = {0};
     uint32_t max_live[kClasses] = {0};  // bound on live items of a pass: sum over queries of the largest level
-    uint32_t n_tcjobs = 0, max_tc_tiles = 0, max_tc_w = 0;
+    uint32_t n_tcjobs = 0, max_tc_tiles = 0, max_tc_w = 0, max_expand_w = 0;
     uint32_t tile_kind = kTileFp8Pair;  // the tile jobs' kernel (every query of an executor shares it)
     uint32_t item_scale = 1;            // work items span item_scale times the usual rows (a power of 2)
     cudaGraphExec_t exec = nullptr;

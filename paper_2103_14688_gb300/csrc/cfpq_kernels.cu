@@ -710,6 +710,159 @@ __global__ void __launch_bounds__(256, GatherOcc<VPL>::value)
 }
 
 // --------------------------------------------------------------------------
+// Closure pass of the blocks that read no closure row (kExpandNarrow / Wide):
+// every source is a product edge into t itself (a terminal's CSR row or a
+// nonterminal's adjacency row) or a nonterminal edge into a pure-terminal
+// block, whose rows are read as CSR rows (SrcDesc::pure_n).  On Dyck-4 these are
+// C[p, F], C[x_i, y_i], C[x_i, F] and C[q0, p]: every new S-edge (x, y) is
+// expanded by the c_i edges of y, four times.
+//
+// Bound by the latency of that chain (adjacency word -> CSR offsets -> column
+// -> shared-memory atomic) and by uneven rows (most have no new edge, hubs have
+// tens of thousands).  So: no registers or shared memory for closure rows, which
+// leaves 48 warps per SM; the item's rows with work are listed first, 256 marks
+// at a time; a row is expanded by a whole CTA (rows of more than
+// kExpandNarrowW words) or by a warp that takes rows from the list, each
+// thread on its own adjacency words, into a row-sized shared-memory bitmap that is
+// merged into the output row at the end.  As part of k_gather (one warp per row,
+// 8 warps per SM beside the closure-row ring) this took 110 of the 190 ms of
+// gather of Dyck-4 at n = 65536; the query went from 303 to 233 ms.
+// --------------------------------------------------------------------------
+constexpr int kExpandOcc = 6;  // CTAs per SM (40 registers a thread; 32 would spill)
+template <bool WIDE>
+__global__ void __launch_bounds__(256, kExpandOcc)
+    k_expand(const GItem *__restrict__ items, const SrcDesc *__restrict__ srcs, ExecTables T, int cls) {
+    extern __shared__ unsigned long long s_bitmap[];  // WIDE: one row; else one row per warp
+    __shared__ uint16_t s_rows[1024];                 // (an item has at most 1024 rows)
+    __shared__ uint32_t s_nrows, s_take, s_changed;
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const uint32_t t0 = WIDE ? tid : lane;            // this thread's place in its row's group
+    constexpr uint32_t TPR = WIDE ? 256u : 32u;
+    const uint32_t total = T.g_total[cls];
+    for (uint32_t li = blockIdx.x; li < total; li += gridDim.x) {
+        const uint32_t q = find_owner(T.g_pre[cls], T.nq, li);
+        const GItem &it = items[T.g_beg[cls][q] + (li - T.g_pre[cls][q])];
+        QCtl *const c = it.ctl;
+        if (c->phase != kPhaseRun || c->level != it.level) continue;  // (uniform)
+        const uint32_t g = c->g, iter = c->iter, mode = c->mode, g0 = c->g_iter_start, W = it.W;
+        const uint32_t src0 = it.src0, nsrc = it.nsrc, row0 = it.row0, row1 = it.row1;
+        int act = 0;
+        for (uint32_t k = tid; k < nsrc; k += 256u) act |= src_channels<true>(srcs[src0 + k], mode, iter, g, g0, 0u) != 0u;
+        if (!__syncthreads_or(act)) continue;
+        if (tid == 0) { s_nrows = 0u; s_take = 0u; s_changed = 0u; }
+        __syncthreads();
+        // rows with an edge of a source that takes part
+        for (uint32_t r = row0 + tid; r - tid < row1; r += 256u) {
+            bool has = false;
+            if (r < row1 && (!it.rmask || ((it.rmask[r >> 6] >> (r & 63u)) & 1ull))) {
+                for (uint32_t k = 0; k < nsrc && !has; ++k) {
+                    const SrcDesc &d = srcs[src0 + k];
+                    const uint32_t ch = src_channels<true>(d, mode, iter, g, g0, 0u);
+                    if (!ch) continue;
+                    if (d.csr_off) has = d.csr_off[r + 1] > d.csr_off[r];
+                    else has = (ch & 6u) ? d.nt_new_it[r] != 0u : d.nt_new_it[r] == iter;  // (0: the row has no edge)
+                }
+            }
+            const unsigned bal = __ballot_sync(FULLMASK, has);
+            uint32_t base = 0u;
+            if (lane == 0u && bal) base = atomicAdd(&s_nrows, (uint32_t)__popc(bal));
+            base = __shfl_sync(FULLMASK, base, 0);
+            if (has) s_rows[base + (uint32_t)__popc(bal & ((1u << lane) - 1u))] = (uint16_t)(r - row0);
+        }
+        __syncthreads();
+        const uint32_t nrows = s_nrows;
+        unsigned long long *const bm = s_bitmap + (WIDE ? 0u : warp * W);
+        unsigned int *const bm32 = reinterpret_cast<unsigned int *>(bm);
+        const uint32_t w0 = c->col_v0 * 2u, w1 = min(c->col_v1, W / 2u) * 2u;  // this rank's columns (all unless sharded)
+        uint32_t my_changed = 0u;
+        for (uint32_t i = 0;; ++i) {
+            if (!WIDE) {
+                if (lane == 0u) i = atomicAdd(&s_take, 1u);
+                i = __shfl_sync(FULLMASK, i, 0);
+            }
+            if (i >= nrows) break;
+            const uint32_t row = row0 + s_rows[i];
+            for (uint32_t w = t0; w < W; w += TPR) bm[w] = 0ull;
+            if (WIDE) __syncthreads();
+            else __syncwarp();
+            for (uint32_t k = 0; k < nsrc; ++k) {
+                const SrcDesc &d = srcs[src0 + k];
+                const uint32_t ch = src_channels<true>(d, mode, iter, g, g0, 0u);
+                if (!ch) continue;
+                if (d.csr_off) {  // the terminal's product edges (iteration 1)
+                    const uint32_t e1 = d.csr_off[row + 1];
+                    for (uint32_t e = d.csr_off[row] + t0; e < e1; e += TPR) {
+                        const uint32_t z = d.csr_col[e];
+                        atomicOr(bm32 + (z >> 5), 1u << (z & 31u));
+                    }
+                    continue;
+                }
+                for (uint32_t cb = 1u; cb <= ch; cb <<= 1) {
+                    if (!(ch & cb)) continue;
+                    const bool new_edges = cb == 1u;
+                    if (new_edges && d.nt_new_it[row] != iter) continue;
+                    const unsigned long long *adj = reinterpret_cast<const unsigned long long *>(
+                        (new_edges ? d.nt_new : d.nt_all) + (size_t)row * W);
+                    if (d.ident) {
+                        if (new_edges)
+                            for (uint32_t w = t0; w < W; w += TPR) {
+                                const unsigned long long v = adj[w];
+                                if (v) atomicOr(bm + w, v);
+                            }
+                        continue;
+                    }
+                    const uint32_t thr = new_edges ? 0u : (cb == 2u ? g0 : g - 1u);
+                    const uint32_t pn = d.pure_n;
+                    for (uint32_t w = t0; w < W; w += TPR) {
+                        unsigned long long v = adj[w];
+                        if (!v) continue;
+                        v &= pn > 1u ? d.pure_mask[0][w] | d.pure_mask[1][w] : d.pure_mask[0][w];
+                        while (v) {
+                            const uint32_t y = w * 64u + (uint32_t)__ffsll((long long)v) - 1u;
+                            v &= v - 1ull;
+                            if (thr && d.rstamp[y] < thr) continue;
+                            for (uint32_t p = 0; p < pn; ++p) {
+                                const uint32_t e1 = d.pure_off[p][y + 1];
+                                for (uint32_t e = d.pure_off[p][y]; e < e1; ++e) {
+                                    const uint32_t z = d.pure_col[e];
+                                    atomicOr(bm32 + (z >> 5), 1u << (z & 31u));
+                                }
+                            }
+                        }
+                    }
+                }
+            }
+            if (WIDE) __syncthreads();
+            else __syncwarp();
+            bool ch = false;
+            unsigned long long *const o = reinterpret_cast<unsigned long long *>(it.out) + (size_t)row * W;
+            for (uint32_t w = w0 + t0; w < w1; w += TPR) {
+                const unsigned long long v = bm[w];
+                if (!v) continue;
+                const unsigned long long old = o[w];
+                if (v & ~old) {
+                    o[w] = old | v;
+                    ch = true;
+                }
+            }
+            // (also orders this row's bitmap reads before the next row's clearing)
+            const bool any = WIDE ? __syncthreads_or(ch) != 0 : __any_sync(FULLMASK, ch) != 0;
+            if (any && t0 == 0u) {
+                it.out_stamp[row] = g;
+                ++my_changed;
+            }
+        }
+        if (my_changed) atomicAdd(&s_changed, my_changed);
+        __syncthreads();
+        if (tid == 0 && s_changed) {
+            *it.out_last = g;
+            atomicAdd(&c->changed_rows, (unsigned long long)s_changed);
+        }
+        __syncthreads();
+    }
+}
+
+// --------------------------------------------------------------------------
 // Extraction: runs for a query only after a pass that changed no row.
 // --------------------------------------------------------------------------
 __device__ void control_body(QCtl *const *ctls, uint32_t nq, QCtl *mirror, cudaGraphConditionalHandle handle,
@@ -919,10 +1072,11 @@ __device__ void control_body(QCtl *const *ctls, uint32_t nq, QCtl *mirror, cudaG
     }
     running = __syncthreads_or(running);
     // Live work of the next pass: the items of the current level of every
-    // running query.  All 2 * kClasses + 1 counts of a query sit in registers
+    // running query.  All kClasses + kXClasses + 1 counts of a query sit in registers
     // and are scanned together across the CTA (warp shuffles, then the warp
     // totals), one chunk of blockDim queries at a time.
-    constexpr int K = 2 * kClasses + 1;
+    constexpr int K = kClasses + kXClasses + 1;
+    static_assert(K <= 32, "one thread per count");
     __shared__ uint32_t s_wsum[32][K];
     __shared__ uint32_t s_carry[K];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (int)((blockDim.x + 31) >> 5);
@@ -943,6 +1097,9 @@ __device__ void control_body(QCtl *const *ctls, uint32_t nq, QCtl *mirror, cudaG
                 const uint32_t gb = run ? T.g_lvl[v][base] : 0u, ge = run ? T.g_lvl[v][base + 1] : 0u;
                 T.g_beg[v][q] = gb;
                 cnt[v] = ge - gb;
+            }
+#pragma unroll
+            for (int v = 0; v < kXClasses; ++v) {
                 const uint32_t xb = last ? T.x_rng[v][q] : 0u, xe = last ? T.x_rng[v][q + 1] : 0u;
                 T.x_beg[v][q] = xb;
                 cnt[kClasses + v] = xe - xb;
@@ -982,7 +1139,7 @@ __device__ void control_body(QCtl *const *ctls, uint32_t nq, QCtl *mirror, cudaG
             for (int k = 0; k < K; ++k) {
                 const uint32_t pre = s_carry[k] + (wid ? s_wsum[wid - 1][k] : 0u) + inc[k] - cnt[k];
                 if (k < kClasses) T.g_pre[k][q] = pre;
-                else if (k < 2 * kClasses) T.x_pre[k - kClasses][q] = pre;
+                else if (k < kClasses + kXClasses) T.x_pre[k - kClasses][q] = pre;
                 else T.t_pre[q] = pre;
             }
         }
@@ -1010,7 +1167,7 @@ __device__ void control_body(QCtl *const *ctls, uint32_t nq, QCtl *mirror, cudaG
         const int k = threadIdx.x;
         if (k < kClasses) T.g_next[k] = 0u;  // dynamic gather units of the next pass
         if (k < kClasses) T.g_total[k] = s_carry[k];
-        else if (k < 2 * kClasses) T.x_total[k - kClasses] = s_carry[k];
+        else if (k < kClasses + kXClasses) T.x_total[k - kClasses] = s_carry[k];
         else *T.t_total = s_carry[k];
     }
     if (threadIdx.x == 0) {
@@ -1320,6 +1477,18 @@ cudaError_t launch_gather(int vpl, bool nt, const GItem *items, uint32_t n_items
         default: return cudaErrorInvalidValue;
     }
 #undef CFPQ_GATHER
+    return cudaGetLastError();
+}
+
+cudaError_t launch_expand(bool wide, const GItem *items, uint32_t n_items, const SrcDesc *srcs, uint32_t max_w,
+                          const ExecTables &T, int cls, cudaStream_t st) {
+    if (n_items == 0) return cudaSuccess;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const uint32_t sms = (dev >= 0 && dev < 64 && g_gather_sms[dev]) ? (uint32_t)g_gather_sms[dev] : 0u;
+    const uint32_t grid = sms ? std::min<uint32_t>(n_items, sms * (uint32_t)kExpandOcc) : n_items;  // resident CTAs stride over the items
+    if (wide) k_expand<true><<<grid, 256, (size_t)max_w * 8, st>>>(items, srcs, T, cls);
+    else k_expand<false><<<grid, 256, (size_t)std::min(max_w, kExpandNarrowW) * 8 * 8, st>>>(items, srcs, T, cls);
     return cudaGetLastError();
 }
 

@@ -116,8 +116,7 @@ struct SrcDesc {
     const uint32_t *pure_col;
     const uint64_t *pure_mask[2];  // per label: bit y set iff y has an edge of it (W words)
     // Tile source with a product job for the iteration's new edges
-    // (TcJob::covers_new): while its tiles are on and that job runs in this
-    // pass (new_tiles_pay on its counts: tc_kcount, tagged with the pass, at
+    // (TcJob::covers_new): when that job runs in this pass (new_tiles_pay on its counts: tc_kcount, tagged with the pass, at
     // most tc_kcap rows; tc_mcount; tc_ecount), the row gather leaves the new
     // edges' row ORs to the tiles and keeps only the product edges
     // themselves (ident).
@@ -196,7 +195,7 @@ struct TcJob {
     uint32_t tiles_m, tiles_n;  // tiles of this job
     uint32_t tile0;             // first global tile index of this job
     uint32_t box;               // nonterminal label (switchable jobs)
-    uint32_t switchable;        // active only while the box is dense (closure mode AUTO)
+    uint32_t switchable;        // channels 2, 4: active only while the box is dense (closure mode AUTO)
     uint32_t kcap;              // most compacted rows (a multiple of 128)
     // Dirty-row compaction (channels 2 and 4): before the products of a pass,
     // the B rows with stamp >= thr are listed in `ys`; A's columns at those
@@ -320,7 +319,9 @@ __device__ inline bool tc_job_active(const TcJob &j, uint32_t *thr, uint32_t *it
     }
     const QCtl *c = j.ctl;
     if (c->phase != kPhaseRun || c->level != j.level) return false;
-    if (j.switchable && (j.box >= 32u || !((c->dense_mask >> j.box) & 1u))) return false;
+    // (a channel-1 job's own counts say whether it pays; the other channels
+    // of a switchable source move to tiles once its box is dense)
+    if (j.switchable && j.chan != 1u && (j.box >= 32u || !((c->dense_mask >> j.box) & 1u))) return false;
     *iter = c->iter;
     *g = c->g;
     const uint32_t g0 = c->g_iter_start;

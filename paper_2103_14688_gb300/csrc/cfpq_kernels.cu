@@ -188,8 +188,11 @@ __device__ __forceinline__ int lowbit4(uint4 &v, bool clear) {
 // its box is dense) run as tile products over the dirty rows instead.  When
 // the source's channel-1 tile job (SrcDesc::tile_new) runs in this pass,
 // channel 1's row ORs go to the tiles too: the result keeps channel 1 only
-// for the product edges themselves (ident), flagged by bit 8 (read no
-// closure rows).
+// for the product edges themselves (ident), flagged by bit 8 (channel 1 reads
+// no closure rows).  That job does not wait for the box to be dense: the
+// iteration in which Dyck-4's answer turns dense adds a quarter of its edges to a box that
+// was sparse at its start, and the hub rows of its row gather took 30 ms
+// of the n = 65536 query (4 ms of 16384's); see new_tiles_pay.
 template <bool NT>
 __device__ __forceinline__ uint32_t src_channels(const SrcDesc &d, uint32_t mode, uint32_t iter, uint32_t g,
                                                  uint32_t g0, uint32_t dense_mask) {
@@ -203,12 +206,12 @@ __device__ __forceinline__ uint32_t src_channels(const SrcDesc &d, uint32_t mode
     } else {
         if (d.rblk && d.same_level && *d.rlast + 1u >= g) ch |= 4u;
     }
-    if (!tiles) return ch;
-    ch &= 1u;
-    if (NT && ch && d.tile_new && d.tc_kcount) {
+    if (tiles) ch &= 1u;
+    if (NT && (ch & 1u) && d.tile_new && d.tc_kcount) {
         const unsigned long long kc = *reinterpret_cast<const volatile unsigned long long *>(d.tc_kcount);
         const uint32_t listed = ((uint32_t)(kc >> 32) == g) ? (uint32_t)kc : 0u;
-        if (new_tiles_pay(listed, d.tc_kcap, *d.tc_mcount, *d.tc_ecount, d.tc_ratio)) ch = d.ident ? 9u : 0u;
+        if (new_tiles_pay(listed, d.tc_kcap, *d.tc_mcount, *d.tc_ecount, d.tc_ratio))
+            ch = (ch & ~1u) | (d.ident ? 9u : 0u);
     }
     return ch;
 }
@@ -406,12 +409,12 @@ __global__ void __launch_bounds__(256, GatherOcc<VPL>::value)
                 chans = src_channels<NT>(srcs[it.src0 + k], mode, iter, g, g0, dmask);
             if (!chans) continue;  // the source takes no part in this pass
             const SrcDesc d = srcs[it.src0 + k];
-            // closure rows read by this source (none when the tiles OR them:
-            // only the product edges themselves are left here)
-            const uint64_t *const rblk = (NT && (chans & 8u)) ? nullptr : d.rblk;
             for (uint32_t cbit = 1u; cbit <= 4u; cbit <<= 1) {
                 if (!(chans & cbit)) continue;
                 const bool new_edges = cbit == 1u;
+                // closure rows read (none for new edges whose rows the tiles OR:
+                // only the product edges themselves are left here)
+                const uint64_t *const rblk = (NT && new_edges && (chans & 8u)) ? nullptr : d.rblk;
                 const bool use_ident = new_edges && d.ident;
                 if (!use_ident && rblk == nullptr) continue;
                 // a source row takes part when its stamp is >= thr

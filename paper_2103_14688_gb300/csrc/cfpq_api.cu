@@ -186,6 +186,7 @@ int ensure_query(cfpq_ctx *ctx, bool restricted = false) {
         if (int rc = set_device(ctx)) return rc;  // (a probe may have run)
     }
     q.gather_slices = ctx->opt.gather_slices;
+    q.use_slices = ctx->opt.max_rounds == 0;
     q.full_kcap = true;
     if (q.restricted != restricted) ctx->exec_dirty = true;  // the work items carry the row masks
     q.restricted = restricted;
@@ -945,6 +946,7 @@ extern "C" int cfpq_batch_run(cfpq_ctx *ctx, uint32_t n_queries, const cfpq_quer
         q->closure_mode = ctx->opt.closure_mode;
         set_tiles(*q, ctx->opt, ctx->stream, max_n);
         q->gather_slices = ctx->opt.gather_slices;
+        q->use_slices = ctx->opt.max_rounds == 0;
         rc = copy_rsm(qq.rsm, &q->rsm, &e);
         if (rc) return fail(ctx, rc, "query " + std::to_string(i) + ": " + e);
         q->g = g.get();

@@ -123,6 +123,7 @@ struct SrcDesc {
     uint32_t tile_new;
     uint32_t tc_kcap;
     uint32_t tc_ratio;         // new_tiles_pay's ratio for the job's tile format
+    uint32_t slice_mem;        // source of a sliced block: member whose block it reads, or kSliceNone
     const unsigned long long *tc_kcount;
     const unsigned long long *tc_mcount;
     const unsigned long long *tc_ecount;
@@ -152,6 +153,28 @@ struct GItem {
     uint32_t slice;
     uint32_t nt_boxes;
     uint32_t pad;
+};
+
+// A cyclic component of RSM states whose transitions all read terminals, with
+// one target state t: its blocks C[s, t], s in the component, are closed
+// together, one column word at a time (k_slice).  Item: one word of one group.
+constexpr uint32_t kSliceNone = 0xFFFFFFFFu;
+constexpr uint32_t kSliceMaxSrc = 32;              // sources of a group that read its own blocks
+constexpr uint32_t kSliceMaxBytes = 200u << 10;    // shared memory of a slice: members x n x 9 bytes
+struct SliceGroup {
+    QCtl *ctl;
+    const uint32_t *coo;  // the graph's edges as x << 16 | y, in CSR order
+    uint32_t level, n, W;
+    uint32_t mem0, nmem;  // members (SliceMem)
+    uint32_t pad;
+};
+struct SliceMem {
+    uint64_t *out;
+    uint32_t *stamp, *last;
+    uint32_t src0, nsrc;  // sources (SrcDesc::slice_mem: the member read, or kSliceNone)
+};
+struct SliceItem {
+    uint32_t group, w;
 };
 
 // Final-state block used by extraction: C[q0(b), f] with f final in box b.
@@ -280,8 +303,9 @@ constexpr int kVplClasses = 5;
 // Blocks whose sources read no closure row at all (kExpand: see k_expand), rows
 // of at most / of more than kExpandNarrowW words, have classes of their own.
 // Extraction: the row width class.
-constexpr int kExpandNarrow = 2 * kVplClasses, kExpandWide = kExpandNarrow + 1;
-constexpr int kClasses = kExpandWide + 1, kXClasses = kVplClasses;
+// Column slices of cyclic components (kSlice: see k_slice) are the last class.
+constexpr int kExpandNarrow = 2 * kVplClasses, kExpandWide = kExpandNarrow + 1, kSlice = kExpandWide + 1;
+constexpr int kClasses = kSlice + 1, kXClasses = kVplClasses;
 constexpr uint32_t kExpandNarrowW = 128;
 struct ExecTables {
     uint32_t nq;

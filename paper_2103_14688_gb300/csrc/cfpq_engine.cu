@@ -298,6 +298,15 @@ int GraphDev::ensure_nonempty(Allocator *A, cudaStream_t st, std::string *err) {
     return CFPQ_OK;
 }
 
+int GraphDev::ensure_coo(Allocator *A, cudaStream_t st, std::string *err) {
+    if (coo.p && coo_content == content) return CFPQ_OK;
+    if (!coo.ensure(A, csr_col.bytes, err)) return CFPQ_ERR_OUT_OF_MEMORY;  // (as many edges as the CSR has room for)
+    ENG_CK(launch_csr_to_coo(csr_off.as<uint32_t>(), csr_col.as<uint32_t>(), (size_t)n_term * n, n, coo.as<uint32_t>(),
+                             st));
+    coo_content = content;
+    return CFPQ_OK;
+}
+
 int GraphDev::ensure_term_bits(Allocator *A, cudaStream_t st, std::string *err) {
     if (term_bits.p && term_bits_content == content) return CFPQ_OK;
     const size_t rows = (size_t)n_term * n;
@@ -410,6 +419,37 @@ int QueryDev::plan(std::string *err) {
         }
         blk_nsrc[b] = (uint32_t)srcs.size() - blk_src0[b];
     }
+    // Column slices: the blocks C[s, t] of a cyclic component (s over its
+    // states) when every source is a terminal's, none runs on tiles, and the
+    // component's column word fits an SM.
+    blk_slice.assign(blocks.size(), -1);
+    n_slice_groups = 0;
+    loop_mask = cyclic_mask;
+    if (use_slices && !restricted && !closure_all_tiles(closure_mode)) {
+        for (uint32_t c = 0; c < Q; ++c) {
+            if (comp[c] != c || !reach[(size_t)c * Q + c]) continue;
+            uint32_t members = 0;
+            bool ok = true;
+            for (uint32_t s = 0; s < Q; ++s) {
+                if (comp[s] != c) continue;
+                ++members;
+                for (const auto &tr : rsm.tr) ok &= tr.from != s || tr.kind == 0;
+            }
+            ok = ok && (uint64_t)members * n * 9u <= kSliceMaxBytes;
+            for (uint32_t t = 0; t < Q && ok; ++t) {
+                uint32_t same = 0;  // sources of the group's blocks that read its own blocks
+                for (const auto &tr : rsm.tr)
+                    same += (comp[tr.from] == c && comp[tr.to] == c) ? 1u : 0u;
+                if (same > kSliceMaxSrc || blk_of[(size_t)c * Q + t] < 0) continue;
+                for (uint32_t s = 0; s < Q; ++s)
+                    if (comp[s] == c) blk_slice[(size_t)blk_of[(size_t)s * Q + t]] = (int32_t)n_slice_groups;
+                ++n_slice_groups;
+            }
+        }
+        loop_mask = 0;
+        for (size_t b = 0; b < blocks.size(); ++b)
+            if (reach[(size_t)blocks[b].first * Q + blocks[b].first] && blk_slice[b] < 0) loop_mask |= 1ull << blk_level[b];
+    }
     // Boxes read by some transition (bit 63: a box >= 63 is read).
     nt_read_mask = 0;
     for (const auto &tr : rsm.tr)
@@ -517,12 +557,14 @@ int QueryDev::refresh_graph_caches(Allocator *A, cudaStream_t st, std::string *e
         need_term_bits |= (sdesc.dense && sdesc.label_kind == 0);
         need_nonempty |= sdesc.pure_rb != 0;
     }
-    const void *p_ne = g->nonempty.p, *p_tb = g->term_bits.p;
+    const void *p_ne = g->nonempty.p, *p_tb = g->term_bits.p, *p_coo = g->coo.p;
+    if (n_slice_groups)
+        if (int rc = g->ensure_coo(A, st, err)) return rc;
     if (need_nonempty)
         if (int rc = g->ensure_nonempty(A, st, err)) return rc;
     if (need_term_bits)
         if (int rc = g->ensure_term_bits(A, st, err)) return rc;
-    *moved = (need_nonempty && g->nonempty.p != p_ne) || (need_term_bits && g->term_bits.p != p_tb);
+    *moved = (n_slice_groups && g->coo.p != p_coo) || (need_nonempty && g->nonempty.p != p_ne) || (need_term_bits && g->term_bits.p != p_tb);
     return CFPQ_OK;
 }
 
@@ -567,7 +609,7 @@ int QueryDev::enqueue_init(cudaStream_t st, uint32_t max_iter, uint32_t max_roun
     for (uint32_t k = 0; k < n_tc_src; ++k) ENG_CK(cudaMemsetAsync(tc_kcount(k), 0, 8, st));
     // per-box edge counts: the dense-box mask drives AUTO's tile switch and
     // the column slices of the row gather in every mode
-    ENG_CK(launch_ctl_reset(ctl_ptr_mem.as<QCtl *>(), 1, max_iter, max_rounds, max_passes, n_levels, cyclic_mask,
+    ENG_CK(launch_ctl_reset(ctl_ptr_mem.as<QCtl *>(), 1, max_iter, max_rounds, max_passes, n_levels, loop_mask,
                             boxedge_mem.as<unsigned long long>(), B, n, boxit_mem.as<uint32_t>(), nt_read_mask, st));
     ENG_CK(launch_eps_init(eps_mem.p, n_eps, 152, st));
     if (seeded)
@@ -601,7 +643,11 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
     for (QueryDev *q : qs) maxL1 = std::max(maxL1, q->n_levels + 1);
     std::vector<QCtl *> hp;
     std::vector<SrcDesc> hs;
-    std::vector<GItem> hi[kClasses];
+    std::vector<GItem> hi[kSlice];
+    std::vector<SliceItem> hsi;
+    std::vector<SliceGroup> hsg;
+    std::vector<SliceMem> hsm;
+    slice_smem = 0;
     std::vector<FDesc> hf;
     std::vector<XItem> hx[kXClasses];
     std::vector<TcJob> hj;
@@ -679,6 +725,7 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
             d.dense = sd.dense;
             d.box_switch = sd.box_switch;
             d.label_box = sd.label_kind == 1 ? sd.label : 0u;
+            d.slice_mem = kSliceNone;
             if (sd.tc_slot_new >= 0) {
                 // the channel-1 job's counts, in the executor's scratch buffer
                 // (offsets, made pointers below)
@@ -701,12 +748,33 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
         // product jobs: tcgen05 tiles of 128 rows x 256 columns
         const uint32_t tiles_m = (q.n + 127u) / 128u, tiles_n = (q.n + 255u) / 256u;
         for (uint32_t L = 0; L <= q.n_levels; ++L) {
-            for (int v = 0; v < kClasses; ++v) g_lvl[v][(size_t)qi * maxL1 + L] = (uint32_t)hi[v].size();
+            for (int v = 0; v < kClasses; ++v)
+                g_lvl[v][(size_t)qi * maxL1 + L] = (uint32_t)(v == kSlice ? hsi.size() : hi[v].size());
             t_lvl[(size_t)qi * maxL1 + L] = (uint32_t)hj.size();
             if (L == q.n_levels) break;
             uint32_t lvl_tiles = 0;
+            for (uint32_t sg = 0; sg < q.n_slice_groups; ++sg) {
+                const uint32_t mem0 = (uint32_t)hsm.size();
+                std::vector<int32_t> member_of(q.blocks.size(), -1);
+                for (size_t b = 0; b < q.blocks.size(); ++b) {
+                    if (q.blk_slice[b] != (int32_t)sg || q.blk_level[b] != L) continue;
+                    member_of[b] = (int32_t)(hsm.size() - mem0);
+                    hsm.push_back(SliceMem{q.blk_ptr((uint32_t)b), q.stamp_ptr((uint32_t)b),
+                                           q.last_mem.as<uint32_t>() + b, base + q.blk_src0[b], q.blk_nsrc[b]});
+                }
+                const uint32_t nmem = (uint32_t)hsm.size() - mem0;
+                if (nmem == 0) continue;  // a group of another level
+                for (uint32_t k = 0; k < nmem; ++k)
+                    for (uint32_t j = hsm[mem0 + k].src0; j < hsm[mem0 + k].src0 + hsm[mem0 + k].nsrc; ++j) {
+                        const int32_t rb = q.srcs[j - base].rblk;
+                        if (rb >= 0 && member_of[(size_t)rb] >= 0) hs[j].slice_mem = (uint32_t)member_of[(size_t)rb];
+                    }
+                for (uint32_t w = 0; w < q.W; ++w) hsi.push_back(SliceItem{(uint32_t)hsg.size(), w});
+                hsg.push_back(SliceGroup{cp, g.coo.as<uint32_t>(), L, q.n, q.W, mem0, nmem, 0u});
+                slice_smem = std::max(slice_smem, nmem * q.n * 9u);
+            }
             for (size_t b = 0; b < q.blocks.size(); ++b) {
-                if (q.blk_level[b] != L || q.blk_nsrc[b] == 0) continue;
+                if (q.blk_level[b] != L || q.blk_nsrc[b] == 0 || q.blk_slice[b] >= 0) continue;
                 bool has_nt = false, expand = true;
                 for (uint32_t k = 0; k < q.blk_nsrc[b]; ++k) {
                     const auto &sd = q.srcs[q.blk_src0[b] + k];
@@ -925,9 +993,13 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
     }
     for (int v = 0; v < kClasses; ++v) {
         max_live[v] = live_bound[v];
-        n_items[v] = (uint32_t)hi[v].size();
-        if ((rc = upload(items[v], hi[v].data(), hi[v].size() * sizeof(GItem)))) return rc;
+        n_items[v] = (uint32_t)(v == kSlice ? hsi.size() : hi[v].size());
+        rc = v == kSlice ? upload(items[v], hsi.data(), hsi.size() * sizeof(SliceItem))
+                         : upload(items[v], hi[v].data(), hi[v].size() * sizeof(GItem));
+        if (rc) return rc;
     }
+    if ((rc = upload(slice_groups, hsg.data(), hsg.size() * sizeof(SliceGroup)))) return rc;
+    if ((rc = upload(slice_mems, hsm.data(), hsm.size() * sizeof(SliceMem)))) return rc;
     for (int v = 0; v < kXClasses; ++v) {
         n_xitems[v] = (uint32_t)hx[v].size();
         if ((rc = upload(xitems[v], hx[v].data(), hx[v].size() * sizeof(XItem)))) return rc;
@@ -1013,6 +1085,8 @@ int Executor::enqueue_pass(cudaStream_t st, cudaGraphConditionalHandle h, int us
         ENG_CK(launch_tc_compact(tcjobs.as<TcJob>(), T, max_tc_w, tc_err.as<int>(), st));
     }
     if (ev) ENG_CK(cudaEventRecord(ev[1], st));
+    ENG_CK(launch_slice(items[kSlice].as<SliceItem>(), max_live[kSlice], slice_groups.as<SliceGroup>(),
+                        slice_mems.as<SliceMem>(), srcs.as<SrcDesc>(), slice_smem, T, kSlice, st));
     for (int c = kExpandNarrow; c <= kExpandWide; ++c)
         ENG_CK(launch_expand(c == kExpandWide, items[c].as<GItem>(), max_live[c], srcs.as<SrcDesc>(), max_expand_w, T, c,
                              st));

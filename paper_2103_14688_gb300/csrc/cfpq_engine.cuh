@@ -28,6 +28,8 @@ cudaError_t launch_gather(int vpl, bool nt, const GItem *items, uint32_t n_items
                           const ExecTables &T, int cls, cudaStream_t st);
 cudaError_t launch_expand(bool wide, const GItem *items, uint32_t n_items, const SrcDesc *srcs, uint32_t max_w,
                           const ExecTables &T, int cls, cudaStream_t st);
+cudaError_t launch_slice(const SliceItem *items, uint32_t n_items, const SliceGroup *groups, const SliceMem *mems,
+                         const SrcDesc *srcs, uint32_t smem, const ExecTables &T, int cls, cudaStream_t st);
 cudaError_t launch_extract(int vpl, const XItem *items, uint32_t n_items, const FDesc *fds, const ExecTables &T,
                            int cls, QCtl *const *ctls, uint32_t nq, QCtl *mirror, cudaGraphConditionalHandle h,
                            int use_handle, int *running_out, unsigned int *done_counter, cudaStream_t st);
@@ -76,6 +78,8 @@ cudaError_t launch_stage_unique(const uint32_t *off, uint32_t *col, uint32_t *uc
 cudaError_t launch_stage_compact(const uint32_t *off, const uint32_t *col, const uint32_t *uoff, uint32_t *ucol,
                                  size_t rows, cudaStream_t st);
 cudaError_t launch_popcount(const uint64_t *p, size_t nwords, unsigned long long *out, cudaStream_t st);
+cudaError_t launch_csr_to_coo(const uint32_t *off, const uint32_t *col, size_t rows, uint32_t n, uint32_t *coo,
+                              cudaStream_t st);
 cudaError_t launch_nonempty_bits(const uint32_t *off, uint32_t n, uint32_t n_term, uint32_t W, uint64_t *bits,
                                  cudaStream_t st);
 cudaError_t launch_pack_rows(const uint64_t *src, uint32_t W, uint32_t wn, uint32_t r0, uint32_t rows, uint64_t *out,
@@ -187,6 +191,9 @@ struct GraphDev {
     DBuf nonempty;  // [n_term * W] bit y of label l: row (l, y) of the CSR has an edge (pure-terminal reads)
     uint64_t nonempty_content = ~0ull;
     int ensure_nonempty(Allocator *A, cudaStream_t st, std::string *err);
+    DBuf coo;  // [m] edges as x << 16 | y (column slices)
+    uint64_t coo_content = ~0ull;
+    int ensure_coo(Allocator *A, cudaStream_t st, std::string *err);
     // staging scratch
     DBuf e_src, e_lbl, e_dst, cnt, off, col, ucnt, scan_tmp, label_map, err;
     std::vector<uint32_t> h_off;  // host copies on demand (paths)
@@ -259,6 +266,14 @@ struct QueryDev {
     std::vector<uint32_t> blk_level;           // per block, 0..n_levels-1
     uint32_t n_levels = 1;
     uint64_t cyclic_mask = 0;
+    // Cyclic components closed in column slices (use_slices: not with a round
+    // cap, whose rounds they do not take): per block its group or -1, and the
+    // levels that still repeat, cyclic_mask without those all of whose cyclic
+    // blocks are sliced.
+    bool use_slices = false;
+    std::vector<int32_t> blk_slice;
+    uint32_t n_slice_groups = 0;
+    uint64_t loop_mask = 0;
     unsigned long long nt_read_mask = 0;  // boxes read by some transition (bit 63: some box >= 63)
     std::vector<Src> srcs;
     std::vector<uint32_t> box_f0, box_nf;
@@ -335,6 +350,8 @@ struct Executor {
     DBuf tcjobs, tcmaps, tables, tc_err, done_counter;
     DBuf scratch;              // the tile jobs' column bitmaps and counts (zeroed every pass)
     size_t scratch_words_total = 0;
+    DBuf slice_groups, slice_mems;
+    uint32_t slice_smem = 0;  // shared memory of the largest slice
     ExecTables T;
     uint32_t n_items[kClasses] = {0}, n_xitems[kXClasses] = {0};
     uint32_t max_live[kClasses] = {0};  // bound on live items of a pass: sum over queries of the largest level

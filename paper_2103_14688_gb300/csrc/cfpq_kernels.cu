@@ -866,6 +866,186 @@ __global__ void __launch_bounds__(256, kExpandOcc)
 }
 
 // --------------------------------------------------------------------------
+// Closure of a cyclic component, one column word at a time (kSlice).  Word w
+// of row x of C[s, t] depends only on word w of the rows it reads, so a CTA
+// holds that word of every row of the component's blocks C[., t] in shared
+// memory and sweeps the component's product edges until nothing changes, with
+// a barrier per sweep: the level's fixpoint in one pass.
+//
+// The row gather needs a pass (two launches and a grid-wide wait, 22 us at
+// least) per hop of the longest path: (ab)*c|a*b* took 70 passes at n = 1000 and
+// 32 at n = 8192.  What bounds a sweep is instructions and shared-memory bank
+// conflicts, so it runs over edges, not rows (rows of unequal degree left two
+// thirds of the lanes idle: 9 us a sweep at n = 8192): 32 packed edges (x << 16 |
+// y) per warp and coalesced load, eight in flight a thread; a byte per row holds
+// the sweep that last changed it, and only edges from rows changed in this sweep or
+// the one before read their words.  Regular query: n = 1000 1785 -> 385 us,
+// n = 8192 2119 -> 1369 us.  Above 200 KB a slice (n = 22755 for one state) the
+// component stays on the row gather, which also does less work on the sparse
+// rows that such graphs have.
+// --------------------------------------------------------------------------
+constexpr uint32_t kSliceThreads = 1024, kSliceEdges = 4;
+__device__ __forceinline__ void or64(uint64_t *p, uint64_t v) {  // (32-bit shared atomics are native)
+    unsigned int *h = reinterpret_cast<unsigned int *>(p);
+    if ((uint32_t)v) atomicOr(h, (uint32_t)v);
+    if ((uint32_t)(v >> 32)) atomicOr(h + 1, (uint32_t)(v >> 32));
+}
+__global__ void __launch_bounds__(kSliceThreads, 1)
+    k_slice(const SliceItem *__restrict__ items, const SliceGroup *__restrict__ groups,
+            const SliceMem *__restrict__ mems, const SrcDesc *__restrict__ srcs, ExecTables T, int cls) {
+    extern __shared__ uint64_t s_col[];  // [nmem][n] words, then [nmem][n] bytes
+    __shared__ uint32_t s_e0[kSliceMaxSrc], s_e1[kSliceMaxSrc], s_to[kSliceMaxSrc], s_from[kSliceMaxSrc], s_n;
+    __shared__ unsigned long long s_changed, s_ors;
+    const uint32_t tid = threadIdx.x, NT = blockDim.x, total = T.g_total[cls];
+    for (uint32_t li = blockIdx.x; li < total; li += gridDim.x) {
+        const uint32_t q = find_owner(T.g_pre[cls], T.nq, li);
+        const SliceItem it = items[T.g_beg[cls][q] + (li - T.g_pre[cls][q])];
+        const SliceGroup G = groups[it.group];
+        QCtl *const c = G.ctl;
+        if (c->phase != kPhaseRun || c->level != G.level || c->mode != kModeNew) continue;  // (uniform)
+        const uint32_t w = it.w, n = G.n, W = G.W, g = c->g, g0 = c->g_iter_start, rows = G.nmem * n;
+        const uint32_t *const coo = G.coo;
+        const bool first = c->iter == 1u;
+        if ((w >> 1) < c->col_v0 || (w >> 1) >= c->col_v1) continue;  // another rank's columns
+        // work: the terminal edges in iteration 1, afterwards rows of lower levels that changed
+        int act = first ? 1 : 0;
+        for (uint32_t m = 0; m < G.nmem && !first; ++m) {
+            const SliceMem M = mems[G.mem0 + m];
+            for (uint32_t k = tid; k < M.nsrc; k += NT) {
+                const SrcDesc &d = srcs[M.src0 + k];
+                act |= d.rblk && d.slice_mem == kSliceNone && *d.rlast >= g0;
+            }
+        }
+        if (!__syncthreads_or(act)) continue;
+        uint8_t *const s_mark = reinterpret_cast<uint8_t *>(s_col + rows);
+        if (tid == 0) {
+            s_changed = 0ull;
+            s_ors = 0ull;
+            uint32_t k2 = 0u;
+            for (uint32_t m = 0; m < G.nmem; ++m) {
+                const SliceMem M = mems[G.mem0 + m];
+                for (uint32_t k = 0; k < M.nsrc; ++k) {
+                    const SrcDesc &d = srcs[M.src0 + k];
+                    if (d.slice_mem == kSliceNone) continue;
+                    s_e0[k2] = d.csr_off[0];
+                    s_e1[k2] = d.csr_off[n];
+                    s_to[k2] = m * n;
+                    s_from[k2] = d.slice_mem * n;
+                    ++k2;
+                }
+            }
+            s_n = k2;
+        }
+        for (uint32_t m = 0; m < G.nmem; ++m) {
+            const uint64_t *const o = mems[G.mem0 + m].out;
+            for (uint32_t x = tid; x < n; x += NT) s_col[m * n + x] = first ? 0ull : o[(size_t)x * W + w];
+        }
+        __syncthreads();
+        // product edges into t, and rows of lower levels
+        uint32_t my_ors = 0u;
+        for (uint32_t m = 0; m < G.nmem; ++m) {
+            const SliceMem M = mems[G.mem0 + m];
+            uint64_t *const to = s_col + m * n;
+            for (uint32_t k = 0; k < M.nsrc; ++k) {
+                const SrcDesc &d = srcs[M.src0 + k];
+                const bool read = d.rblk && d.slice_mem == kSliceNone && (first || *d.rlast >= g0);
+                const bool ident = first && d.ident;
+                if (!read && !ident) continue;
+                const uint64_t *const r = d.rblk + w;
+                const uint32_t e1 = d.csr_off[n];
+                for (uint32_t e = d.csr_off[0] + tid; e < e1; e += NT) {
+                    const uint32_t xy = coo[e], x = xy >> 16, y = xy & 0xFFFFu;
+                    uint64_t v = 0ull;
+                    if (ident && (y >> 6) == w) v = 1ull << (y & 63u);
+                    if (read && (first || d.rstamp[y] >= g0)) {
+                        v |= r[(size_t)y * W];
+                        ++my_ors;
+                    }
+                    if (v & ~to[x]) or64(to + x, v);
+                }
+            }
+        }
+        __syncthreads();
+        // mark: the low byte of the sweep that last changed the row (rows with bits start as
+        // changed in sweep 0; 128 is no sweep within reach of the first ones)
+        for (uint32_t x = tid; x < rows; x += NT) s_mark[x] = s_col[x] ? 0u : 128u;
+        const uint32_t ns = s_n;
+        uint32_t sweep = 0u;
+        bool ch = true;
+        while (__syncthreads_or(ch)) {
+            ch = false;
+            ++sweep;
+            for (uint32_t k = 0; k < ns; ++k) {
+                uint64_t *const to = s_col + s_to[k];
+                const uint64_t *const from = s_col + s_from[k];
+                uint8_t *const to_mark = s_mark + s_to[k];
+                const uint8_t *const from_mark = s_mark + s_from[k];
+                const uint32_t e1 = s_e1[k];
+                uint32_t next[kSliceEdges];
+#pragma unroll
+                for (uint32_t i = 0; i < kSliceEdges; ++i) {
+                    const uint32_t e = s_e0[k] + tid + i * NT;
+                    next[i] = e < e1 ? coo[e] : 0u;
+                }
+                for (uint32_t e0 = s_e0[k] + tid; e0 < e1; e0 += NT * kSliceEdges) {
+                    uint32_t xy[kSliceEdges];
+                    bool on[kSliceEdges];
+#pragma unroll
+                    for (uint32_t i = 0; i < kSliceEdges; ++i) {
+                        const uint32_t e = e0 + i * NT, ne = e + NT * kSliceEdges;
+                        xy[i] = next[i];
+                        on[i] = e < e1 && ((sweep - from_mark[xy[i] & 0xFFFFu]) & 0xFFu) <= 1u;
+                        next[i] = ne < e1 ? coo[ne] : 0u;  // (in flight while this round is applied)
+                    }
+#pragma unroll
+                    for (uint32_t i = 0; i < kSliceEdges; ++i) {
+                        if (!on[i]) continue;
+                        const uint32_t x = xy[i] >> 16;
+                        const uint64_t v = from[xy[i] & 0xFFFFu] & ~to[x];
+                        ++my_ors;
+                        if (v) {
+                            or64(to + x, v);
+                            to_mark[x] = (uint8_t)sweep;
+                            ch = true;
+                        }
+                    }
+                }
+            }
+        }
+        uint32_t my_changed = 0u;
+        for (uint32_t m = 0; m < G.nmem; ++m) {
+            const SliceMem M = mems[G.mem0 + m];
+            bool any = false;
+            for (uint32_t x = tid; x < n; x += NT) {
+                const uint64_t v = s_col[m * n + x];
+                if (!v) continue;
+                uint64_t *const o = M.out + (size_t)x * W + w;
+                if (first || (v & ~*o)) {
+                    *o = v;
+                    M.stamp[x] = g;
+                    any = true;
+                    ++my_changed;
+                }
+            }
+            if (any) *M.last = g;
+        }
+        // counted in whole rows: W slices make a row
+        my_ors = __reduce_add_sync(FULLMASK, my_ors);
+        my_changed = __reduce_add_sync(FULLMASK, my_changed);
+        if ((tid & 31u) == 0u) {
+            if (my_ors) atomicAdd(&s_ors, (unsigned long long)my_ors);
+            if (my_changed) atomicAdd(&s_changed, (unsigned long long)my_changed);
+        }
+        __syncthreads();  // (also: the next item overwrites s_col and the tables)
+        if (tid == 0) {
+            if (s_ors) atomicAdd(&c->row_ors, (s_ors + W - 1u) / W);
+            if (s_changed) atomicAdd(&c->changed_rows, (s_changed + W - 1u) / W);
+        }
+        __syncthreads();
+    }
+}
+
+// --------------------------------------------------------------------------
 // Extraction: runs for a query only after a pass that changed no row.
 // --------------------------------------------------------------------------
 __device__ void control_body(QCtl *const *ctls, uint32_t nq, QCtl *mirror, cudaGraphConditionalHandle handle,
@@ -1386,6 +1566,15 @@ __global__ void k_csr_to_bits(const uint32_t *__restrict__ off, const uint32_t *
     }
 }
 
+// The CSR's edges with their row: coo[e] = row's vertex << 16 | column (both below 65536).
+__global__ void k_csr_to_coo(const uint32_t *__restrict__ off, const uint32_t *__restrict__ col, size_t rows, uint32_t n,
+                             uint32_t *coo) {
+    for (size_t r = (size_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += (size_t)gridDim.x * blockDim.x) {
+        const uint32_t x = (uint32_t)(r % n) << 16;
+        for (uint32_t e = off[r]; e < off[r + 1]; ++e) coo[e] = x | col[e];
+    }
+}
+
 // bits[l * W + w] bit b = row (l, 64 w + b) of the CSR has an edge.
 __global__ void k_nonempty_bits(const uint32_t *__restrict__ off, uint32_t n, uint32_t n_term, uint32_t W,
                                 uint64_t *bits) {
@@ -1495,9 +1684,28 @@ cudaError_t launch_expand(bool wide, const GItem *items, uint32_t n_items, const
     return cudaGetLastError();
 }
 
-// Shared-memory limits of the general gather variants (call outside any
-// stream capture).
+cudaError_t launch_slice(const SliceItem *items, uint32_t n_items, const SliceGroup *groups, const SliceMem *mems,
+                         const SrcDesc *srcs, uint32_t smem, const ExecTables &T, int cls, cudaStream_t st) {
+    if (n_items == 0) return cudaSuccess;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const uint32_t sms = (dev >= 0 && dev < 64 && g_gather_sms[dev]) ? (uint32_t)g_gather_sms[dev] : 0u;
+    const uint32_t grid = sms ? std::min<uint32_t>(n_items, sms * 4u) : n_items;
+    // small slices: a barrier over 16 warps costs less than their extra loads gain (n = 1000: 44 us
+    // against 56 for a level; n = 8192: 115 against 98)
+    const uint32_t threads = smem >= 4096u * 9u ? kSliceThreads : kSliceThreads / 2u;
+    k_slice<<<grid, threads, smem, st>>>(items, groups, mems, srcs, T, cls);
+    return cudaGetLastError();
+}
+
+// Shared-memory limits of the general gather variants and of the column slices
+// (call outside any stream capture).
 cudaError_t prepare_gather_launch() {
+    {
+        const cudaError_t e =
+            cudaFuncSetAttribute(k_slice, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSliceMaxBytes);
+        if (e != cudaSuccess) return e;
+    }
 #define CFPQ_RING(V)                                                                                      \
     {                                                                                                     \
         const cudaError_t e = cudaFuncSetAttribute(k_gather<V, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
@@ -1620,6 +1828,12 @@ cudaError_t launch_csr_to_bits(const uint32_t *off, const uint32_t *col, size_t 
                                cudaStream_t st) {
     if (rows == 0) return cudaSuccess;
     k_csr_to_bits<<<grid_for(rows, 128), 128, 0, st>>>(off, col, rows, W, bits);
+    return cudaGetLastError();
+}
+cudaError_t launch_csr_to_coo(const uint32_t *off, const uint32_t *col, size_t rows, uint32_t n, uint32_t *coo,
+                              cudaStream_t st) {
+    if (rows == 0) return cudaSuccess;
+    k_csr_to_coo<<<grid_for(rows, 128), 128, 0, st>>>(off, col, rows, n, coo);
     return cudaGetLastError();
 }
 cudaError_t launch_nonempty_bits(const uint32_t *off, uint32_t n, uint32_t n_term, uint32_t W, uint64_t *bits,

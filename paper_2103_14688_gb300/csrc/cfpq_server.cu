@@ -132,6 +132,7 @@ int cfpq_submit(cfpq_server *s, const cfpq_rsm *rsm, uint64_t *ticket) {
             set_tiles(*j.q, o, s->stream, s->graph.n);
         }
         j.q->gather_slices = s->opt.gather_slices;
+        j.q->use_slices = s->opt.max_rounds == 0;
         std::string e;
         int rc = copy_rsm(rsm, &j.q->rsm, &e);
         if (rc) return sfail(s, rc, e);

@@ -243,7 +243,7 @@ struct TcJob {
     // listed rows as W words), and the output row lacks a column that some
     // listed row has (ucols: their OR, W words).  a8 row m is A's row xs[m],
     // m < *mrows.  a_live (null: every row) is zero for rows of A without
-    // any edge.  ucols and mrows are zeroed before every pass.
+    // any edge.  ucols and mrows are zero before every pass.
     const uint32_t *a_live;
     uint64_t *kmask;
     uint64_t *ucols;
@@ -253,7 +253,7 @@ struct TcJob {
     // a_it = their iteration marks) times whole rows of B; K = the columns y
     // of some new edge (newcols, W words) whose row of B was ever written.
     // *mcount = rows with a new edge, *ecount = the number of new edges;
-    // newcols and the counts are zeroed before every pass.  The job runs only
+    // newcols and the counts are zero before every pass.  The job runs only
     // when new_tiles_pay says the tiles beat the row gather on those counts;
     // the gather then skips the channel's row ORs.
     uint32_t covers_new;

@@ -961,6 +961,7 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
     scratch_words_total = n_scratch;
     if (n_scratch) {
         if (!scratch.ensure(A, n_scratch * 8, err)) return CFPQ_ERR_OUT_OF_MEMORY;
+        ENG_CK(cudaMemsetAsync(scratch.p, 0, n_scratch * 8, st));
         uint64_t *nb = scratch.as<uint64_t>();
         auto fix = [nb](auto *&p) {
             using T = std::remove_pointer_t<std::remove_reference_t<decltype(p)>>;
@@ -985,6 +986,8 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
     if ((rc = upload(fds, hf.data(), hf.size() * sizeof(FDesc)))) return rc;
     if ((rc = upload(tcjobs, hj.data(), hj.size() * sizeof(TcJob)))) return rc;
     n_tcjobs = (uint32_t)hj.size();
+    any_uncompacted = false;
+    for (const auto &j : hj) any_uncompacted |= !j.covers_new && j.kcap < j.n;
     // TMA descriptors of the jobs' FP8 operands (a8, b8 per job)
     if (n_maps) {
         std::vector<unsigned char> hm((size_t)n_maps * 2 * tc_map_bytes());
@@ -1062,8 +1065,10 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
 }
 
 int Executor::enqueue_prologue(cudaStream_t st, uint32_t max_iter, uint32_t max_rounds, uint32_t max_passes) {
+    std::string *err = nullptr;
     for (QueryDev *q : qs)
         if (int rc = q->enqueue_init(st, max_iter, max_rounds, max_passes)) return rc;
+    if (scratch_words_total) ENG_CK(cudaMemsetAsync(scratch.p, 0, scratch_words_total * 8, st));
     return enqueue_lists(st);
 }
 
@@ -1073,33 +1078,53 @@ int Executor::enqueue_lists(cudaStream_t st) {
     return CFPQ_OK;
 }
 
+// One pass.  With `branches` (the captured graph) kernels that touch different
+// blocks run side by side: a pass of a small query is a chain of launches that
+// each wait out their memory latency, so what counts is the chain's length.
+//   main:  new columns, row lists, B and A operands, general gathers, tile products
+//   side:  column slices and expanded blocks; CSR gathers
+// The products follow the general gathers, whose plain stores to the same output
+// rows would drop their atomics; extraction and control follow everything.
 int Executor::enqueue_pass(cudaStream_t st, cudaGraphConditionalHandle h, int use_handle, int *running_out,
-                           const cudaEvent_t *ev) {
+                           const cudaEvent_t *ev, bool branches) {
     std::string *err = nullptr;
+    const cudaStream_t sa = branches ? side[0] : st, sb = branches ? side[1] : st;
+    bool side_work[kBranches] = {max_live[kSlice] || max_live[kExpandNarrow] || max_live[kExpandWide], false};
+    for (int c = 0; c < kExpandNarrow; c += 2) side_work[1] |= max_live[c] != 0;
+    if (branches && (side_work[0] || side_work[1])) {
+        ENG_CK(cudaEventRecord(fork_ev, st));
+        for (int i = 0; i < kBranches; ++i)
+            if (side_work[i]) ENG_CK(cudaStreamWaitEvent(side[i], fork_ev, 0));
+    }
     // Tile operands first: the rows the tile jobs multiply were final before
     // this pass (lower levels, or the previous pass of a cyclic level), and a
     // gather whose source's new edges the tiles take needs the job's list.
     if (ev) ENG_CK(cudaEventRecord(ev[0], st));
-    if (n_tcjobs) {
-        if (scratch_words_total) ENG_CK(cudaMemsetAsync(scratch.p, 0, scratch_words_total * 8, st));
-        ENG_CK(launch_tc_compact(tcjobs.as<TcJob>(), T, max_tc_w, tc_err.as<int>(), st));
-    }
+    if (n_tcjobs) ENG_CK(launch_tc_compact(tcjobs.as<TcJob>(), T, max_tc_w, tc_err.as<int>(), st));
     if (ev) ENG_CK(cudaEventRecord(ev[1], st));
     ENG_CK(launch_slice(items[kSlice].as<SliceItem>(), max_live[kSlice], slice_groups.as<SliceGroup>(),
-                        slice_mems.as<SliceMem>(), srcs.as<SrcDesc>(), slice_smem, T, kSlice, st));
+                        slice_mems.as<SliceMem>(), srcs.as<SrcDesc>(), slice_smem, T, kSlice, sa));
     for (int c = kExpandNarrow; c <= kExpandWide; ++c)
         ENG_CK(launch_expand(c == kExpandWide, items[c].as<GItem>(), max_live[c], srcs.as<SrcDesc>(), max_expand_w, T, c,
-                             st));
+                             sa));
     for (int c = 0; c < kExpandNarrow; ++c)
         ENG_CK(launch_gather(kVplOf[c / 2], (c & 1) != 0, items[c].as<GItem>(), max_live[c], srcs.as<SrcDesc>(), T, c,
-                             st));
+                             (c & 1) ? st : sb));
     if (ev) ENG_CK(cudaEventRecord(ev[2], st));
     if (n_tcjobs) {
-        ENG_CK(launch_tc_product(false, tcjobs.as<TcJob>(), max_tc_tiles, T, tc_err.as<int>(), st));
+        if (any_uncompacted)
+            ENG_CK(launch_tc_product(false, tcjobs.as<TcJob>(), max_tc_tiles, T, tc_err.as<int>(), st));
         ENG_CK(launch_tc_product_tma(tcjobs.as<TcJob>(), tcmaps.p, max_tc_tiles, T, tc_err.as<int>(), st, tile_kind));
     }
     if (ev) ENG_CK(cudaEventRecord(ev[3], st));
-    // the last extraction launch of the pass also runs the loop control
+    if (branches)
+        for (int i = 0; i < kBranches; ++i)
+            if (side_work[i]) {
+                ENG_CK(cudaEventRecord(join_ev[i], side[i]));
+                ENG_CK(cudaStreamWaitEvent(st, join_ev[i], 0));
+            }
+    // the last extraction launch of the pass also zeroes the tile jobs'
+    // scratch and runs the loop control
     int last_x = -1;
     for (int c = 0; c < kXClasses; ++c)
         if (n_xitems[c]) last_x = c;
@@ -1107,11 +1132,14 @@ int Executor::enqueue_pass(cudaStream_t st, cudaGraphConditionalHandle h, int us
         const bool fuse = c == last_x;
         ENG_CK(launch_extract(kVplOf[c], xitems[c].as<XItem>(), n_xitems[c], fds.as<FDesc>(), T, c,
                               fuse ? ctl_ptrs.as<QCtl *>() : nullptr, (uint32_t)qs.size(), mirror.as<QCtl>(), h,
-                              use_handle, running_out, done_counter.as<unsigned int>(), st));
+                              use_handle, running_out, done_counter.as<unsigned int>(), scratch.as<uint64_t>(),
+                              scratch_words_total, st));
     }
-    if (last_x < 0)
+    if (last_x < 0) {
+        if (scratch_words_total) ENG_CK(cudaMemsetAsync(scratch.p, 0, scratch_words_total * 8, st));
         ENG_CK(launch_control(ctl_ptrs.as<QCtl *>(), (uint32_t)qs.size(), mirror.as<QCtl>(), h, use_handle,
                               running_out, T, 1, st));
+    }
     return CFPQ_OK;
 }
 
@@ -1119,6 +1147,11 @@ int Executor::build_graph(cudaStream_t st, uint32_t max_iter, uint32_t max_round
                           std::string *err) {
     drop_graph();
     if (!cap_stream) ENG_CK(cudaStreamCreateWithFlags(&cap_stream, cudaStreamNonBlocking));
+    if (!fork_ev) ENG_CK(cudaEventCreateWithFlags(&fork_ev, cudaEventDisableTiming));
+    for (int i = 0; i < kBranches; ++i) {
+        if (!side[i]) ENG_CK(cudaStreamCreateWithFlags(&side[i], cudaStreamNonBlocking));
+        if (!join_ev[i]) ENG_CK(cudaEventCreateWithFlags(&join_ev[i], cudaEventDisableTiming));
+    }
     // Everything the graph reads was uploaded on `st`; order the capture after it.
     ENG_CK(cudaStreamSynchronize(st));
     const cudaStream_t cs = cap_stream;
@@ -1152,7 +1185,7 @@ int Executor::build_graph(cudaStream_t st, uint32_t max_iter, uint32_t max_round
     ENG_CK(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     // kPassesPerLoop passes per evaluation of the while node: a pass after the
     // loop finished finds no live work and leaves the control state unchanged
-    for (uint32_t p = 0; p < kPassesPerLoop && rc == 0; ++p) rc = enqueue_pass(cs, handle, 1, nullptr);
+    for (uint32_t p = 0; p < kPassesPerLoop && rc == 0; ++p) rc = enqueue_pass(cs, handle, 1, nullptr, nullptr, true);
     cudaGraph_t body_out = body;
     ce = cudaStreamEndCapture(cs, &body_out);
     if (rc || ce != cudaSuccess) {

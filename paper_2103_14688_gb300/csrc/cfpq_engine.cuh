@@ -32,7 +32,8 @@ cudaError_t launch_slice(const SliceItem *items, uint32_t n_items, const SliceGr
                          const SrcDesc *srcs, uint32_t smem, const ExecTables &T, int cls, cudaStream_t st);
 cudaError_t launch_extract(int vpl, const XItem *items, uint32_t n_items, const FDesc *fds, const ExecTables &T,
                            int cls, QCtl *const *ctls, uint32_t nq, QCtl *mirror, cudaGraphConditionalHandle h,
-                           int use_handle, int *running_out, unsigned int *done_counter, cudaStream_t st);
+                           int use_handle, int *running_out, unsigned int *done_counter, uint64_t *zero,
+                           size_t zero_words, cudaStream_t st);
 cudaError_t launch_control(QCtl *const *ctls, uint32_t nq, QCtl *mirror, cudaGraphConditionalHandle h, int use_handle,
                            int *running_out, const ExecTables &T, int advance, cudaStream_t st);
 cudaError_t launch_tc_product(bool int8, const TcJob *jobs, uint32_t max_tiles, const ExecTables &T, int *err_flag,
@@ -361,10 +362,20 @@ struct Executor {
     cudaGraphExec_t exec = nullptr;
     cudaGraph_t graph = nullptr;
     cudaStream_t cap_stream = nullptr;  // private stream: capture is not allowed on the legacy default stream
+    // Branches of a captured pass (independent kernels of different classes run side by side).
+    static constexpr int kBranches = 2;
+    cudaStream_t side[kBranches] = {nullptr, nullptr};
+    cudaEvent_t fork_ev = nullptr, join_ev[kBranches] = {nullptr, nullptr};
+    bool any_uncompacted = false;  // some tile job's list may exceed its operands' room (k_tc_product)
     bool built = false;
     ~Executor() {
         drop_graph();
         if (cap_stream) cudaStreamDestroy(cap_stream);
+        for (int i = 0; i < kBranches; ++i) {
+            if (side[i]) cudaStreamDestroy(side[i]);
+            if (join_ev[i]) cudaEventDestroy(join_ev[i]);
+        }
+        if (fork_ev) cudaEventDestroy(fork_ev);
     }
     void drop_graph() {
         if (exec) cudaGraphExecDestroy(exec);
@@ -378,8 +389,9 @@ struct Executor {
     // ev (profiling, may be null): four events recorded before the tile
     // operands, after them (before the row gathers), after the gathers and
     // after the tile products.
+    // branches: launch independent kernels on the side streams (graph capture).
     int enqueue_pass(cudaStream_t st, cudaGraphConditionalHandle h, int use_handle, int *running_out,
-                     const cudaEvent_t *ev = nullptr);
+                     const cudaEvent_t *ev = nullptr, bool branches = false);
     int build_graph(cudaStream_t st, uint32_t max_iter, uint32_t max_rounds, uint32_t max_passes, std::string *err);
     int read_ctls(cudaStream_t st, std::vector<QCtl> *out, int *tc_error = nullptr);
 };

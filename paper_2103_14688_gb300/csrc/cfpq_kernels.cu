@@ -1062,6 +1062,8 @@ struct FusedControl {
     uint32_t nq;
     int use_handle;
     int enabled;
+    uint64_t *zero;  // the tile jobs' scratch, zeroed here for the next pass
+    size_t zero_words;
 };
 
 template <int VPL>
@@ -1148,6 +1150,8 @@ __global__ void __launch_bounds__(256) k_extract(const XItem *__restrict__ items
     __syncthreads();
     }
     if (FC.enabled) {
+        for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < FC.zero_words; i += (size_t)gridDim.x * blockDim.x)
+            FC.zero[i] = 0ull;
         __threadfence();
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -1729,9 +1733,11 @@ cudaError_t prepare_gather_launch() {
 // control in its last CTA; done_counter must be 0 before the first launch.
 cudaError_t launch_extract(int vpl, const XItem *items, uint32_t n_items, const FDesc *fds, const ExecTables &T,
                            int cls, QCtl *const *ctls, uint32_t nq, QCtl *mirror, cudaGraphConditionalHandle h,
-                           int use_handle, int *running_out, unsigned int *done_counter, cudaStream_t st) {
+                           int use_handle, int *running_out, unsigned int *done_counter, uint64_t *zero,
+                           size_t zero_words, cudaStream_t st) {
     if (n_items == 0) return cudaSuccess;
-    FusedControl fc{ctls, mirror, running_out, done_counter, h, nq, use_handle, ctls != nullptr ? 1 : 0};
+    FusedControl fc{ctls, mirror, running_out, done_counter, h, nq, use_handle, ctls != nullptr ? 1 : 0, zero,
+                    zero_words};
     // (the CTAs stride over the live items; see launch_gather)
     int dev = 0;
     cudaGetDevice(&dev);

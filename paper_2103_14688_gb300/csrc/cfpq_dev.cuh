@@ -382,4 +382,12 @@ __host__ __device__ inline uint32_t find_owner(const uint32_t *pre, uint32_t nq,
     return lo;
 }
 
+// Index of live item li in its class's list: the owning query's first live item
+// plus the place within it (a single query's list needs no search).
+__device__ __forceinline__ uint32_t live_item(const uint32_t *pre, const uint32_t *beg, uint32_t nq, uint32_t li) {
+    if (nq == 1u) return beg[0] + li;
+    const uint32_t q = find_owner(pre, nq, li);
+    return beg[q] + (li - pre[q]);
+}
+
 }  // namespace cfpq

@@ -812,10 +812,13 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
                 uint32_t n_slices = sliceable ? 4u : 1u;
                 if (q.gather_slices) n_slices = sliceable ? std::min<uint32_t>(q.gather_slices, 16u) : 1u;
                 // nonterminal blocks of wide rows: 128-row items (measured on
-                // Dyck-4; the CSR blocks of the RPQ bench prefer 64)
+                // Dyck-4; the CSR blocks of the RPQ bench prefer 64); rows of
+                // multiple-source runs are few and far between: 1024-row items
                 const uint32_t rows_item =
-                    (has_nt && !expand && q.W >= 256u) ? std::min<uint32_t>(1024u, std::max<uint32_t>(rpi, 128u * item_scale)) : rpi;
-                // the gather keeps an item's row mask in 16 words of shared memory
+                    q.restricted ? 1024u
+                    : (has_nt && !expand && q.W >= 256u) ? std::min<uint32_t>(1024u, std::max<uint32_t>(rpi, 128u * item_scale))
+                                                         : rpi;
+                // the gather lists an item's rows in 1024 entries of shared memory
                 if (rows_item > 1024u || rows_item % 64u != 0u) {
                     *err = "gather items: rows per item must be a multiple of 64 and at most 1024";
                     return CFPQ_ERR_INVALID_ARG;

@@ -216,6 +216,29 @@ __device__ __forceinline__ uint32_t src_channels(const SrcDesc &d, uint32_t mode
     return ch;
 }
 
+// Does row x have an edge of source d that takes part (channels `chans`, not
+// zero)?  Called by one lane per row, 32 rows of a warp side by side: a pass
+// changes few of the rows it could (one in nine on the regular query at n = 30011), and a
+// warp that owns a row finds that out behind four dependent loads.  Loop time, visiting
+// every row -> only these: regular query n = 30011 7.27 -> 3.05 ms, Dyck-4 n = 3001
+// 4.84 -> 4.07, n = 65536 209 -> 186, 16 sources at n = 65536 5.0 -> 2.8.
+template <bool NT>
+__device__ __forceinline__ bool row_has_work(const SrcDesc &d, uint32_t chans, uint32_t x, uint32_t iter, uint32_t g,
+                                             uint32_t g0) {
+    if (d.csr_off) {
+        const uint32_t e1 = d.csr_off[x + 1];
+        uint32_t e = d.csr_off[x];
+        if (e >= e1) return false;
+        if (chans & 1u) return true;
+        const uint32_t thr = (chans & 2u) ? g0 : g - 1u;
+        for (; e < e1; ++e)
+            if (d.rstamp[d.csr_col[e]] >= thr) return true;
+        return false;
+    }
+    if (!NT) return false;
+    return (chans & 6u) ? d.nt_new_it[x] != 0u : d.nt_new_it[x] == iter;  // (0: the row has no edge)
+}
+
 // --------------------------------------------------------------------------
 // Closure pass (bit-packed rows).  One CTA of 8 warps per work item; a row is
 // handled by a group of `lpr` lanes, each lane holding VPL 128-bit vectors
@@ -227,6 +250,12 @@ __device__ __forceinline__ uint32_t src_channels(const SrcDesc &d, uint32_t mode
 template <int VPL>
 struct GatherOcc {
     static constexpr int value = VPL <= 2 ? 4 : (VPL == 4 ? 2 : 1);
+};
+// CSR variant of wide rows: one source row in registers beside the output row
+// leaves room for two CTAs (it was one CTA with two source rows in flight).
+template <int VPL, bool NT>
+struct GatherCtas {
+    static constexpr int value = !NT && VPL >= 8 ? 2 : GatherOcc<VPL>::value;
 };
 
 // Scheduling.  Narrow rows: one CTA per live item (the grid covers every
@@ -250,14 +279,14 @@ constexpr uint32_t kGatherParts = 8;
 constexpr uint32_t kStrideWaves = 8;  // launch_gather / launch_extract: waves of resident CTAs at most
 
 template <int VPL, bool NT>
-__global__ void __launch_bounds__(256, GatherOcc<VPL>::value)
+__global__ void __launch_bounds__(256, GatherCtas<VPL, NT>::value)
     k_gather(const GItem *__restrict__ items, const SrcDesc *__restrict__ srcs, ExecTables T, int cls) {
     constexpr bool kDyn = GatherDyn<VPL, NT>::on;
     __shared__ unsigned long long s_changed, s_ors;
-    // rows of the item to compute (multiple-source runs; else all): the item's
-    // rows start at a multiple of 64 and number at most 1024, so its 16 mask
-    // words have distinct indices modulo 16
-    __shared__ unsigned long long s_rmask[16];
+    // rows of the item with work: their bits, then the list (an item has at
+    // most 1024 rows and starts at a multiple of 64)
+    __shared__ uint32_t s_rowbits[32];
+    __shared__ uint16_t s_rows[1024];
     // general variant: per-warp ring of source rows loaded with cp.async
     extern __shared__ uint4 s_ring[];
     constexpr int P = GatherRing<VPL>::depth;
@@ -289,16 +318,17 @@ __global__ void __launch_bounds__(256, GatherOcc<VPL>::value)
             act |= src_channels<NT>(srcs[it.src0 + k], mode, iter, g, g0, dmask) != 0u;
         if (!__any_sync(FULLMASK, act)) continue;
     } else {
+        if (it.rmask) {  // multiple-source runs: no row of the item is reached
+            const uint32_t w = (it.row0 >> 6) + threadIdx.x;
+            if (!__syncthreads_or(w * 64u < it.row1 && it.rmask[w] != 0ull)) continue;
+        }
         int act = 0;
         for (uint32_t k = threadIdx.x; k < it.nsrc; k += blockDim.x)
             act |= src_channels<NT>(srcs[it.src0 + k], mode, iter, g, g0, dmask) != 0u;
         if (!__syncthreads_or(act)) continue;
 
         if (threadIdx.x == 0) { s_changed = 0; s_ors = 0; }
-        if (threadIdx.x < 16u) {
-            const uint32_t wrow = it.row0 + threadIdx.x * 64u;
-            s_rmask[(wrow >> 6) & 15u] = (it.rmask && wrow < it.row1) ? it.rmask[wrow >> 6] : ~0ull;
-        }
+        if (threadIdx.x < 32u) s_rowbits[threadIdx.x] = 0u;
         __syncthreads();
     }
 
@@ -332,80 +362,80 @@ __global__ void __launch_bounds__(256, GatherOcc<VPL>::value)
     // channels of the item's first 16 sources in this pass (4 bits each): the
     // same for every row of the unit
     unsigned long long chpack = 0ull;
-    if constexpr (NT)
-        for (uint32_t k = 0; k < it.nsrc && k < 16u; ++k)
-            chpack |= (unsigned long long)src_channels<NT>(srcs[it.src0 + k], mode, iter, g, g0, dmask) << (4u * k);
+    for (uint32_t k = 0; k < it.nsrc && k < 16u; ++k)
+        chpack |= (unsigned long long)src_channels<NT>(srcs[it.src0 + k], mode, iter, g, g0, dmask) << (4u * k);
+    auto chans_of = [&](uint32_t k) -> uint32_t {
+        return k < 16u ? (uint32_t)(chpack >> (4u * k)) & 15u
+                       : src_channels<NT>(srcs[it.src0 + k], mode, iter, g, g0, dmask);
+    };
+    auto wanted = [&](uint32_t r) { return !it.rmask || ((it.rmask[r >> 6] >> (r & 63u)) & 1ull) != 0ull; };
 
-    // rows of this warp: the unit's range of rpw-row steps (dynamic), or
-    // every eighth step of the item (one CTA per item)
-    uint32_t r_first = it.row0 + (uint32_t)(warp * rpw), r_end = it.row1, r_step = 8u * rpw;
+    // Rows with work, found a lane a row.  Dynamic units: the warp tests its
+    // range of rows 32 at a time and takes them in turn.  One CTA per item: up to
+    // four threads a row share its sources, and the rows found are listed for the
+    // groups of all warps.
+    uint32_t r_next = 0u, r_end = 0u, nrows = 0u;
+    unsigned r_mask = 0u;  // rows of the window [r_next - 32, r_next) still to take
     if constexpr (kDyn) {
-        const uint32_t steps = (it.row1 - it.row0 + (uint32_t)rpw - 1u) / (uint32_t)rpw;
-        const uint32_t per = (steps + kGatherParts - 1u) / kGatherParts;
-        r_first = it.row0 + part * per * (uint32_t)rpw;
-        r_end = min(it.row1, r_first + per * (uint32_t)rpw);
-        r_step = (uint32_t)rpw;
-    }
-    // Rows with nothing to do: when every source taking part in the pass
-    // reads only the iteration's new edges of a nonterminal (channel 1; the
-    // late passes of Dyck-4's x_i and p levels), a row has work only if one
-    // of those boxes has a new edge in it (its A2 stamp is this iteration),
-    // so a warp that owns whole rows (dynamic units) jumps from one such row
-    // to the next, 32 stamps per coalesced load, instead of visiting every
-    // row and source.
-    const uint32_t *skip_it[2] = {nullptr, nullptr};
-    bool skip_rows = false;
-    if constexpr (kDyn) {
-        skip_rows = it.nsrc <= 16u;
-        uint32_t ns = 0;
-        for (uint32_t k = 0; k < it.nsrc && skip_rows; ++k) {
-            const uint32_t chans = (uint32_t)(chpack >> (4u * k)) & 15u;
-            if (!chans) continue;
-            const SrcDesc &d = srcs[it.src0 + k];
-            if ((chans & ~9u) != 0u || d.csr_off != nullptr || d.nt_new_it == nullptr) {
-                skip_rows = false;
-                break;
-            }
-            if (ns < 2u && (ns == 0u || skip_it[0] != d.nt_new_it)) skip_it[ns++] = d.nt_new_it;
-            else if (skip_it[0] != d.nt_new_it && skip_it[1] != d.nt_new_it) skip_rows = false;
-        }
-        skip_rows = skip_rows && ns > 0u && lpr == 32;
-    }
-    for (uint32_t rbase = r_first; rbase < r_end; rbase += r_step) {
-        if constexpr (kDyn) {
-            if (skip_rows) {
-                // the next row at or after rbase with a new edge in one of the boxes
-                bool found = false;
-                while (rbase < r_end) {
-                    const uint32_t b32 = rbase & ~31u, r = b32 + (uint32_t)lane;
-                    const bool w = r >= rbase && r < r_end &&
-                                   (skip_it[0][r] == iter || (skip_it[1] != nullptr && skip_it[1][r] == iter));
-                    const unsigned m = __ballot_sync(FULLMASK, w);
-                    if (m) {
-                        rbase = b32 + (uint32_t)(__ffs(m) - 1);
-                        found = true;
-                        break;
-                    }
-                    rbase = b32 + 32u;
+        const uint32_t per = (it.row1 - it.row0 + kGatherParts - 1u) / kGatherParts;
+        r_next = it.row0 + part * per;
+        r_end = min(it.row1, r_next + per);
+    } else {
+        const uint32_t nr = it.row1 - it.row0;
+        const uint32_t step = nr > 128u ? 256u : nr > 64u ? 128u : 64u, parts = 256u / step;
+        for (uint32_t r0 = 0; r0 < nr; r0 += step) {
+            const uint32_t r = r0 + threadIdx.x % step;
+            bool has = false;
+            if (r < nr && wanted(it.row0 + r))
+                for (uint32_t k = threadIdx.x / step; k < it.nsrc && !has; k += parts) {
+                    const uint32_t chans = chans_of(k);
+                    has = chans != 0u && row_has_work<NT>(srcs[it.src0 + k], chans, it.row0 + r, iter, g, g0);
                 }
-                if (!found) break;
-            }
+            const unsigned bal = __ballot_sync(FULLMASK, has);
+            if (lane == 0 && bal) atomicOr(&s_rowbits[r >> 5], bal);
         }
-        const uint32_t row = rbase + grp;
-        bool valid = row < r_end;
-        if constexpr (kDyn) valid = valid && (!it.rmask || ((it.rmask[row >> 6] >> (row & 63u)) & 1ull));
-        else valid = valid && ((s_rmask[(row >> 6) & 15u] >> (row & 63u)) & 1ull);
+        __syncthreads();
+        const uint32_t nw = (nr + 31u) >> 5;
+        for (uint32_t r = threadIdx.x; r < nr; r += 256u) {
+            const uint32_t bits = s_rowbits[r >> 5];
+            if (!((bits >> (r & 31u)) & 1u)) continue;
+            uint32_t pos = (uint32_t)__popc(bits & ((1u << (r & 31u)) - 1u));
+            for (uint32_t w = 0; w < (r >> 5); ++w) pos += (uint32_t)__popc(s_rowbits[w]);
+            s_rows[pos] = (uint16_t)r;
+        }
+        for (uint32_t w = 0; w < nw; ++w) nrows += (uint32_t)__popc(s_rowbits[w]);
+        __syncthreads();
+    }
+    for (uint32_t i0 = (uint32_t)(warp * rpw);; i0 += 8u * rpw) {
+        uint32_t row;
+        bool valid;
+        if constexpr (kDyn) {
+            while (!r_mask && r_next < r_end) {
+                const uint32_t r = r_next + (uint32_t)lane;
+                bool has = false;
+                if (r < r_end && wanted(r))
+                    for (uint32_t k = 0; k < it.nsrc && !has; ++k) {
+                        const uint32_t chans = chans_of(k);
+                        has = chans != 0u && row_has_work<NT>(srcs[it.src0 + k], chans, r, iter, g, g0);
+                    }
+                r_mask = __ballot_sync(FULLMASK, has);
+                r_next += 32u;
+            }
+            if (!r_mask) break;
+            row = r_next - 32u + (uint32_t)(__ffs(r_mask) - 1);
+            r_mask &= r_mask - 1u;
+            valid = true;
+        } else {
+            if (i0 >= nrows) break;
+            valid = i0 + (uint32_t)grp < nrows;
+            row = it.row0 + (valid ? s_rows[i0 + (uint32_t)grp] : 0u);
+        }
         uint4 acc[VPL];
 #pragma unroll
         for (int j = 0; j < VPL; ++j) acc[j] = make_uint4(0, 0, 0, 0);
 
         for (uint32_t k = 0; k < it.nsrc; ++k) {
-            uint32_t chans;
-            if constexpr (NT)
-                chans = k < 16u ? (uint32_t)(chpack >> (4u * k)) & 15u
-                                : src_channels<NT>(srcs[it.src0 + k], mode, iter, g, g0, dmask);
-            else
-                chans = src_channels<NT>(srcs[it.src0 + k], mode, iter, g, g0, dmask);
+            const uint32_t chans = chans_of(k);
             if (!chans) continue;  // the source takes no part in this pass
             const SrcDesc d = srcs[it.src0 + k];
             for (uint32_t cbit = 1u; cbit <= 4u; cbit <<= 1) {
@@ -512,7 +542,22 @@ __global__ void __launch_bounds__(256, GatherOcc<VPL>::value)
                                 }
                             }
                         }
-                        if (rblk && (!NT || !d.pure_n)) {
+                        if constexpr (!NT && VPL > 8) {
+                            if (rblk && hs[0]) {
+                                const uint4 *r = reinterpret_cast<const uint4 *>(rblk + (size_t)ys[0] * W);
+#pragma unroll
+                                for (int j0 = 0; j0 < VPL; j0 += 8) {
+                                    uint4 a[8];
+#pragma unroll
+                                    for (int j = 0; j < 8; ++j)
+                                        a[j] = ((winmask >> (j0 + j)) & 1u) ? r[(uint32_t)gl + (uint32_t)(j0 + j) * lpr]
+                                                                            : make_uint4(0, 0, 0, 0);
+#pragma unroll
+                                    for (int j = 0; j < 8; ++j) or4(acc[j0 + j], a[j]);
+                                }
+                                if (gl == 0) ++my_ors;
+                            }
+                        } else if (rblk && (!NT || !d.pure_n)) {
                             uint4 rv[U][VPL];
 #pragma unroll
                             for (int u = 0; u < U; ++u) {
@@ -551,6 +596,27 @@ __global__ void __launch_bounds__(256, GatherOcc<VPL>::value)
                                     if (jj == j) setbit4(acc[jj], y & 127u);
                             }
                         };
+                        if constexpr (!NT && VPL >= 8) {
+                            // (a warp owns the row: e0, e1 and the stamps are the same in every lane)
+                            for (uint32_t e = e0; e < e1; ++e) {
+                                const uint32_t y = d.csr_col[e];
+                                if (use_ident) ident_bit(y);
+                                if (!rblk || (thr && d.rstamp[y] < thr)) continue;
+                                const uint4 *r = reinterpret_cast<const uint4 *>(rblk + (size_t)y * W);
+                                // eight vectors in flight (sixteen would spill at two CTAs)
+#pragma unroll
+                                for (int j0 = 0; j0 < VPL; j0 += 8) {
+                                    uint4 a[8];
+#pragma unroll
+                                    for (int j = 0; j < 8; ++j)
+                                        a[j] = ((winmask >> (j0 + j)) & 1u) ? r[(uint32_t)gl + (uint32_t)(j0 + j) * lpr]
+                                                                            : make_uint4(0, 0, 0, 0);
+#pragma unroll
+                                    for (int j = 0; j < 8; ++j) or4(acc[j0 + j], a[j]);
+                                }
+                                if (gl == 0) ++my_ors;
+                            }
+                        } else
                         for (uint32_t e = e0; e < e1; e += 2) {
                             const bool two = e + 1 < e1;
                             const uint32_t y0 = d.csr_col[e], y1 = two ? d.csr_col[e + 1] : 0u;
@@ -1703,9 +1769,9 @@ cudaError_t launch_gather(int vpl, bool nt, const GItem *items, uint32_t n_items
         return std::max<uint32_t>(1u, std::min<uint32_t>(want, sms * (uint32_t)occ));
     };
 #define CFPQ_GATHER(V)                                                                                          \
-    if (nt) k_gather<V, true><<<grid_of(GatherDyn<V, true>::on, GatherOcc<V>::value), 256, GatherRing<V>::bytes, \
+    if (nt) k_gather<V, true><<<grid_of(GatherDyn<V, true>::on, GatherCtas<V, true>::value), 256, GatherRing<V>::bytes, \
                                 st>>>(items, srcs, T, cls);                                                     \
-    else k_gather<V, false><<<grid_of(false, GatherOcc<V>::value), 256, 0, st>>>(items, srcs, T, cls);
+    else k_gather<V, false><<<grid_of(false, GatherCtas<V, false>::value), 256, 0, st>>>(items, srcs, T, cls);
     switch (vpl) {
         case 1: CFPQ_GATHER(1) break;
         case 2: CFPQ_GATHER(2) break;

@@ -251,7 +251,9 @@ struct TcJob {
     unsigned long long *mrows;
     // Channel-1 job (covers_new): the iteration's new edges A2 (A = A2 rows,
     // a_it = their iteration marks) times whole rows of B; K = the columns y
-    // of some new edge (newcols, W words) whose row of B was ever written.
+    // of some new edge (newcols, W words) whose row of B was written before
+    // this iteration and not in it: the rows changed in this iteration are read
+    // by channel 2, over all edges, the new ones among them.
     // *mcount = rows with a new edge, *ecount = the number of new edges;
     // newcols and the counts are zero before every pass.  The job runs only
     // when new_tiles_pay says the tiles beat the row gather on those counts;
@@ -269,7 +271,8 @@ struct TcJob {
 // PFLOP/s, the tiles win when M * K < e * 2.5e15 / (16 * 3.5e12), i.e.
 // about 44 * e; n cancels.  The ratio scales with the tile format's rate
 // (kTileEdgeRatio for FP8, kTileEdgeRatioFp4 for FP4).  listed_k = K for
-// this pass (0 if the list was not built), kcap = the job's room for it.
+// this pass, kcap = the job's room for it.  With new edges (m > 0) and no row
+// listed there is nothing to OR, which tiles do for free.
 constexpr unsigned long long kTileEdgeRatio = 44;
 constexpr unsigned long long kTileEdgeRatioFp4 = 88;
 
@@ -282,7 +285,8 @@ constexpr uint32_t kTileFp8Pair = 0, kTileFp8Single = 1, kTileFp4Pair = 2, kTile
 __host__ __device__ constexpr bool tile_kind_fp4(uint32_t k) { return k == kTileFp4Pair || k == kTileFp4NvPair; }
 __host__ __device__ inline bool new_tiles_pay(uint32_t listed_k, uint32_t kcap, unsigned long long m,
                                               unsigned long long e, unsigned long long ratio) {
-    if (listed_k == 0 || listed_k > kcap || m == 0) return false;
+    if (listed_k > kcap || m == 0) return false;
+    if (listed_k == 0) return true;
     const unsigned long long pm = (m + 127ull) & ~127ull, pk = ((unsigned long long)listed_k + 127ull) & ~127ull;
     return pm * pk < ratio * e;
 }

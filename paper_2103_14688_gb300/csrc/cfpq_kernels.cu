@@ -446,8 +446,12 @@ __global__ void __launch_bounds__(256, GatherCtas<VPL, NT>::value)
                 const uint64_t *const rblk = (NT && new_edges && (chans & 8u)) ? nullptr : d.rblk;
                 const bool use_ident = new_edges && d.ident;
                 if (!use_ident && rblk == nullptr) continue;
-                // a source row takes part when its stamp is >= thr
+                // a source row takes part when its stamp is >= thr; new edges
+                // take whole rows: those ever written and, where channel 2
+                // reads the rows changed in this iteration over all edges,
+                // not those (nt_lo <= stamp < nt_hi, nonterminal sources)
                 const uint32_t thr = new_edges ? 0u : (cbit == 2u ? g0 : g - 1u);
+                const uint32_t nt_lo = new_edges ? 1u : thr, nt_hi = (new_edges && !d.same_level) ? g0 : 0xFFFFFFFFu;
 
                 // Every lane proposes one candidate edge (x, y) of its group's
                 // row (y_l, has_l).  The group keeps those whose source row is
@@ -455,8 +459,17 @@ __global__ void __launch_bounds__(256, GatherCtas<VPL, NT>::value)
                 // before any is combined, so several 128-bit loads per lane are
                 // in flight.
                 constexpr int U = VPL >= 4 ? 1 : 4 / VPL;
+                const bool bitrow = NT && d.csr_off == nullptr;
                 auto take_batch = [&](uint32_t y_l, bool has_l) {
-                    const bool keep = has_l && (rblk == nullptr || thr == 0u || d.rstamp[y_l] >= thr);
+                    bool keep = has_l;
+                    if (has_l && rblk != nullptr) {
+                        if (bitrow) {
+                            const uint32_t sy = d.rstamp[y_l];
+                            keep = sy >= nt_lo && sy < nt_hi;
+                        } else {
+                            keep = thr == 0u || d.rstamp[y_l] >= thr;
+                        }
+                    }
                     if constexpr (NT) {
                         if (d.pure_n && !use_ident) {
                             if (lpr == 32) {  // one row per warp: the bitmap in the warp's first slot

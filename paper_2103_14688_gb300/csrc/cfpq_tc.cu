@@ -643,10 +643,13 @@ __global__ void __launch_bounds__(256) k_tc_newcols(const TcJob *__restrict__ jo
     });
 }
 
-// List the rows y of B with stamp >= thr; for a channel-1 job the columns
-// of its newcols whose row of B was ever written (stamp != 0: on Dyck-4 two
-// thirds of the vertices start no path, so their rows are empty).  The order
-// is irrelevant (the product sums over them).  kmask = the listed rows.
+// List the rows y of B with stamp >= thr; for a channel-1 job the columns of
+// its newcols whose row of B was ever written (stamp != 0: on Dyck-4 two
+// thirds of the vertices start no path, so their rows are empty) and did not
+// change in this iteration (channel 2 reads those over all edges: while Dyck-4's
+// answer grows, nearly every row changes in every iteration, and the new edges' product
+// repeated the all-edges one).  The order is irrelevant (the product sums over
+// them).  kmask = the listed rows.
 __global__ void __launch_bounds__(256) k_tc_rows(const TcJob *__restrict__ jobs, ExecTables T, int *err_flag) {
     // a unit's listed rows are counted over the CTA first, so that the unit
     // reserves its part of the list with one atomic (one per warp step kept
@@ -659,12 +662,14 @@ __global__ void __launch_bounds__(256) k_tc_rows(const TcJob *__restrict__ jobs,
         uint32_t thr, iter, g;
         if (!tc_job_active(J, &thr, &iter, &g) || !J.b_stamp) return;
         const uint32_t y_beg = c * kRowChunk, y_end = min(J.n, y_beg + kRowChunk);
+        // (a channel-1 job reads a lower level: its rows' stamps are final)
+        const uint32_t g0 = J.ctl->g_iter_start;
         uint32_t mask = 0u;
 #pragma unroll
         for (uint32_t i = 0; i < kPer; ++i) {
             const uint32_t y = y_beg + threadIdx.x + 256u * i;
             const bool dirty = y < y_end && (J.covers_new ? ((J.newcols[y >> 6] >> (y & 63u)) & 1ull) != 0ull &&
-                                                                J.b_stamp[y] != 0u
+                                                                J.b_stamp[y] - 1u < g0 - 1u  // 0 < stamp < g0
                                                           : J.b_stamp[y] >= thr);
             if (dirty) mask |= 1u << i;
             const unsigned bal = __ballot_sync(0xffffffffu, dirty);

@@ -810,22 +810,36 @@ __global__ void __launch_bounds__(256, GatherCtas<VPL, NT>::value)
 // gather of Dyck-4 at n = 65536; the query went from 303 to 233 ms.
 // --------------------------------------------------------------------------
 constexpr int kExpandOcc = 6;  // CTAs per SM (40 registers a thread; 32 would spill)
+constexpr uint32_t kExpandParts = 4;
 template <bool WIDE>
 __global__ void __launch_bounds__(256, kExpandOcc)
     k_expand(const GItem *__restrict__ items, const SrcDesc *__restrict__ srcs, ExecTables T, int cls) {
     extern __shared__ unsigned long long s_bitmap[];  // WIDE: one row; else one row per warp
     __shared__ uint16_t s_rows[1024];                 // (an item has at most 1024 rows)
-    __shared__ uint32_t s_nrows, s_take, s_changed;
+    __shared__ uint32_t s_nrows, s_take, s_changed, s_unit;
+    __shared__ uint16_t s_list[8][1024];              // per warp: columns (below 65536) to expand
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    uint16_t *const list = s_list[warp];
     const uint32_t t0 = WIDE ? tid : lane;            // this thread's place in its row's group
     constexpr uint32_t TPR = WIDE ? 256u : 32u;
-    const uint32_t total = T.g_total[cls];
-    for (uint32_t li = blockIdx.x; li < total; li += gridDim.x) {
+    // units: a wide item's rows in kExpandParts ranges, narrow items whole; the
+    // first one by block index, the others from the pass's counter (a few units
+    // hold most of a pass's work)
+    constexpr uint32_t kParts = WIDE ? kExpandParts : 1u;
+    const uint32_t total = T.g_total[cls] * kParts;
+    for (uint32_t u = blockIdx.x; u < total;) {
+        const uint32_t li = u / kParts, part = u % kParts;
+        __syncthreads();  // (s_unit of the last round has been read)
+        if (tid == 0) s_unit = gridDim.x + atomicAdd(T.g_next + cls, 1u);
+        __syncthreads();
+        u = s_unit;
         const GItem &it = items[live_item(T.g_pre[cls], T.g_beg[cls], T.nq, li)];
         QCtl *const c = it.ctl;
         if (c->phase != kPhaseRun || c->level != it.level) continue;  // (uniform)
         const uint32_t g = c->g, iter = c->iter, mode = c->mode, g0 = c->g_iter_start, W = it.W;
-        const uint32_t src0 = it.src0, nsrc = it.nsrc, row0 = it.row0, row1 = it.row1;
+        const uint32_t src0 = it.src0, nsrc = it.nsrc;
+        const uint32_t per = (it.row1 - it.row0 + kParts - 1u) / kParts;
+        const uint32_t row0 = it.row0 + part * per, row1 = min(it.row1, row0 + per);
         int act = 0;
         for (uint32_t k = tid; k < nsrc; k += 256u) act |= src_channels<true>(srcs[src0 + k], mode, iter, g, g0, 0u) != 0u;
         if (!__syncthreads_or(act)) continue;
@@ -892,14 +906,31 @@ __global__ void __launch_bounds__(256, kExpandOcc)
                         continue;
                     }
                     const uint32_t thr = new_edges ? 0u : (cb == 2u ? g0 : g - 1u);
+                    // 1024 columns a warp and step: the set bits' columns are
+                    // listed in order, then expanded a lane each, so that the
+                    // lanes' CSR loads fall into a few neighbouring lines
+                    // (each lane on its own word: 32 lines a load)
                     const uint32_t pn = d.pure_n;
-                    for (uint32_t w = t0; w < W; w += TPR) {
-                        unsigned long long v = adj[w];
-                        if (!v) continue;
-                        v &= pn > 1u ? d.pure_mask[0][w] | d.pure_mask[1][w] : d.pure_mask[0][w];
-                        while (v) {
-                            const uint32_t y = w * 64u + (uint32_t)__ffsll((long long)v) - 1u;
-                            v &= v - 1ull;
+                    const uint32_t *const a32 = reinterpret_cast<const uint32_t *>(adj);
+                    const uint32_t *const m0 = reinterpret_cast<const uint32_t *>(d.pure_mask[0]);
+                    const uint32_t *const m1 = reinterpret_cast<const uint32_t *>(d.pure_mask[1]);
+                    for (uint32_t b0 = (WIDE ? warp : 0u) * 32u; b0 < 2u * W; b0 += WIDE ? 256u : 32u) {
+                        const uint32_t wi = b0 + lane;
+                        uint32_t v = wi < 2u * W ? a32[wi] : 0u;
+                        if (v) v &= pn > 1u ? m0[wi] | m1[wi] : m0[wi];
+                        const uint32_t cnt = (uint32_t)__popc(v);
+                        uint32_t incl = cnt;
+#pragma unroll
+                        for (int o2 = 1; o2 < 32; o2 <<= 1) {
+                            const uint32_t u = __shfl_up_sync(FULLMASK, incl, o2);
+                            if (lane >= (uint32_t)o2) incl += u;
+                        }
+                        const uint32_t n_set = __shfl_sync(FULLMASK, incl, 31);
+                        if (n_set == 0u) continue;
+                        for (uint32_t at = incl - cnt; v; v &= v - 1u) list[at++] = (uint16_t)(wi * 32u + (uint32_t)__ffs(v) - 1u);
+                        __syncwarp();
+                        for (uint32_t j = lane; j < n_set; j += 32u) {
+                            const uint32_t y = list[j];
                             if (thr && d.rstamp[y] < thr) continue;
                             for (uint32_t p = 0; p < pn; ++p) {
                                 const uint32_t e1 = d.pure_off[p][y + 1];
@@ -909,6 +940,7 @@ __global__ void __launch_bounds__(256, kExpandOcc)
                                 }
                             }
                         }
+                        __syncwarp();  // the list is reused
                     }
                 }
             }
@@ -1803,7 +1835,8 @@ cudaError_t launch_expand(bool wide, const GItem *items, uint32_t n_items, const
     int dev = 0;
     cudaGetDevice(&dev);
     const uint32_t sms = (dev >= 0 && dev < 64 && g_gather_sms[dev]) ? (uint32_t)g_gather_sms[dev] : 0u;
-    const uint32_t grid = sms ? std::min<uint32_t>(n_items, sms * (uint32_t)kExpandOcc) : n_items;  // resident CTAs stride over the items
+    const uint32_t units = n_items * (wide ? kExpandParts : 1u);
+    const uint32_t grid = sms ? std::min<uint32_t>(units, sms * (uint32_t)kExpandOcc) : units;  // resident CTAs take units
     if (wide) k_expand<true><<<grid, 256, (size_t)max_w * 8, st>>>(items, srcs, T, cls);
     else k_expand<false><<<grid, 256, (size_t)std::min(max_w, kExpandNarrowW) * 8 * 8, st>>>(items, srcs, T, cls);
     return cudaGetLastError();

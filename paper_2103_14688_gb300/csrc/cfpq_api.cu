@@ -158,6 +158,7 @@ int run_executor(cfpq_ctx *ctx, Executor &ex, std::vector<QCtl> *ctls, uint32_t 
             if (ex.build_graph(st, mi, mr, mp, &e)) return fail(ctx, CFPQ_ERR_CUDA, e);
         }
         CK(ctx, cudaGraphLaunch(ex.exec, st));
+        for (QueryDev *q : ex.qs) q->all_dirty_set = false;
     }
     int tc_error = 0;
     if (ex.read_ctls(st, ctls, &tc_error)) return fail(ctx, CFPQ_ERR_CUDA, "reading loop state failed");
@@ -373,7 +374,10 @@ int cfpq_run(cfpq_ctx *ctx, cfpq_run_stats *stats) {
     ClosureProfile prof;
     if (ctx->query.small_ok && ctx->opt.loop_mode == CFPQ_LOOP_DEVICE) {
         // the whole fixpoint in one CTA (state in shared memory)
-        const QueryDev &q = ctx->query;
+        QueryDev &q = ctx->query;
+        // (it writes blocks and M2 without their marks)
+        std::string e;
+        if (int rc = q.mark_all_dirty(ctx->stream, &e)) return fail(ctx, rc, e);
         CK(ctx, launch_small_fixpoint(q.small_desc.p, q.W, q.small_smem, q.small_meta,
                                       (uint64_t)ctx->graph.n_term * ctx->graph.n, ctx->graph.m_unique, q.small_items,
                                       ctx->stream));

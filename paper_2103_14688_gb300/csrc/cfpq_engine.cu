@@ -526,7 +526,7 @@ int QueryDev::prepare(Allocator *A, std::string *err) {
         !last_mem.ensure(A, std::max<size_t>(nblk, 1) * 4, err) || !m2_mem.ensure(A, (size_t)B * bw, err) ||
         !a2_mem.ensure(A, (size_t)B * bw, err) || !a2it_mem.ensure(A, (size_t)B * n * 4, err) ||
         !boxit_mem.ensure(A, (size_t)B * 4, err) || !ctl_mem.ensure(A, sizeof(QCtl), err) ||
-        !boxedge_mem.ensure(A, (size_t)B * 8, err) ||
+        !boxedge_mem.ensure(A, (size_t)B * 8, err) || !all_dirty.ensure(A, 16, err) ||
         !ctl_ptr_mem.ensure(A, sizeof(QCtl *), err) ||
         !eps_mem.ensure(A, std::max<size_t>(n_eps, 1) * eps_desc_size(), err) ||
         !tc_mem.ensure(A, std::max<size_t>(n_tc_src * tc_slot_bytes(), 64), err))
@@ -543,11 +543,21 @@ int QueryDev::prepare(Allocator *A, std::string *err) {
         ++k;
     }
     QCtl *cp = ctl();
+    // (fresh buffers, or another plan's rows at these addresses)
+    all_dirty_set = false;
+    if ((rc = mark_all_dirty(A->stream, err))) return rc;
     ENG_CK(cudaMemcpyAsync(eps_mem.p, he.data(), he.size(), cudaMemcpyHostToDevice, A->stream));
     ENG_CK(cudaMemcpyAsync(ctl_ptr_mem.p, &cp, sizeof(cp), cudaMemcpyHostToDevice, A->stream));
     ENG_CK(cudaStreamSynchronize(A->stream));
     prepared = true;
     graph_generation = g->generation;
+    return CFPQ_OK;
+}
+
+int QueryDev::mark_all_dirty(cudaStream_t st, std::string *err) {
+    if (all_dirty_set) return CFPQ_OK;
+    ENG_CK(cudaMemsetAsync(all_dirty.p, 0xFF, 4, st));
+    all_dirty_set = true;
     return CFPQ_OK;
 }
 
@@ -597,13 +607,13 @@ int QueryDev::prepare_small(Allocator *A, cudaStream_t st, uint32_t max_iter, ui
 int QueryDev::enqueue_init(cudaStream_t st, uint32_t max_iter, uint32_t max_rounds, uint32_t max_passes) {
     std::string *err = nullptr;
     const size_t nblk = blocks.size();
-    if (nblk) {
-        ENG_CK(cudaMemsetAsync(blk_mem.p, 0, nblk * (size_t)n * W * 8, st));
-        ENG_CK(cudaMemsetAsync(stamp_mem.p, 0, nblk * (size_t)n * 4, st));
-        ENG_CK(cudaMemsetAsync(last_mem.p, 0, nblk * 4, st));
-    }
-    ENG_CK(cudaMemsetAsync(m2_mem.p, 0, (size_t)B * n * W * 8, st));
-    ENG_CK(cudaMemsetAsync(a2it_mem.p, 0, (size_t)B * n * 4, st));
+    if (nblk) ENG_CK(cudaMemsetAsync(last_mem.p, 0, nblk * 4, st));
+    ENG_CK(launch_clear_rows(blk_mem.as<uint64_t>(), stamp_mem.as<uint32_t>(), nblk * (size_t)n, W,
+                             all_dirty.as<uint32_t>(), st));
+    ENG_CK(launch_clear_rows(m2_mem.as<uint64_t>(), a2it_mem.as<uint32_t>(), (size_t)B * n, W, all_dirty.as<uint32_t>(),
+                             st));
+    ENG_CK(cudaMemsetAsync(all_dirty.p, 0, 4, st));
+    all_dirty_set = false;  // (also when captured: a launch of the graph clears the word)
     ENG_CK(cudaMemsetAsync(boxit_mem.p, 0, (size_t)B * 4, st));
     ENG_CK(cudaMemsetAsync(boxedge_mem.p, 0, (size_t)B * 8, st));
     for (uint32_t k = 0; k < n_tc_src; ++k) ENG_CK(cudaMemsetAsync(tc_kcount(k), 0, 8, st));
@@ -611,7 +621,7 @@ int QueryDev::enqueue_init(cudaStream_t st, uint32_t max_iter, uint32_t max_roun
     // the column slices of the row gather in every mode
     ENG_CK(launch_ctl_reset(ctl_ptr_mem.as<QCtl *>(), 1, max_iter, max_rounds, max_passes, n_levels, loop_mask,
                             boxedge_mem.as<unsigned long long>(), B, n, boxit_mem.as<uint32_t>(), nt_read_mask, st));
-    ENG_CK(launch_eps_init(eps_mem.p, n_eps, 152, st));
+    ENG_CK(launch_eps_init(eps_mem.p, n_eps, n, st));
     if (seeded)
         ENG_CK(launch_seed_apply(seed_mem.as<uint64_t>(), m2_mem.as<uint64_t>(), a2_mem.as<uint64_t>(),
                                  a2it_mem.as<uint32_t>(), boxit_mem.as<uint32_t>(), ctl(),

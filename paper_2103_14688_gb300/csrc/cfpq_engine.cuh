@@ -60,7 +60,9 @@ cudaError_t launch_ctl_reset(QCtl *const *ctls, uint32_t nq, uint32_t max_iter, 
                              uint32_t max_passes, uint32_t n_levels, unsigned long long cyclic_mask,
                              unsigned long long *box_edges, uint32_t n_boxes, uint32_t n,
                              const uint32_t *box_new_it, unsigned long long nt_read_mask, cudaStream_t st);
-cudaError_t launch_eps_init(const void *eds, uint32_t ned, uint32_t grid, cudaStream_t st);
+cudaError_t launch_eps_init(const void *eds, uint32_t ned, uint32_t n, cudaStream_t st);
+cudaError_t launch_clear_rows(uint64_t *rows, uint32_t *mark, size_t n_rows, uint32_t W, const uint32_t *all,
+                              cudaStream_t st);
 // Resume: OR seed (n_boxes x n rows of W words) into M2, A2 := M2 on the
 // rows it touches, those rows new in iteration 1.
 cudaError_t launch_seed_apply(const uint64_t *seed, uint64_t *m2, uint64_t *a2, uint32_t *a2_it, uint32_t *box_new_it,
@@ -216,6 +218,9 @@ struct QueryDev {
     std::vector<int32_t> blk_of;  // Q*Q -> block or -1
     std::vector<std::pair<uint32_t, uint32_t>> blocks;
     DBuf blk_mem, stamp_mem, last_mem, m2_mem, a2_mem, a2it_mem, boxit_mem, ctl_mem, eps_mem, ctl_ptr_mem, boxedge_mem;
+    DBuf all_dirty;  // one word: the bit rows' marks do not tell which rows hold bits (k_clear_rows)
+    bool all_dirty_set = false;  // the word is known to be set
+    int mark_all_dirty(cudaStream_t st, std::string *err);
     uint32_t n_eps = 0;
     uint64_t device_bytes = 0;
     // host descriptors (pointers filled once buffers exist; ctl set by the executor)

@@ -165,10 +165,21 @@ int run_executor(cfpq_ctx *ctx, Executor &ex, std::vector<QCtl> *ctls, uint32_t 
     if (tc_error)
         return fail(ctx, CFPQ_ERR_TIMEOUT, "a tile-product kernel gave up (bounded wait on its MMAs or on a counter)");
     if (ctx->opt.loop_mode != CFPQ_LOOP_HOST && launches) {
-        // the graph's loop body holds kLoopUnroll passes
         uint32_t passes = 0;
         for (const auto &c : *ctls) passes = std::max(passes, c.passes);
-        *launches = (passes + kLoopUnroll - 1) / kLoopUnroll * kLoopUnroll * per_pass + 2;
+        const uint32_t per = ex.loop_passes(), loops = (passes + per - 1) / per;
+        if (ex.level_work.empty()) {
+            *launches = loops * per * per_pass + 2;
+        } else {  // per level: its classes, its tile kernels, and extraction or control
+            uint32_t body = 0;
+            for (uint32_t p = 0; p < per; ++p) {
+                const auto &w = ex.level_work[p % ex.level_work.size()];
+                for (uint32_t k : w.items) body += k ? 1 : 0;
+                body += w.tiles ? (ex.any_uncompacted ? 6 : 5) : 0;
+                body += (p + 1) % ex.level_work.size() == 0 && n_extract ? n_extract : 1;
+            }
+            *launches = loops * body + 2;
+        }
     }
     CK(ctx, cudaGetLastError());
     return CFPQ_OK;

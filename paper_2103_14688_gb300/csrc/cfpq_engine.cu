@@ -1073,6 +1073,14 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
     ENG_CK(prepare_gather_launch());
     ENG_CK(cudaStreamSynchronize(st));
     drop_graph();
+    level_work.clear();
+    if (nq == 1 && qs[0]->loop_mask == 0) {
+        level_work.resize(qs[0]->n_levels);
+        for (uint32_t L = 0; L < qs[0]->n_levels; ++L) {
+            for (int v = 0; v < kClasses; ++v) level_work[L].items[v] = g_lvl[v][L + 1] - g_lvl[v][L];
+            level_work[L].tiles = t_lvl_tiles[L];
+        }
+    }
     built = true;
     return CFPQ_OK;
 }
@@ -1098,12 +1106,18 @@ int Executor::enqueue_lists(cudaStream_t st) {
 //   side:  column slices and expanded blocks; CSR gathers
 // The products follow the general gathers, whose plain stores to the same output
 // rows would drop their atomics; extraction and control follow everything.
+// With a level, kernels without work there are left out: of Dyck-4's three levels
+// only the last has tile jobs, general gathers and the extraction.
 int Executor::enqueue_pass(cudaStream_t st, cudaGraphConditionalHandle h, int use_handle, int *running_out,
-                           const cudaEvent_t *ev, bool branches) {
+                           const cudaEvent_t *ev, bool branches, int level) {
     std::string *err = nullptr;
+    const LevelWork *const lw = level >= 0 ? &level_work[(size_t)level] : nullptr;
+    const bool extract = !lw || (size_t)level + 1 == level_work.size();
+    auto live = [&](int c) { return lw ? lw->items[c] : max_live[c]; };
+    const uint32_t tiles = n_tcjobs == 0 ? 0u : lw ? lw->tiles : max_tc_tiles;
     const cudaStream_t sa = branches ? side[0] : st, sb = branches ? side[1] : st;
-    bool side_work[kBranches] = {max_live[kSlice] || max_live[kExpandNarrow] || max_live[kExpandWide], false};
-    for (int c = 0; c < kExpandNarrow; c += 2) side_work[1] |= max_live[c] != 0;
+    bool side_work[kBranches] = {live(kSlice) || live(kExpandNarrow) || live(kExpandWide), false};
+    for (int c = 0; c < kExpandNarrow; c += 2) side_work[1] |= live(c) != 0;
     if (branches && (side_work[0] || side_work[1])) {
         ENG_CK(cudaEventRecord(fork_ev, st));
         for (int i = 0; i < kBranches; ++i)
@@ -1113,21 +1127,19 @@ int Executor::enqueue_pass(cudaStream_t st, cudaGraphConditionalHandle h, int us
     // this pass (lower levels, or the previous pass of a cyclic level), and a
     // gather whose source's new edges the tiles take needs the job's list.
     if (ev) ENG_CK(cudaEventRecord(ev[0], st));
-    if (n_tcjobs) ENG_CK(launch_tc_compact(tcjobs.as<TcJob>(), T, max_tc_w, tc_err.as<int>(), st));
+    if (tiles) ENG_CK(launch_tc_compact(tcjobs.as<TcJob>(), T, max_tc_w, tc_err.as<int>(), st));
     if (ev) ENG_CK(cudaEventRecord(ev[1], st));
-    ENG_CK(launch_slice(items[kSlice].as<SliceItem>(), max_live[kSlice], slice_groups.as<SliceGroup>(),
+    ENG_CK(launch_slice(items[kSlice].as<SliceItem>(), live(kSlice), slice_groups.as<SliceGroup>(),
                         slice_mems.as<SliceMem>(), srcs.as<SrcDesc>(), slice_smem, T, kSlice, sa));
     for (int c = kExpandNarrow; c <= kExpandWide; ++c)
-        ENG_CK(launch_expand(c == kExpandWide, items[c].as<GItem>(), max_live[c], srcs.as<SrcDesc>(), max_expand_w, T, c,
-                             sa));
+        ENG_CK(launch_expand(c == kExpandWide, items[c].as<GItem>(), live(c), srcs.as<SrcDesc>(), max_expand_w, T, c, sa));
     for (int c = 0; c < kExpandNarrow; ++c)
-        ENG_CK(launch_gather(kVplOf[c / 2], (c & 1) != 0, items[c].as<GItem>(), max_live[c], srcs.as<SrcDesc>(), T, c,
+        ENG_CK(launch_gather(kVplOf[c / 2], (c & 1) != 0, items[c].as<GItem>(), live(c), srcs.as<SrcDesc>(), T, c,
                              (c & 1) ? st : sb));
     if (ev) ENG_CK(cudaEventRecord(ev[2], st));
-    if (n_tcjobs) {
-        if (any_uncompacted)
-            ENG_CK(launch_tc_product(false, tcjobs.as<TcJob>(), max_tc_tiles, T, tc_err.as<int>(), st));
-        ENG_CK(launch_tc_product_tma(tcjobs.as<TcJob>(), tcmaps.p, max_tc_tiles, T, tc_err.as<int>(), st, tile_kind));
+    if (tiles) {
+        if (any_uncompacted) ENG_CK(launch_tc_product(false, tcjobs.as<TcJob>(), tiles, T, tc_err.as<int>(), st));
+        ENG_CK(launch_tc_product_tma(tcjobs.as<TcJob>(), tcmaps.p, tiles, T, tc_err.as<int>(), st, tile_kind));
     }
     if (ev) ENG_CK(cudaEventRecord(ev[3], st));
     if (branches)
@@ -1139,9 +1151,9 @@ int Executor::enqueue_pass(cudaStream_t st, cudaGraphConditionalHandle h, int us
     // the last extraction launch of the pass also zeroes the tile jobs'
     // scratch and runs the loop control
     int last_x = -1;
-    for (int c = 0; c < kXClasses; ++c)
+    for (int c = 0; c < kXClasses && extract; ++c)
         if (n_xitems[c]) last_x = c;
-    for (int c = 0; c < kXClasses; ++c) {
+    for (int c = 0; c <= last_x; ++c) {
         const bool fuse = c == last_x;
         ENG_CK(launch_extract(kVplOf[c], xitems[c].as<XItem>(), n_xitems[c], fds.as<FDesc>(), T, c,
                               fuse ? ctl_ptrs.as<QCtl *>() : nullptr, (uint32_t)qs.size(), mirror.as<QCtl>(), h,
@@ -1149,7 +1161,7 @@ int Executor::enqueue_pass(cudaStream_t st, cudaGraphConditionalHandle h, int us
                               scratch_words_total, st));
     }
     if (last_x < 0) {
-        if (scratch_words_total) ENG_CK(cudaMemsetAsync(scratch.p, 0, scratch_words_total * 8, st));
+        if (tiles && scratch_words_total) ENG_CK(cudaMemsetAsync(scratch.p, 0, scratch_words_total * 8, st));
         ENG_CK(launch_control(ctl_ptrs.as<QCtl *>(), (uint32_t)qs.size(), mirror.as<QCtl>(), h, use_handle,
                               running_out, T, 1, st));
     }
@@ -1171,7 +1183,6 @@ int Executor::build_graph(cudaStream_t st, uint32_t max_iter, uint32_t max_round
     cudaGraph_t prologue = nullptr;
     ENG_CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     int rc = enqueue_prologue(cs, max_iter, max_rounds, max_passes);
-    const uint32_t kPassesPerLoop = kLoopUnroll;
     cudaError_t ce = cudaStreamEndCapture(cs, &prologue);
     if (rc || ce != cudaSuccess) {
         if (prologue) cudaGraphDestroy(prologue);
@@ -1196,9 +1207,12 @@ int Executor::build_graph(cudaStream_t st, uint32_t max_iter, uint32_t max_round
     ENG_CK(cudaGraphAddNode(&loop_node, graph, &pro_node, nullptr, 1, &cp));
     cudaGraph_t body = cp.conditional.phGraph_out[0];
     ENG_CK(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    // kPassesPerLoop passes per evaluation of the while node: a pass after the
-    // loop finished finds no live work and leaves the control state unchanged
-    for (uint32_t p = 0; p < kPassesPerLoop && rc == 0; ++p) rc = enqueue_pass(cs, handle, 1, nullptr, nullptr, true);
+    // Several passes per evaluation of the while node: a pass after the loop
+    // finished finds no live work and leaves the control state unchanged.  A
+    // query without repeating levels takes whole iterations, pass p on level p.
+    for (uint32_t p = 0; p < loop_passes() && rc == 0; ++p)
+        rc = enqueue_pass(cs, handle, 1, nullptr, nullptr, true,
+                          level_work.empty() ? -1 : (int)(p % (uint32_t)level_work.size()));
     cudaGraph_t body_out = body;
     ce = cudaStreamEndCapture(cs, &body_out);
     if (rc || ce != cudaSuccess) {

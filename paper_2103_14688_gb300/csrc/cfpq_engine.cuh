@@ -346,7 +346,8 @@ uint32_t tile_kind_of(uint32_t mode, uint32_t fmt, const Tuning &t);
 // measured rates when tuned, else the built-in constant of its format.
 uint32_t tile_ratio_of(uint32_t kind, const Tuning &t, uint32_t n);
 
-// Closure passes per iteration of the CUDA graph's while node.
+// Closure passes per iteration of the CUDA graph's while node (queries with one
+// level or with repeating levels, and several queries at once).
 constexpr uint32_t kLoopUnroll = 2;
 
 // Runs the fixpoint of a set of queries with shared launches.
@@ -395,8 +396,19 @@ struct Executor {
     // operands, after them (before the row gathers), after the gathers and
     // after the tile products.
     // branches: launch independent kernels on the side streams (graph capture).
+    // level: the level every running query is on (-1: any); only the kernels
+    // with work on that level are launched.
     int enqueue_pass(cudaStream_t st, cudaGraphConditionalHandle h, int use_handle, int *running_out,
-                     const cudaEvent_t *ev = nullptr, bool branches = false);
+                     const cudaEvent_t *ev = nullptr, bool branches = false, int level = -1);
+    // A single query without repeating levels passes through its levels in order:
+    // per level, the items of every class and the tile jobs; empty otherwise.
+    struct LevelWork {
+        uint32_t items[kClasses] = {0};
+        uint32_t tiles = 0;
+    };
+    std::vector<LevelWork> level_work;
+    // Passes in the body of the graph's while node.
+    uint32_t loop_passes() const { return level_work.size() <= 1 ? kLoopUnroll : (uint32_t)level_work.size(); }
     int build_graph(cudaStream_t st, uint32_t max_iter, uint32_t max_rounds, uint32_t max_passes, std::string *err);
     int read_ctls(cudaStream_t st, std::vector<QCtl> *out, int *tc_error = nullptr);
 };

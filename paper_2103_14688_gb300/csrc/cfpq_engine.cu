@@ -755,6 +755,19 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
         // executor's item scale (the server's larger items keep its frequent
         // re-assembly cheap), at most 1024
         const uint32_t rpi = std::min<uint32_t>(1024u, std::max<uint32_t>(64u, rows_per_step * 4u) * item_scale);
+        // Small graphs: items of that size would leave SMs without work (47
+        // items of 64 rows for a block at n = 3001, each warp on eight rows in turn:
+        // 27 us a pass; with items of 8 rows Dyck-4 went from 3.64 to 3.40 ms), so
+        // `blocks` blocks of a level are cut into four CTAs an SM's worth of items, a
+        // row per group at the least.  Not on levels that repeat: fewer, larger items see more of the rows that
+        // changed earlier in the same pass, which saves passes.
+        auto rows_for = [&](uint32_t blocks, bool repeats) -> uint32_t {
+            if (item_scale > 1u || repeats || blocks == 0u) return rpi;
+            const uint64_t want = (uint64_t)q.n * blocks * nq / (4u * 152u);
+            uint32_t rows = rpi;
+            while (rows > rows_per_step && rows > want) rows >>= 1;
+            return rows;
+        };
         // product jobs: tcgen05 tiles of 128 rows x 256 columns
         const uint32_t tiles_m = (q.n + 127u) / 128u, tiles_n = (q.n + 255u) / 256u;
         for (uint32_t L = 0; L <= q.n_levels; ++L) {
@@ -763,6 +776,10 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
             t_lvl[(size_t)qi * maxL1 + L] = (uint32_t)hj.size();
             if (L == q.n_levels) break;
             uint32_t lvl_tiles = 0;
+            uint32_t lvl_blocks = 0;
+            for (size_t b = 0; b < q.blocks.size(); ++b)
+                lvl_blocks += q.blk_level[b] == L && q.blk_nsrc[b] != 0 && q.blk_slice[b] < 0 ? 1u : 0u;
+            const uint32_t rpl = rows_for(lvl_blocks, (q.loop_mask >> L) & 1ull);
             for (uint32_t sg = 0; sg < q.n_slice_groups; ++sg) {
                 const uint32_t mem0 = (uint32_t)hsm.size();
                 std::vector<int32_t> member_of(q.blocks.size(), -1);
@@ -827,10 +844,10 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
                 const uint32_t rows_item =
                     q.restricted ? 1024u
                     : (has_nt && !expand && q.W >= 256u) ? std::min<uint32_t>(1024u, std::max<uint32_t>(rpi, 128u * item_scale))
-                                                         : rpi;
+                                                         : rpl;
                 // the gather lists an item's rows in 1024 entries of shared memory
-                if (rows_item > 1024u || rows_item % 64u != 0u) {
-                    *err = "gather items: rows per item must be a multiple of 64 and at most 1024";
+                if (rows_item == 0u || rows_item > 1024u) {
+                    *err = "gather items: at most 1024 rows per item";
                     return CFPQ_ERR_INVALID_ARG;
                 }
                 // slice-major: CTAs running side by side enumerate the same
@@ -946,7 +963,8 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
         for (int v = 0; v < kXClasses; ++v) x_rng[v][qi] = (uint32_t)hx[v].size();
         for (uint32_t b = 0; b < q.B; ++b) {
             if (q.box_nf[b] == 0) continue;
-            for (uint32_t r0 = 0; r0 < q.n; r0 += rpi) {
+            const uint32_t rpx = rows_for(2u * q.B, false);  // (its CTAs are counted one by one)
+            for (uint32_t r0 = 0; r0 < q.n; r0 += rpx) {
                 XItem x;
                 x.box_edges = q.boxedge_mem.as<unsigned long long>() + b;
                 x.m2 = q.m2_ptr(b);
@@ -957,7 +975,7 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
                 x.f0 = fbase + q.box_f0[b];
                 x.nf = q.box_nf[b];
                 x.row0 = r0;
-                x.row1 = std::min(q.n, r0 + rpi);
+                x.row1 = std::min(q.n, r0 + rpx);
                 x.W = q.W;
                 x.lpr = q.lpr;
                 hx[vi].push_back(x);

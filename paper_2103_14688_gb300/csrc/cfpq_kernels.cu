@@ -283,8 +283,7 @@ __global__ void __launch_bounds__(256, GatherCtas<VPL, NT>::value)
     k_gather(const GItem *__restrict__ items, const SrcDesc *__restrict__ srcs, ExecTables T, int cls) {
     constexpr bool kDyn = GatherDyn<VPL, NT>::on;
     __shared__ unsigned long long s_changed, s_ors;
-    // rows of the item with work: their bits, then the list (an item has at
-    // most 1024 rows and starts at a multiple of 64)
+    // rows of the item with work: their bits, then the list (an item has at most 1024 rows)
     __shared__ uint32_t s_rowbits[32];
     __shared__ uint16_t s_rows[1024];
     // general variant: per-warp ring of source rows loaded with cp.async

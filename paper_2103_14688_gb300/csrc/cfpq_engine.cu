@@ -259,21 +259,25 @@ int stage_graph(GraphDev *g, Allocator *A, cudaStream_t st, uint32_t n, uint32_t
     uint32_t *cnt = g->cnt.as<uint32_t>(), *off = g->off.as<uint32_t>(), *col = g->col.as<uint32_t>();
     uint32_t *ucnt = g->ucnt.as<uint32_t>(), *tmp = g->scan_tmp.as<uint32_t>();
     int *errf = g->err.as<int>();
-    ENG_CK(cudaMemsetAsync(cnt, 0, rows * 4, st));
-    ENG_CK(cudaMemsetAsync(errf, 0, 16, st));
-    ENG_CK(launch_stage_count(s, l, d, m, n, n_term, g->label_map.as<int32_t>(), cnt, errf, st));
-    ENG_CK(scan_exclusive(cnt, off, rows, tmp, st));
-    ENG_CK(cudaMemsetAsync(ucnt, 0, rows * 4, st));
-    ENG_CK(launch_stage_fill(s, l, d, m, n, n_term, g->label_map.as<int32_t>(), off, ucnt, col, st));
-    ENG_CK(launch_stage_unique(off, col, ucnt, rows, st));
-    ENG_CK(scan_exclusive(ucnt, g->csr_off.as<uint32_t>(), rows, tmp, st));
-    ENG_CK(launch_stage_compact(off, col, g->csr_off.as<uint32_t>(), g->csr_col.as<uint32_t>(), rows, st));
-    int herr = 0;
-    uint32_t total = 0;
-    ENG_CK(cudaMemcpyAsync(&herr, errf, 4, cudaMemcpyDeviceToHost, st));
-    ENG_CK(cudaMemcpyAsync(&total, g->csr_off.as<uint32_t>() + rows, 4, cudaMemcpyDeviceToHost, st));
+    if (stage_small_bytes(n, n_term, m)) {
+        ENG_CK(launch_stage_small(s, l, d, m, n, n_term, g->csr_off.as<uint32_t>(), g->csr_col.as<uint32_t>(), errf, st));
+    } else {
+        ENG_CK(cudaMemsetAsync(cnt, 0, rows * 4, st));
+        ENG_CK(cudaMemsetAsync(errf, 0, 16, st));
+        ENG_CK(launch_stage_count(s, l, d, m, n, n_term, g->label_map.as<int32_t>(), cnt, errf, st));
+        ENG_CK(scan_exclusive(cnt, off, rows, tmp, st));
+        ENG_CK(cudaMemsetAsync(ucnt, 0, rows * 4, st));
+        ENG_CK(launch_stage_fill(s, l, d, m, n, n_term, g->label_map.as<int32_t>(), off, ucnt, col, st));
+        ENG_CK(launch_stage_unique(off, col, ucnt, rows, st));
+        ENG_CK(scan_exclusive(ucnt, g->csr_off.as<uint32_t>(), rows, tmp, st));
+        ENG_CK(launch_stage_compact(off, col, g->csr_off.as<uint32_t>(), g->csr_col.as<uint32_t>(), rows,
+                                    reinterpret_cast<uint32_t *>(errf + 1), st));
+    }
+    int result[2] = {0, 0};  // an edge out of range; edges kept
+    ENG_CK(cudaMemcpyAsync(result, errf, sizeof(result), cudaMemcpyDeviceToHost, st));
     ENG_CK(cudaStreamSynchronize(st));
-    if (herr) {
+    const uint32_t total = (uint32_t)result[1];
+    if (result[0]) {
         *err = "an edge names a vertex >= n_vertices or a label >= n_terminals";
         g->n = 0;
         return CFPQ_ERR_INVALID_ARG;

@@ -79,7 +79,10 @@ cudaError_t launch_stage_fill(const uint32_t *src, const uint32_t *lbl, const ui
                               uint32_t *col, cudaStream_t st);
 cudaError_t launch_stage_unique(const uint32_t *off, uint32_t *col, uint32_t *ucnt, size_t rows, cudaStream_t st);
 cudaError_t launch_stage_compact(const uint32_t *off, const uint32_t *col, const uint32_t *uoff, uint32_t *ucol,
-                                 size_t rows, cudaStream_t st);
+                                 size_t rows, uint32_t *total_out, cudaStream_t st);
+size_t stage_small_bytes(uint32_t n, uint32_t n_term, size_t m);
+cudaError_t launch_stage_small(const uint32_t *src, const uint32_t *lbl, const uint32_t *dst, size_t m, uint32_t n,
+                               uint32_t n_term, uint32_t *csr_off, uint32_t *csr_col, int *result, cudaStream_t st);
 cudaError_t launch_popcount(const uint64_t *p, size_t nwords, unsigned long long *out, cudaStream_t st);
 cudaError_t launch_csr_to_coo(const uint32_t *off, const uint32_t *col, size_t rows, uint32_t n, uint32_t *coo,
                               cudaStream_t st);

@@ -126,7 +126,7 @@ extern "C" int cfpq_load_graph_device_noalloc(cfpq_ctx *ctx, uint32_t n, uint32_
         NA_CK(launch_stage_fill(d_src, d_label, d_dst, m, n, n_term, map, off, ucnt, col, st));
         NA_CK(launch_stage_unique(off, col, ucnt, rows, st));
         NA_CK(scan_exclusive(ucnt, g.csr_off.as<uint32_t>(), rows, tmp, st));
-        NA_CK(launch_stage_compact(off, col, g.csr_off.as<uint32_t>(), g.csr_col.as<uint32_t>(), rows, st));
+        NA_CK(launch_stage_compact(off, col, g.csr_off.as<uint32_t>(), g.csr_col.as<uint32_t>(), rows, nullptr, st));
         int herr = 0;
         uint32_t total = 0;
         NA_CK(cudaMemcpyAsync(&herr, errf, 4, cudaMemcpyDeviceToHost, st));

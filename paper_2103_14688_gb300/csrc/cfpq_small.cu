@@ -41,7 +41,11 @@ struct SmallDesc {
     uint32_t n, W, B, nblk, n_levels, max_iter, max_passes;
     uint32_t magic;           // ceil(2^32 / n): item / n = umulhi(item, magic) while item * n < 2^32; 0 for n = 1
     uint32_t meta_words;      // words of the plan's tables at `meta` (a multiple of 4)
-    uint32_t o_srcs, o_blk, o_src0, o_nsrc, o_f0, o_nf, o_null, o_fb;  // word offsets in `meta` (levels at 0)
+    uint32_t o_srcs, o_blk, o_src0, o_nsrc, o_f0, o_nf, o_null, o_fb, o_box;  // word offsets in `meta` (levels at 0)
+    // Every box's answer is one block, on the last level, which does not
+    // repeat and reads no nonterminal: its rows are extracted by the thread that
+    // computed them (o_box: block -> box or ~0).
+    uint32_t fuse;
     uint32_t pad;
     unsigned long long cyclic_mask;
     const uint32_t *meta;
@@ -63,14 +67,19 @@ struct SmallDesc {
 //     over without a barrier: what decides it is the same in every thread
 //     (register masks of the boxes and levels that changed);
 //   - a pass has one barrier, which also carries the "some row changed" flag;
-//     counters stay in registers until the end.
-// Two cycles 63 / 64: 23.1 -> 11.3 ms (1.9 us a pass before, with four barriers,
-// divisions and table loads from global memory); the regular query
-// (ab)*c|a*b* at n = 200: 620 -> 165 us.
-template <uint32_t W>
+//     counters stay in registers until the end;
+//   - where the last level allows it (SmallDesc::fuse) extraction is no phase of
+//     its own;
+//   - whether the tables and the CSR are in shared memory is known at compile
+//     time (SMEM), which makes their loads 32-bit shared ones.
+// Two cycles 63 / 64: 23.1 -> 9.7 ms (1.9 us a pass before, with four barriers,
+// divisions and table loads from global memory; 11.3 with extraction apart and
+// generic loads); the regular query (ab)*c|a*b* at n = 200: 620 -> 142 us.
+template <uint32_t W, bool SMEM>
 __global__ void __launch_bounds__(kSmallMaxThreads, 1)
     k_small_fixpoint(const SmallDesc *__restrict__ desc, uint32_t meta_smem, uint32_t csr_smem, uint32_t csr_rows,
                      uint32_t csr_m) {
+    if (SMEM) meta_smem = csr_smem = 1u;
     const SmallDesc &D = *desc;
     const uint32_t n = D.n, B = D.B, nblk = D.nblk;
     extern __shared__ __align__(16) uint64_t sm[];
@@ -89,26 +98,26 @@ __global__ void __launch_bounds__(kSmallMaxThreads, 1)
     for (uint32_t i = tid; i < words64; i += T) sm[i] = 0ull;
     for (uint32_t i = tid; i < words32; i += T) stamp[i] = 0u;
     uint32_t *extra = stamp + ((words32 + 3u) & ~3u);  // 16-byte aligned: the tables, then the CSR
-    const uint32_t *meta = D.meta;
-    if (meta_smem) {
+    uint32_t *const s_csr = extra + (meta_smem ? D.meta_words : 0u);
+    if (meta_smem)
         for (uint32_t i = tid; i < D.meta_words; i += T) extra[i] = D.meta[i];
-        meta = extra;
-        extra += D.meta_words;
-    }
-    const uint32_t *csr_off = D.csr_off, *csr_col = D.csr_col;
     if (csr_smem) {
-        for (uint32_t i = tid; i <= csr_rows; i += T) extra[i] = D.csr_off[i];
-        for (uint32_t i = tid; i < csr_m; i += T) extra[csr_rows + 1u + i] = D.csr_col[i];
-        csr_off = extra;
-        csr_col = extra + csr_rows + 1u;
+        for (uint32_t i = tid; i <= csr_rows; i += T) s_csr[i] = D.csr_off[i];
+        for (uint32_t i = tid; i < csr_m; i += T) s_csr[csr_rows + 1u + i] = D.csr_col[i];
     }
+    const uint32_t *const meta = SMEM ? extra : meta_smem ? extra : D.meta;
+    const uint32_t *const csr_off = SMEM ? s_csr : csr_smem ? s_csr : D.csr_off;
+    const uint32_t *const csr_col = SMEM ? s_csr + csr_rows + 1u : csr_smem ? s_csr + csr_rows + 1u : D.csr_col;
     if (tid == 0) { s_new = 0; s_ors = 0; s_rows = 0; }
     __syncthreads();
     const SmallLevel *levels = reinterpret_cast<const SmallLevel *>(meta);
     const SmallSrc *srcs = reinterpret_cast<const SmallSrc *>(meta + D.o_srcs);
     const uint32_t *lvl_blk = meta + D.o_blk, *blk_src0 = meta + D.o_src0, *blk_nsrc = meta + D.o_nsrc;
     const uint32_t *box_f0 = meta + D.o_f0, *box_nf = meta + D.o_nf, *nullable = meta + D.o_null;
-    const uint32_t *fblocks = meta + D.o_fb;
+    const uint32_t *fblocks = meta + D.o_fb, *blk_box = meta + D.o_box;
+    const bool fuse = D.fuse != 0u;
+    const uint32_t n_levels = D.n_levels, magic = D.magic, max_passes = D.max_passes;
+    const unsigned long long cyclic_mask = D.cyclic_mask;
 
     unsigned long long edges_eps = 0, my_new = 0;
     unsigned long long new_boxes = 0;  // boxes (< 64) with edges new in this iteration
@@ -134,9 +143,11 @@ __global__ void __launch_bounds__(kSmallMaxThreads, 1)
     while (!done) {
         const uint32_t g0 = g;
         unsigned long long lvl_changed = 0;  // levels that changed in this iteration
-        for (uint32_t L = 0; L < D.n_levels && !done; ++L) {
+        bool added = false;
+        for (uint32_t L = 0; L < n_levels && !done; ++L) {
             const SmallLevel lv = levels[L];
-            const bool cyc = (D.cyclic_mask >> L) & 1ull;
+            const bool cyc = (cyclic_mask >> L) & 1ull;
+            const bool fused = fuse && L + 1u == n_levels;
             bool active = (iter == 1u && lv.has_term) || (lv.boxes & new_boxes) != 0ull || (lv.any_box && new_any) ||
                           (lv.reads & lvl_changed) != 0ull;
             uint32_t mode = kModeNew;
@@ -144,7 +155,7 @@ __global__ void __launch_bounds__(kSmallMaxThreads, 1)
                 bool ch_any = false;
                 const uint32_t items = active ? lv.nblk * n : 0u;
                 for (uint32_t item = tid; item < items; item += T) {
-                    const uint32_t bi = D.magic ? __umulhi(item, D.magic) : item, x = item - bi * n;
+                    const uint32_t bi = magic ? __umulhi(item, magic) : item, x = item - bi * n;
                     const uint32_t b = lvl_blk[lv.blk0 + bi];
                     uint64_t acc[W];
 #pragma unroll
@@ -169,11 +180,11 @@ __global__ void __launch_bounds__(kSmallMaxThreads, 1)
                             const uint32_t thr = new_edges ? 0u : (cb == 2u ? g0 : g - 1u);
                             const uint32_t *rstamp = stamp + (s.rblk >= 0 ? (uint32_t)s.rblk * n : 0u);
                             const uint64_t *rrow = C + (s.rblk >= 0 ? (uint32_t)s.rblk * n * W : 0u);
-                            auto take = [&](uint32_t y) {
-                                if (ident) {
+                            auto take = [&](uint32_t y) __attribute__((always_inline)) {
+                                if (ident && s.kind == 0) {
+                                    const uint64_t bit = 1ull << (y & 63);
 #pragma unroll
-                                    for (uint32_t w = 0; w < W; ++w)
-                                        if (w == (y >> 6)) acc[w] |= 1ull << (y & 63);
+                                    for (uint32_t w = 0; w < W; ++w) acc[w] |= (y >> 6) == w ? bit : 0ull;
                                     any = true;
                                 }
                                 if (s.rblk >= 0 && (thr == 0u || rstamp[y] >= thr)) {
@@ -195,6 +206,12 @@ __global__ void __launch_bounds__(kSmallMaxThreads, 1)
                             } else {
                                 if (new_edges && a2it[s.label * n + x] != iter) continue;
                                 const uint64_t *adj = (new_edges ? A2 : M2) + (s.label * n + x) * W;
+                                if (ident) {  // the row's product edges into t are the row itself
+#pragma unroll
+                                    for (uint32_t w = 0; w < W; ++w) acc[w] |= adj[w];
+                                    any = true;
+                                    if (s.rblk < 0) continue;
+                                }
 #pragma unroll 1
                                 for (uint32_t w = 0; w < W; ++w) {
                                     uint64_t bits = adj[w];
@@ -221,15 +238,38 @@ __global__ void __launch_bounds__(kSmallMaxThreads, 1)
                     if (ch) {
                         stamp[b * n + x] = g;
                         last[b] = g;
-                        ch_any = true;
                         ++my_rows;
+                        if (!fused) ch_any = true;
+                        const uint32_t box = fused ? blk_box[b] : 0xFFFFFFFFu;
+                        if (box != 0xFFFFFFFFu) {  // the row's new pairs
+                            uint64_t *m = M2 + (box * n + x) * W, *a = A2 + (box * n + x) * W;
+                            bool has = false;
+#pragma unroll
+                            for (uint32_t w = 0; w < W; ++w) {
+                                acc[w] = o[w] & ~m[w];
+                                has |= acc[w] != 0ull;
+                            }
+                            if (has) {
+#pragma unroll
+                                for (uint32_t w = 0; w < W; ++w) {
+                                    a[w] = acc[w];
+                                    m[w] |= acc[w];
+                                    my_new += (unsigned long long)__popcll(acc[w]);
+                                }
+                                a2it[box * n + x] = iter + 1;
+                                boxit[box] = iter + 1;
+                                ch_any = true;
+                            }
+                        }
                     }
                 }
+                // (a fused level's flag says whether pairs were added)
                 const bool changed = active && __syncthreads_or(ch_any) != 0;
+                if (fused) added = changed;
                 if (changed) lvl_changed |= 1ull << L;
                 ++passes;
                 g += 1;
-                if (passes >= D.max_passes) {
+                if (passes >= max_passes) {
                     status = kStatusPassCap;
                     done = true;
                     break;
@@ -244,8 +284,8 @@ __global__ void __launch_bounds__(kSmallMaxThreads, 1)
         if (done) break;
         // extraction: new = OR_f C[q0, f] & ~M2 on rows changed this iteration
         bool has_new = false;
-        for (uint32_t item = tid; item < B * n; item += T) {
-            const uint32_t b = D.magic ? __umulhi(item, D.magic) : item, x = item - b * n;
+        for (uint32_t item = tid; item < B * n && !fuse; item += T) {
+            const uint32_t b = magic ? __umulhi(item, magic) : item, x = item - b * n;
             const uint32_t f0 = box_f0[b], f1 = f0 + box_nf[b];
             uint64_t cand[W];
 #pragma unroll
@@ -279,7 +319,7 @@ __global__ void __launch_bounds__(kSmallMaxThreads, 1)
             boxit[b] = iter + 1;
             has_new = true;
         }
-        const bool added = __syncthreads_or(has_new) != 0;
+        if (!fuse) added = __syncthreads_or(has_new) != 0;
         iters_done = iter;
         if (!added) break;
         if (D.max_iter && iter >= D.max_iter) {
@@ -353,11 +393,12 @@ cudaError_t launch_small_fixpoint(const void *desc, uint32_t W, size_t state_sme
                                          (uint32_t)csr_m);
         return cudaGetLastError();
     };
+    const bool both = meta_smem && csr_smem;
     switch (W) {
-        case 2: return run(k_small_fixpoint<2>);
-        case 4: return run(k_small_fixpoint<4>);
-        case 6: return run(k_small_fixpoint<6>);
-        case 8: return run(k_small_fixpoint<8>);
+        case 2: return both ? run(k_small_fixpoint<2, true>) : run(k_small_fixpoint<2, false>);
+        case 4: return both ? run(k_small_fixpoint<4, true>) : run(k_small_fixpoint<4, false>);
+        case 6: return both ? run(k_small_fixpoint<6, true>) : run(k_small_fixpoint<6, false>);
+        case 8: return both ? run(k_small_fixpoint<8, true>) : run(k_small_fixpoint<8, false>);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -407,6 +448,19 @@ std::vector<uint32_t> build_small_plan(const QueryDev &q, void *desc_out) {
     for (uint32_t b = 0; b < q.B; ++b) null_box[b] = q.rsm.final_[q.rsm.box_start[b]] ? 1u : 0u;
     d.o_null = put(null_box.data(), null_box.size() * 4);
     d.o_fb = put(q.fblocks.data(), q.fblocks.size() * 4);
+    std::vector<uint32_t> box_of(nblk, 0xFFFFFFFFu);
+    bool fuse = q.n_levels > 0 && !((q.cyclic_mask >> (q.n_levels - 1u)) & 1ull);
+    for (uint32_t b = 0; b < q.B; ++b) {
+        if (q.box_nf[b] == 0) continue;
+        const uint32_t fb = q.fblocks[q.box_f0[b]];
+        fuse = fuse && q.box_nf[b] == 1u && q.blk_level[fb] + 1u == q.n_levels;
+        box_of[fb] = b;
+    }
+    for (uint32_t b = 0; b < nblk && fuse; ++b)
+        for (uint32_t k = 0; k < q.blk_nsrc[b] && q.blk_level[b] + 1u == q.n_levels; ++k)
+            fuse = fuse && q.srcs[q.blk_src0[b] + k].label_kind == 0;
+    d.o_box = put(box_of.data(), box_of.size() * 4);
+    d.fuse = fuse ? 1u : 0u;
     while (m.size() % 4) m.push_back(0u);
     d.n = q.n;
     d.W = q.W;

@@ -987,10 +987,15 @@ __global__ void __launch_bounds__(256, kExpandOcc)
 // thirds of the lanes idle: 9 us a sweep at n = 8192): 32 packed edges (x << 16 |
 // y) per warp and coalesced load, eight in flight a thread; a byte per row holds
 // the sweep that last changed it, and only edges from rows changed in this sweep or
-// the one before read their words.  Regular query: n = 1000 1785 -> 385 us,
-// n = 8192 2119 -> 1369 us.  Above 200 KB a slice (n = 22755 for one state) the
-// component stays on the row gather, which also does less work on the sparse
-// rows that such graphs have.
+// the one before read their words.  Slices of up to 2048 rows (R > 0) are bound by
+// latency instead: a thread owns R rows for all sweeps and holds the places of their
+// first four edges in registers, so that a row costs five independent loads and no
+// atomics (further edges are listed and applied edge by edge).  Regular query:
+// n = 1000 1785 -> 385 us with edge sweeps (241 us of run time), 183 us of run time with
+// owned rows; n = 8192 2119 -> 1369 us (owned rows: no gain, 1.07 ms of run time against
+// 1.04).  Above 200 KB a slice (n = 22755 for one state) the component stays on
+// the row gather, which also does less work on the sparse rows that such graphs
+// have.
 // --------------------------------------------------------------------------
 constexpr uint32_t kSliceThreads = 1024, kSliceEdges = 4;
 __device__ __forceinline__ void or64(uint64_t *p, uint64_t v) {  // (32-bit shared atomics are native)
@@ -998,11 +1003,14 @@ __device__ __forceinline__ void or64(uint64_t *p, uint64_t v) {  // (32-bit shar
     if ((uint32_t)v) atomicOr(h, (uint32_t)v);
     if ((uint32_t)(v >> 32)) atomicOr(h + 1, (uint32_t)(v >> 32));
 }
+template <int R>
 __global__ void __launch_bounds__(kSliceThreads, 1)
     k_slice(const SliceItem *__restrict__ items, const SliceGroup *__restrict__ groups,
             const SliceMem *__restrict__ mems, const SrcDesc *__restrict__ srcs, ExecTables T, int cls) {
     extern __shared__ uint64_t s_col[];  // [nmem][n] words, then [nmem][n] bytes
     __shared__ uint32_t s_e0[kSliceMaxSrc], s_e1[kSliceMaxSrc], s_to[kSliceMaxSrc], s_from[kSliceMaxSrc], s_n;
+    __shared__ const uint32_t *s_off[kSliceMaxSrc], *s_adj;
+    __shared__ uint32_t s_rest_n;
     __shared__ unsigned long long s_changed, s_ors;
     const uint32_t tid = threadIdx.x, NT = blockDim.x, total = T.g_total[cls];
     for (uint32_t li = blockIdx.x; li < total; li += gridDim.x) {
@@ -1034,6 +1042,8 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
                 for (uint32_t k = 0; k < M.nsrc; ++k) {
                     const SrcDesc &d = srcs[M.src0 + k];
                     if (d.slice_mem == kSliceNone) continue;
+                    s_off[k2] = d.csr_off;
+                    s_adj = d.csr_col;
                     s_e0[k2] = d.csr_off[0];
                     s_e1[k2] = d.csr_off[n];
                     s_to[k2] = m * n;
@@ -1042,6 +1052,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
                 }
             }
             s_n = k2;
+            s_rest_n = 0u;
         }
         for (uint32_t m = 0; m < G.nmem; ++m) {
             const uint64_t *const o = mems[G.mem0 + m].out;
@@ -1073,10 +1084,81 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
             }
         }
         __syncthreads();
+        const uint32_t ns = s_n;
+        if constexpr (R > 0) {
+            // this thread's rows tid, tid + NT, ...: places of their first four
+            // edges (where there are fewer, the row's own: four plain loads beat
+            // four branches, 100 instructions a row), and whether there are more
+            uint32_t place[R][2], more = 0u;
+            uint32_t *const s_rest = reinterpret_cast<uint32_t *>(s_col + rows);  // edges past the fourth
+            const uint32_t rest_cap = rows / 4u;
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                const uint32_t row = tid + (uint32_t)i * NT;
+                place[i][0] = place[i][1] = row < rows ? row | (row << 16) : 0u;
+                if (row >= rows) continue;
+                const uint32_t m0 = row / n * n, x = row - m0;
+                uint32_t got = 0u;
+                for (uint32_t k = 0; k < ns; ++k) {
+                    if (s_to[k] != m0) continue;
+                    const uint32_t e1 = s_off[k][x + 1];
+                    for (uint32_t e = s_off[k][x]; e < e1; ++e, ++got) {
+                        const uint32_t at = s_from[k] + s_adj[e];
+                        if (got == 0u) place[i][0] = (place[i][0] & 0xFFFF0000u) | at;
+                        else if (got == 1u) place[i][0] = (place[i][0] & 0xFFFFu) | (at << 16);
+                        else if (got == 2u) place[i][1] = (place[i][1] & 0xFFFF0000u) | at;
+                        else if (got == 3u) place[i][1] = (place[i][1] & 0xFFFFu) | (at << 16);
+                        else {
+                            const uint32_t j = atomicAdd(&s_rest_n, 1u);
+                            if (j < rest_cap) s_rest[j] = (row << 16) | at;
+                            else more |= 1u << i;  // no room: the row walks its edges in the CSR
+                        }
+                    }
+                }
+            }
+            __syncthreads();
+            const uint32_t rest = min(s_rest_n, rest_cap);
+            bool ch = true;
+            while (__syncthreads_or(ch)) {
+                ch = false;
+                // (a row's owner may overwrite bits set here; the next sweep, which
+                // this one's change causes, sets them again)
+                for (uint32_t j = tid; j < rest; j += NT) {
+                    const uint32_t ra = s_rest[j], row = ra >> 16;
+                    const uint64_t v = s_col[ra & 0xFFFFu] & ~s_col[row];
+                    if (v) {
+                        or64(s_col + row, v);
+                        ch = true;
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < R; ++i) {
+                    const uint32_t row = tid + (uint32_t)i * NT;
+                    if (i * NT >= rows) break;  // (uniform)
+                    const uint64_t old = s_col[row < rows ? row : 0u];
+                    uint64_t v = s_col[place[i][0] & 0xFFFFu] | s_col[place[i][0] >> 16] | s_col[place[i][1] & 0xFFFFu] |
+                                 s_col[place[i][1] >> 16];
+                    if ((more >> i) & 1u) {
+                        const uint32_t m0 = row / n * n, x = row - m0;
+                        uint32_t got = 0u;
+                        for (uint32_t k = 0; k < ns; ++k) {
+                            if (s_to[k] != m0) continue;
+                            const uint32_t e1 = s_off[k][x + 1];
+                            for (uint32_t e = s_off[k][x]; e < e1; ++e, ++got)
+                                if (got >= 4u) v |= s_col[s_from[k] + s_adj[e]];
+                        }
+                    }
+                    if (v & ~old) {
+                        ++my_ors;
+                        s_col[row] = old | v;
+                        ch = true;
+                    }
+                }
+            }
+        } else {
         // mark: the low byte of the sweep that last changed the row (rows with bits start as
         // changed in sweep 0; 128 is no sweep within reach of the first ones)
         for (uint32_t x = tid; x < rows; x += NT) s_mark[x] = s_col[x] ? 0u : 128u;
-        const uint32_t ns = s_n;
         uint32_t sweep = 0u;
         bool ch = true;
         while (__syncthreads_or(ch)) {
@@ -1118,6 +1200,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
                     }
                 }
             }
+        }
         }
         uint32_t my_changed = 0u;
         for (uint32_t m = 0; m < G.nmem; ++m) {
@@ -1963,8 +2046,10 @@ cudaError_t launch_slice(const SliceItem *items, uint32_t n_items, const SliceGr
     const uint32_t grid = sms ? std::min<uint32_t>(n_items, sms * 4u) : n_items;
     // small slices: a barrier over 16 warps costs less than their extra loads gain (n = 1000: 44 us
     // against 56 for a level; n = 8192: 115 against 98)
-    const uint32_t threads = smem >= 4096u * 9u ? kSliceThreads : kSliceThreads / 2u;
-    k_slice<<<grid, threads, smem, st>>>(items, groups, mems, srcs, T, cls);
+    const uint32_t rows = smem / 9u, threads = rows >= 4096u ? kSliceThreads : kSliceThreads / 2u;
+    if (rows <= 1024u) k_slice<2><<<grid, threads, smem, st>>>(items, groups, mems, srcs, T, cls);
+    else if (rows <= 2048u) k_slice<4><<<grid, threads, smem, st>>>(items, groups, mems, srcs, T, cls);
+    else k_slice<0><<<grid, threads, smem, st>>>(items, groups, mems, srcs, T, cls);
     return cudaGetLastError();
 }
 
@@ -1972,8 +2057,14 @@ cudaError_t launch_slice(const SliceItem *items, uint32_t n_items, const SliceGr
 // (call outside any stream capture).
 cudaError_t prepare_gather_launch() {
     {
-        const cudaError_t e =
-            cudaFuncSetAttribute(k_slice, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSliceMaxBytes);
+        cudaError_t e = cudaSuccess;
+        auto room = [&](auto kernel) {
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSliceMaxBytes);
+        };
+        room(k_slice<0>);
+        room(k_slice<2>);
+        room(k_slice<4>);
         if (e != cudaSuccess) return e;
     }
 #define CFPQ_RING(V)                                                                                      \

@@ -367,7 +367,7 @@ class Context:
     # -- results --
     def reachable_words(self, box: int = 0) -> np.ndarray:
         wn = (self.n + 63) // 64
-        out = np.zeros(self.n * wn, dtype=np.uint64)
+        out = np.empty(self.n * wn, dtype=np.uint64)  # (written whole)
         self._check(self.lib.cfpq_get_reachable_bits(self.h, box, c_void_p(out.ctypes.data)),
                     "cfpq_get_reachable_bits")
         return out.reshape(self.n, wn)
@@ -437,7 +437,7 @@ class Context:
         """M2^box of query q of the last batch as bit rows, uint64 [n, ceil(n/64)]."""
         n = self._batch_n[q]
         wn = (n + 63) // 64
-        out = np.zeros(n * wn, dtype=np.uint64)
+        out = np.empty(n * wn, dtype=np.uint64)  # (written whole)
         self._check(self.lib.cfpq_batch_get_reachable_bits(self.h, q, box, c_void_p(out.ctypes.data)),
                     "cfpq_batch_get_reachable_bits")
         return out.reshape(n, wn)
@@ -518,7 +518,7 @@ class Server:
     def result_words(self, ticket: int, box: int = 0) -> np.ndarray:
         """M2^box of a finished query as bit rows, uint64 [n, ceil(n/64)]."""
         wn = (self.n + 63) // 64
-        out = np.zeros(self.n * wn, dtype=np.uint64)
+        out = np.empty(self.n * wn, dtype=np.uint64)  # (written whole)
         rc = self.lib.cfpq_result_reachable_bits(self.h, ticket, box, c_void_p(out.ctypes.data))
         if rc != CFPQ_OK:
             raise CfpqError(rc, "cfpq_result_reachable_bits: " + status_string(rc))

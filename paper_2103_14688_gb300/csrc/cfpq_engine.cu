@@ -94,7 +94,7 @@ void bind_slab(SlabArena *s, Allocator *parent, cudaStream_t st) {
 // present are only counted.  A store only: a load would first map the zero page,
 // whose replacement costs far more than the fault saved (512 MiB: 200 ms).
 static void touch_pages(void *p, size_t bytes) {
-    constexpr size_t kFrom = (size_t)1 << 20, kPerThread = (size_t)8 << 20;
+    constexpr size_t kFrom = (size_t)1 << 20, kPerThread = (size_t)2 << 20;
     if (bytes < kFrom) return;
     cudaPointerAttributes at;  // pinned and managed pages are left alone
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess || at.type != cudaMemoryTypeUnregistered) {

@@ -2095,11 +2095,11 @@ cudaError_t launch_extract(int vpl, const XItem *items, uint32_t n_items, const 
     if (n_items == 0) return cudaSuccess;
     FusedControl fc{ctls, mirror, running_out, done_counter, h, nq, use_handle, ctls != nullptr ? 1 : 0, zero,
                     zero_words};
-    // (the CTAs stride over the live items; see launch_gather)
+    // one wave of CTAs that stride over the live items: every CTA of the fused launch is counted
     int dev = 0;
     cudaGetDevice(&dev);
     const uint32_t sms = (dev >= 0 && dev < 64 && g_gather_sms[dev]) ? (uint32_t)g_gather_sms[dev] : 0u;
-    const uint32_t grid = sms ? std::min<uint32_t>(n_items, sms * 8u * kStrideWaves) : n_items;
+    const uint32_t grid = sms ? std::min<uint32_t>(n_items, sms * 8u) : n_items;
     switch (vpl) {
         case 1: k_extract<1><<<grid, 256, 0, st>>>(items, fds, T, cls, fc); break;
         case 2: k_extract<2><<<grid, 256, 0, st>>>(items, fds, T, cls, fc); break;

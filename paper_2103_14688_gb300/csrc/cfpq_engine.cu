@@ -9,7 +9,6 @@
 #include <algorithm>
 #include <cstring>
 #include <string>
-#include <system_error>
 #include <thread>
 #include <type_traits>
 
@@ -93,7 +92,7 @@ void bind_slab(SlabArena *s, Allocator *parent, cudaStream_t st) {
 // first 512 MiB take 3.6 + 2.9 ms, 18 MiB by one 0.8 + 0.1 instead of 10.  Pages already
 // present are only counted.  A store only: a load would first map the zero page,
 // whose replacement costs far more than the fault saved (512 MiB: 200 ms).
-static void touch_pages(void *p, size_t bytes) {
+static void touch_pages(void *p, size_t bytes) try {
     constexpr size_t kFrom = (size_t)1 << 20, kPerThread = (size_t)2 << 20;
     if (bytes < kFrom) return;
     cudaPointerAttributes at;  // pinned and managed pages are left alone
@@ -122,11 +121,12 @@ static void touch_pages(void *p, size_t bytes) {
     th.reserve(want);
     try {
         for (size_t a = per; a < n_pages; a += per) th.emplace_back(touch, a, std::min(n_pages, a + per));
-    } catch (const std::system_error &) {
+    } catch (...) {
         // fewer threads: the copy faults the other pages in
     }
     touch(0, std::min(n_pages, per));
     for (auto &t : th) t.join();
+} catch (...) {  // (no memory for the page list: the copy faults them all in)
 }
 
 // Always a linear copy: cudaMemcpy2D, also with equal pitches, lets the copy

@@ -1148,7 +1148,9 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
                                 if (got >= 4u) v |= s_col[s_from[k] + s_adj[e]];
                         }
                     }
-                    if (v & ~old) {
+                    // (a thread past the last row read row 0's word five times: it may have
+                    // grown in between, and there is no row to store)
+                    if (row < rows && (v & ~old)) {
                         ++my_ors;
                         s_col[row] = old | v;
                         ch = true;

@@ -1343,21 +1343,19 @@ __global__ void __launch_bounds__(256) k_extract(const XItem *__restrict__ items
     if (FC.enabled) {
         for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < FC.zero_words; i += (size_t)gridDim.x * blockDim.x)
             FC.zero[i] = 0ull;
-        if (total == 0u) {
-            // a pass without extraction: nothing here for the control to wait for
-            if (threadIdx.x == 0) s_last = blockIdx.x == 0 ? 1 : 0;
-        } else {
-            __threadfence();
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                const unsigned int prev = atomicAdd(FC.done_counter, 1u);
-                s_last = (prev == gridDim.x - 1) ? 1 : 0;
-            }
+        // Control rewrites what every CTA of this launch reads (x_total, the live
+        // lists, the queries' state), so the CTA that finishes last runs it, in a pass
+        // without extraction too: CTAs may start late (several waves, other work on the SMs).
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const unsigned int prev = atomicAdd(FC.done_counter, 1u);
+            s_last = (prev == gridDim.x - 1) ? 1 : 0;
         }
         __syncthreads();
         if (s_last) {
             __threadfence();
-            if (threadIdx.x == 0 && total != 0u) *FC.done_counter = 0u;
+            if (threadIdx.x == 0) *FC.done_counter = 0u;
             control_body(FC.ctls, FC.nq, FC.mirror, FC.handle, FC.use_handle, FC.running_out, T, 1);
         }
     }

@@ -276,7 +276,7 @@ struct GatherDyn {
 // than 256-4096 bits to enumerate to a second launch split over 16 warps
 // gained 1-2% in AUTO and cost 10-20% bit-packed: not kept.)
 constexpr uint32_t kGatherParts = 8;
-constexpr uint32_t kStrideWaves = 8;  // launch_gather / launch_extract: waves of resident CTAs at most
+constexpr uint32_t kStrideWaves = 8;  // launch_gather: waves of resident CTAs at most
 
 template <int VPL, bool NT>
 __global__ void __launch_bounds__(256, GatherCtas<VPL, NT>::value)
@@ -1990,6 +1990,7 @@ int vpl_for_words(uint32_t W) {
 }
 
 static int g_gather_sms[64];
+static int g_extract_ctas[64][kXClasses];  // CTAs of k_extract that a device holds at once, per row width
 
 cudaError_t launch_gather(int vpl, bool nt, const GItem *items, uint32_t n_items, const SrcDesc *srcs,
                           const ExecTables &T, int cls, cudaStream_t st) {
@@ -2082,6 +2083,15 @@ cudaError_t prepare_gather_launch() {
     int sms = 0;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
+    int per_sm[kXClasses];
+    const void *const extract[kXClasses] = {(const void *)k_extract<1>, (const void *)k_extract<2>,
+                                            (const void *)k_extract<4>, (const void *)k_extract<8>,
+                                            (const void *)k_extract<16>};
+    for (int c = 0; c < kXClasses; ++c) {
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[c], extract[c], 256, 0);
+        if (e != cudaSuccess) return e;
+    }
+    for (int c = 0; c < kXClasses; ++c) g_extract_ctas[dev][c] = sms * std::max(1, per_sm[c]);
     g_gather_sms[dev] = sms;
     return cudaSuccess;
 }
@@ -2095,11 +2105,12 @@ cudaError_t launch_extract(int vpl, const XItem *items, uint32_t n_items, const 
     if (n_items == 0) return cudaSuccess;
     FusedControl fc{ctls, mirror, running_out, done_counter, h, nq, use_handle, ctls != nullptr ? 1 : 0, zero,
                     zero_words};
-    // one wave of CTAs that stride over the live items: every CTA of the fused launch is counted
+    // resident CTAs that stride over the live items (3, 3, 2, 1 and 1 an SM by row width: registers):
+    // every CTA of the fused launch is counted, and a pass without extraction is nothing but that count
     int dev = 0;
     cudaGetDevice(&dev);
-    const uint32_t sms = (dev >= 0 && dev < 64 && g_gather_sms[dev]) ? (uint32_t)g_gather_sms[dev] : 0u;
-    const uint32_t grid = sms ? std::min<uint32_t>(n_items, sms * 8u) : n_items;
+    const uint32_t ctas = (dev >= 0 && dev < 64) ? (uint32_t)g_extract_ctas[dev][cls] : 0u;
+    const uint32_t grid = ctas ? std::min<uint32_t>(n_items, ctas) : n_items;
     switch (vpl) {
         case 1: k_extract<1><<<grid, 256, 0, st>>>(items, fds, T, cls, fc); break;
         case 2: k_extract<2><<<grid, 256, 0, st>>>(items, fds, T, cls, fc); break;

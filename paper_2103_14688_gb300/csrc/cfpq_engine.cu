@@ -232,7 +232,9 @@ int stage_graph(GraphDev *g, Allocator *A, cudaStream_t st, uint32_t n, uint32_t
     const size_t rows = (size_t)n_term * n;
     if (rows + 1 >= 0xffffffffull) { *err = "n_vertices * n_terminals too large"; return CFPQ_ERR_UNSUPPORTED; }
     const size_t mm = m ? m : 1;
-    const bool realloc = !(g->csr_off.p && g->csr_off.bytes >= (rows + 1) * 4 && g->csr_col.bytes >= mm * 4);
+    const bool realloc = !(g->csr_off.p && g->csr_off.bytes >= (rows + 1) * 4 && g->csr_col.bytes >= mm * 4 &&
+                           g->col.bytes >= mm * 4);
+    g->coo_content = ~0ull;  // (col is overwritten)
     const size_t nb = (rows + 4095) / 4096 + 2;
     if (!g->csr_off.ensure(A, (rows + 1) * 4, err) || !g->csr_col.ensure(A, mm * 4, err) ||
         !g->cnt.ensure(A, rows * 4, err) || !g->off.ensure(A, (rows + 1) * 4, err) || !g->col.ensure(A, mm * 4, err) ||
@@ -303,9 +305,10 @@ int GraphDev::ensure_nonempty(Allocator *A, cudaStream_t st, std::string *err) {
 }
 
 int GraphDev::ensure_coo(Allocator *A, cudaStream_t st, std::string *err) {
-    if (coo.p && coo_content == content) return CFPQ_OK;
-    if (!coo.ensure(A, csr_col.bytes, err)) return CFPQ_ERR_OUT_OF_MEMORY;  // (as many edges as the CSR has room for)
-    ENG_CK(launch_csr_to_coo(csr_off.as<uint32_t>(), csr_col.as<uint32_t>(), (size_t)n_term * n, n, coo.as<uint32_t>(),
+    if (col.p && coo_content == content) return CFPQ_OK;
+    // (col was staged with as much room as the CSR; only a failed load leaves it smaller)
+    if (!col.ensure(A, csr_col.bytes, err)) return CFPQ_ERR_OUT_OF_MEMORY;
+    ENG_CK(launch_csr_to_coo(csr_off.as<uint32_t>(), csr_col.as<uint32_t>(), (size_t)n_term * n, n, col.as<uint32_t>(),
                              st));
     coo_content = content;
     return CFPQ_OK;
@@ -571,14 +574,15 @@ int QueryDev::refresh_graph_caches(Allocator *A, cudaStream_t st, std::string *e
         need_term_bits |= (sdesc.dense && sdesc.label_kind == 0);
         need_nonempty |= sdesc.pure_rb != 0;
     }
-    const void *p_ne = g->nonempty.p, *p_tb = g->term_bits.p, *p_coo = g->coo.p;
+    const void *p_ne = g->nonempty.p, *p_tb = g->term_bits.p, *p_coo = g->col.p;
     if (n_slice_groups)
         if (int rc = g->ensure_coo(A, st, err)) return rc;
     if (need_nonempty)
         if (int rc = g->ensure_nonempty(A, st, err)) return rc;
     if (need_term_bits)
         if (int rc = g->ensure_term_bits(A, st, err)) return rc;
-    *moved = (n_slice_groups && g->coo.p != p_coo) || (need_nonempty && g->nonempty.p != p_ne) || (need_term_bits && g->term_bits.p != p_tb);
+    *moved = (n_slice_groups && g->col.p != p_coo) || (need_nonempty && g->nonempty.p != p_ne) ||
+             (need_term_bits && g->term_bits.p != p_tb);
     return CFPQ_OK;
 }
 
@@ -801,7 +805,7 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
                         if (rb >= 0 && member_of[(size_t)rb] >= 0) hs[j].slice_mem = (uint32_t)member_of[(size_t)rb];
                     }
                 for (uint32_t w = 0; w < q.W; ++w) hsi.push_back(SliceItem{(uint32_t)hsg.size(), w});
-                hsg.push_back(SliceGroup{cp, g.coo.as<uint32_t>(), L, q.n, q.W, mem0, nmem, 0u});
+                hsg.push_back(SliceGroup{cp, g.coo(), L, q.n, q.W, mem0, nmem, 0u});
                 slice_smem = std::max(slice_smem, nmem * q.n * 9u);
             }
             for (size_t b = 0; b < q.blocks.size(); ++b) {

@@ -197,8 +197,10 @@ struct GraphDev {
     DBuf nonempty;  // [n_term * W] bit y of label l: row (l, y) of the CSR has an edge (pure-terminal reads)
     uint64_t nonempty_content = ~0ull;
     int ensure_nonempty(Allocator *A, cudaStream_t st, std::string *err);
-    DBuf coo;  // [m] edges as x << 16 | y (column slices)
+    // [m] edges as x << 16 | y (column slices), in the staging's edge copy `col`, which
+    // is done with then: a list of its own would take 4 bytes an edge more
     uint64_t coo_content = ~0ull;
+    const uint32_t *coo() const { return col.as<uint32_t>(); }
     int ensure_coo(Allocator *A, cudaStream_t st, std::string *err);
     // staging scratch
     DBuf e_src, e_lbl, e_dst, cnt, off, col, ucnt, scan_tmp, label_map, err;

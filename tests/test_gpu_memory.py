@@ -1,0 +1,89 @@
+"""Device memory at its limits: what a run needs, and what a context does after a call
+that ran out of memory.  The allocator callbacks count the bytes held and can refuse."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from paper_2103_14688_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+T = W.TERM
+
+
+@pytest.fixture(scope="module")
+def C():
+    from paper_2103_14688_gb300 import cfpq
+    cfpq.load()
+    return cfpq
+
+
+class Memory:
+    """Allocator callbacks over torch's allocator: bytes held, their peak, and a rule that refuses requests."""
+
+    def __init__(self, C):
+        import torch
+        torch.cuda.init()
+        self.held = self.peak = self.calls = 0
+        self.refuse = lambda call, nbytes: False
+
+        def alloc(nbytes, stream, user):
+            self.calls += 1
+            if self.refuse(self.calls, nbytes):
+                return None
+            try:
+                p = torch.cuda.caching_allocator_alloc(int(nbytes), 0, stream or 0)
+            except Exception:
+                return None
+            self.held += nbytes
+            self.peak = max(self.peak, self.held)
+            return p
+
+        def free(ptr, nbytes, stream, user):
+            torch.cuda.caching_allocator_delete(ptr)
+            self.held -= nbytes
+
+        self.options = {"alloc": C.cfpq_alloc_fn(alloc), "free": C.cfpq_free_fn(free)}
+
+    def context(self, C, **opts):
+        import torch
+        return C.Context(use_torch=False, stream=torch.cuda.current_stream().cuda_stream, **self.options, **opts)
+
+
+def _plus():
+    return W.make_rsm(2, [0], [0, 0], [1], [(0, T, 0, 1), (1, T, 0, 1)])
+
+
+def _dense(n, m, seed):
+    rng = np.random.Generator(np.random.PCG64(seed))
+    return W.Graph(n, 3, rng.integers(0, n, m, dtype=np.uint32), rng.integers(0, 3, m, dtype=np.uint32),
+                   rng.integers(0, n, m, dtype=np.uint32))
+
+
+def _run(ctx, g, r):
+    ctx.load_graph(g)
+    ctx.load_rsm(r)
+    ctx.run()
+    return [ctx.reachable_words(b) for b in range(r.n_boxes)]
+
+
+def test_column_slices_need_no_memory_per_edge(C):
+    """A run with column slices fits where the row gather's run of the same query does (its round cap is never
+    reached), up to the work lists (1 MiB here); an edge list of its own would be 4 MiB."""
+    g, r = _dense(1500, 1 << 20, 1), _plus()
+    mem = Memory(C)
+    with mem.context(C, max_rounds=1 << 19) as ctx:
+        want = _run(ctx, g, r)
+    with Memory(C).context(C, memory_budget=mem.peak + (1 << 20)) as ctx:
+        for _ in range(2):  # (the second load overwrites the edge copy that holds the first one's list)
+            assert (_run(ctx, g, r)[0] == want[0]).all()
+    g2 = _dense(1500, 9000, 2)
+    with mem.context(C, max_rounds=1 << 19) as ctx:
+        want2 = _run(ctx, g2, r)
+    with mem.context(C) as ctx:
+        for a, w in ((g, want), (g2, want2), (g, want)):
+            assert (_run(ctx, a, r)[0] == w[0]).all()
+        bad = W.Graph(g.n, g.n_terminals, g.src, g.lbl, np.where(np.arange(g.m) == g.m - 1, g.n, g.dst).astype(np.uint32))
+        with pytest.raises(C.CfpqError):  # a load that is refused has overwritten the edge copy too
+            ctx.load_graph(bad)
+        assert (_run(ctx, g2, r)[0] == want2[0]).all()

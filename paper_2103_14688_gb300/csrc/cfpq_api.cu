@@ -212,11 +212,15 @@ int ensure_query(cfpq_ctx *ctx, bool restricted = false) {
         // loaded since, so rebuild what was derived from the old edges.
         std::string e;
         bool moved = false;
+        ctx->exec_dirty = true;  // (also when it fails: a buffer may have moved before)
         if (int rc = q.refresh_graph_caches(&ctx->A, ctx->stream, &e, &moved)) return fail(ctx, rc, e);
-        if (moved) ctx->exec_dirty = true;
+        ctx->exec_dirty = moved;
     }
     if (!q.prepared || q.graph_generation != ctx->graph.generation || ctx->exec_dirty) {
         std::string e;
+        // until all of it is done: after a failure the work lists and the captured
+        // loop still hold buffers of the plan before, some of them freed
+        ctx->exec_dirty = true;
         int rc = q.prepare(&ctx->A, &e);
         if (rc) return fail(ctx, rc, e);
         if (restricted && !q.reach_mem.ensure(&ctx->A, (size_t)q.Q * q.W * 8, &e))

@@ -87,3 +87,55 @@ def test_column_slices_need_no_memory_per_edge(C):
         with pytest.raises(C.CfpqError):  # a load that is refused has overwritten the edge copy too
             ctx.load_graph(bad)
         assert (_run(ctx, g2, r)[0] == want2[0]).all()
+
+
+def _refused_runs(C, first, r, call, opts):
+    """For every allocation that `call` makes on a context that ran `first`: refuse it alone, let `call` fail, and yield
+    the context, its memory and whether it failed; ends after the first call that needed no more allocations."""
+    for k in range(1, 200):
+        mem = Memory(C)
+        with mem.context(C, **opts) as ctx:
+            _run(ctx, first, r)
+            stop = [None]
+            try:
+                call(ctx, mem, lambda: (stop.__setitem__(0, mem.calls + k),
+                                        setattr(mem, "refuse", lambda i, b: i == stop[0])))
+                failed = False
+            except C.CfpqError as e:
+                assert e.status == C.CFPQ_ERR_OUT_OF_MEMORY
+                failed = True
+            refused = mem.calls >= stop[0]
+            mem.refuse = lambda i, b: False
+            yield ctx, failed
+        if not refused:
+            return
+    assert False, "more allocations than expected"
+
+
+RUNS = [("column slices", lambda: (_dense(700, 1500, 3), _dense(1900, 60000, 4), _plus()), {"no_single_cta": 1}),
+        ("single CTA", lambda: (_dense(60, 100, 5), _dense(200, 400, 6), _plus()), {}),
+        ("tiles", lambda: (W.dyck_zipf(2100, seed=1)[0], W.dyck_zipf(2600, seed=2)[0], W.dyck_rsm(2)), {"no_autotune": 1})]
+
+
+@pytest.mark.parametrize("name,make,opts", RUNS, ids=[x[0] for x in RUNS])
+def test_run_again_after_a_run_out_of_memory(C, name, make, opts):
+    """A run of a larger graph whose k-th allocation is refused fails; the same run again gives the graph's answer,
+    and so does the smaller graph afterwards."""
+    first, then, r = make()
+    with C.Context(**opts) as ctx:
+        want = [_run(ctx, g, r) for g in (first, then)]
+
+    def call(ctx, mem, refuse_from_here):
+        ctx.load_graph(then)
+        refuse_from_here()
+        ctx.run()
+
+    fails = 0
+    for ctx, failed in _refused_runs(C, first, r, call, opts):
+        fails += failed
+        ctx.run()
+        assert all((ctx.reachable_words(b) == want[1][b]).all() for b in range(r.n_boxes))
+        ctx.load_graph(first)
+        ctx.run()
+        assert all((ctx.reachable_words(b) == want[0][b]).all() for b in range(r.n_boxes))
+    assert fails >= 5

@@ -232,8 +232,10 @@ int stage_graph(GraphDev *g, Allocator *A, cudaStream_t st, uint32_t n, uint32_t
     const size_t rows = (size_t)n_term * n;
     if (rows + 1 >= 0xffffffffull) { *err = "n_vertices * n_terminals too large"; return CFPQ_ERR_UNSUPPORTED; }
     const size_t mm = m ? m : 1;
-    const bool realloc = !(g->csr_off.p && g->csr_off.bytes >= (rows + 1) * 4 && g->csr_col.bytes >= mm * 4 &&
-                           g->col.bytes >= mm * 4);
+    // (kept over a load that fails: the next one may find every buffer large enough,
+    // but plans hold the old ones and the label map is not filled)
+    g->moved |= !(g->csr_off.p && g->csr_off.bytes >= (rows + 1) * 4 && g->csr_col.bytes >= mm * 4 &&
+                  g->col.bytes >= mm * 4 && g->label_map.bytes >= (size_t)n_term * 4);
     g->coo_content = ~0ull;  // (col is overwritten)
     const size_t nb = (rows + 4095) / 4096 + 2;
     if (!g->csr_off.ensure(A, (rows + 1) * 4, err) || !g->csr_col.ensure(A, mm * 4, err) ||
@@ -252,7 +254,7 @@ int stage_graph(GraphDev *g, Allocator *A, cudaStream_t st, uint32_t n, uint32_t
         l = g->e_lbl.as<uint32_t>();
         d = g->e_dst.as<uint32_t>();
     }
-    if (g->n_term != n_term || realloc) {
+    if (g->n_term != n_term || g->moved) {
         std::vector<int32_t> lm(n_term);
         for (uint32_t i = 0; i < n_term; ++i) lm[i] = (int32_t)i;
         ENG_CK(cudaMemcpyAsync(g->label_map.p, lm.data(), n_term * 4, cudaMemcpyHostToDevice, st));
@@ -284,7 +286,8 @@ int stage_graph(GraphDev *g, Allocator *A, cudaStream_t st, uint32_t n, uint32_t
         g->n = 0;
         return CFPQ_ERR_INVALID_ARG;
     }
-    if (realloc || g->n != n || g->n_term != n_term) g->generation += 1;
+    if (g->moved || g->n != n || g->n_term != n_term) g->generation += 1;
+    g->moved = false;
     g->content += 1;
     g->n = n;
     g->n_pad = n_pad;

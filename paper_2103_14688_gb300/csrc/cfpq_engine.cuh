@@ -213,6 +213,7 @@ struct GraphDev {
     // also a same-size one: everything derived from the edges is stale then.
     uint64_t generation = 0;
     uint64_t content = 0;
+    bool moved = false;  // a staging buffer was reallocated and no load has succeeded with it yet
 };
 
 // Device state and descriptors of one query (graph + RSM).

@@ -137,7 +137,7 @@ extern "C" int cfpq_load_graph_device_noalloc(cfpq_ctx *ctx, uint32_t n, uint32_
             g.n = 0;
             return fail(CFPQ_ERR_INVALID_ARG, "an edge names a vertex >= n_vertices or a label >= n_terminals");
         }
-        if (g.n != n || g.n_term != n_term) g.generation += 1;
+        if (g.moved || g.n != n || g.n_term != n_term) g.generation += 1;
         g.content += 1;  // the row bitmaps derived from the old edges are stale
         g.n = n;
         g.n_pad = n_pad;

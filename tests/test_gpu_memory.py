@@ -139,3 +139,27 @@ def test_run_again_after_a_run_out_of_memory(C, name, make, opts):
         ctx.run()
         assert all((ctx.reachable_words(b) == want[0][b]).all() for b in range(r.n_boxes))
     assert fails >= 5
+
+
+@pytest.mark.parametrize("after", ["the first graph", "the refused graph"])
+@pytest.mark.parametrize("name,make,opts", RUNS[:2], ids=[x[0] for x in RUNS[:2]])
+def test_load_again_after_a_load_out_of_memory(C, name, make, opts, after):
+    """A load of a larger graph with more labels whose k-th allocation is refused fails; the graph loaded next is
+    staged and run as in a new context, also when it has the shape of the one before the failure."""
+    first, then, r = make()
+    first, then = (W.Graph(g.n, k, g.src, g.lbl, g.dst) for g, k in ((first, 3), (then, 9)))
+    g = first if after == "the first graph" else then
+    with C.Context(**opts) as ctx:
+        want = _run(ctx, g, r)
+
+    def call(ctx, mem, refuse_from_here):
+        refuse_from_here()
+        ctx.load_graph(then)
+
+    fails = 0
+    for ctx, failed in _refused_runs(C, first, r, call, opts):
+        fails += failed
+        ctx.load_graph(g)
+        ctx.run()
+        assert all((ctx.reachable_words(b) == want[b]).all() for b in range(r.n_boxes))
+    assert fails >= 5

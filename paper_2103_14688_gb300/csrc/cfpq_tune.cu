@@ -166,12 +166,12 @@ double read_gbs(Allocator &A, cudaStream_t st, int dev, size_t bytes, uint32_t r
     return best;
 }
 
-// Rate of a tile kernel (TFLOP/s): one dense product of two n x n 0/1
-// matrices, operands already expanded, best of 3 launches after an untimed
-// one; 0 on error.  (Not taken from the probe query: its products keep only
+// Rate of a tile kernel (TFLOP/s, in *tflops): one dense product of two n x n
+// 0/1 matrices, operands already expanded, best of 3 launches after an untimed
+// one; returns a CFPQ status.  (Not taken from the probe query: its products keep only
 // the rows that can change and are too small to show a kernel's rate -- they
 // put the FP8 kernel first, at half the E2M1 kernels' rate on a large product.)
-double tile_rate(Allocator &A, cudaStream_t st, uint32_t kind) {
+int tile_rate(Allocator &A, cudaStream_t st, uint32_t kind, double *tflops) {
     constexpr uint32_t n = kProbeN, W = n / 64u;
     const bool fp4 = tile_kind_fp4(kind);
     const uint32_t kstride = fp4 ? n / 2u : n;
@@ -184,10 +184,11 @@ double tile_rate(Allocator &A, cudaStream_t st, uint32_t kind) {
         int err_flag;
     };
     DBuf head, out, xs, a8, b8;
-    if (tc_map_bytes() != 128 || !head.ensure(&A, sizeof(Head), &err) || !out.ensure(&A, (size_t)n * W * 8, &err) ||
+    if (tc_map_bytes() != 128) return CFPQ_ERR_CUDA;
+    if (!head.ensure(&A, sizeof(Head), &err) || !out.ensure(&A, (size_t)n * W * 8, &err) ||
         !xs.ensure(&A, (size_t)n * 4, &err) || !a8.ensure(&A, (size_t)n * kstride, &err) ||
         !b8.ensure(&A, (size_t)n * kstride, &err))
-        return 0;
+        return CFPQ_ERR_OUT_OF_MEMORY;
     std::vector<uint32_t> ids(n);
     for (uint32_t i = 0; i < n; ++i) ids[i] = i;
     alignas(64) Head h;
@@ -245,7 +246,8 @@ double tile_rate(Allocator &A, cudaStream_t st, uint32_t kind) {
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     cudaGetLastError();
-    return best;
+    *tflops = best;
+    return best > 0 ? CFPQ_OK : CFPQ_ERR_CUDA;
 }
 
 uint32_t ratio_for(double tflops, double gather_gbs) {
@@ -295,8 +297,7 @@ Tuning run_probe(const cfpq_options &like, cudaStream_t st) {
         A.free = like.free;
         A.user = like.alloc_user;
         A.stream = st;
-        t.tflops[k] = tile_rate(A, st, k);
-        if (t.tflops[k] <= 0) rc = CFPQ_ERR_CUDA;
+        rc = tile_rate(A, st, k, &t.tflops[k]);
     }
     t.probe_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     t.status = rc;

@@ -163,3 +163,16 @@ def test_load_again_after_a_load_out_of_memory(C, name, make, opts, after):
         ctx.run()
         assert all((ctx.reachable_words(b) == want[b]).all() for b in range(r.n_boxes))
     assert fails >= 5
+
+
+def test_tuning_reports_out_of_memory(C):
+    """The autotuner's product of two 8192 x 8192 matrices takes 64 MiB of FP8 bytes a side: without them it keeps the
+    built-in choices and says why."""
+    mem = Memory(C)
+    mem.refuse = lambda i, b: b == 64 << 20
+    with mem.context(C) as ctx:
+        t = ctx.tune(force=True)
+    assert t.tuned == 0 and t.probe_status == C.CFPQ_ERR_OUT_OF_MEMORY
+    assert t.gather_gbs > 0  # (the probe query before it ran)
+    with C.Context() as ctx:
+        assert ctx.tune(force=True).tuned == 1

@@ -452,7 +452,7 @@ int cfpq_release(cfpq_server *srv, uint64_t ticket);
  * cfpq_get_closure_rows and cfpq_count_index describe those columns only.
  *
  * Errors: CFPQ_ERR_STATE (no graph/RSM, a start answer set, step/apply
- * without begin), CFPQ_ERR_INVALID_ARG (columns, NULL buffers),
+ * without begin, or after a graph was loaded since), CFPQ_ERR_INVALID_ARG (columns, NULL buffers),
  * CFPQ_ERR_TIMEOUT (a cap of cfpq_options stopped the loop), CFPQ_ERR_CUDA. */
 int cfpq_shard_begin(cfpq_ctx *ctx, uint32_t col0, uint32_t col1);
 

@@ -325,6 +325,7 @@ static int load_graph_impl(cfpq_ctx *ctx, uint32_t n, uint32_t nt, size_t m, con
     if (int rc = set_device(ctx)) return rc;
     ctx->has_result = false;
     ++ctx->result_gen;
+    ctx->shard_on = false;  // (its passes would read the buffers staged into here)
     std::string e;
     int rc = stage_graph(&ctx->graph, &ctx->A, ctx->stream, n, nt, m, s, l, d, dev, &e);
     if (rc) {

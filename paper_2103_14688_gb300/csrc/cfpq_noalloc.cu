@@ -110,6 +110,7 @@ extern "C" int cfpq_load_graph_device_noalloc(cfpq_ctx *ctx, uint32_t n, uint32_
         const cudaStream_t st = ctx->stream;
         ctx->has_result = false;
         ++ctx->result_gen;
+        ctx->shard_on = false;  // (its passes would read the buffers staged into here)
         ctx->has_graph = false;
 #define NA_CK(call)                                                                                 \
     do {                                                                                            \

@@ -146,14 +146,20 @@ typedef struct {
 /* Statistics of one cfpq_run (or one query of a batch). */
 typedef struct {
     uint32_t iterations;       /* loop iterations, counting the last one that adds no edge */
-    uint32_t rounds;           /* closure passes over all blocks, all iterations */
+    uint32_t rounds;           /* closure passes over all blocks, all iterations (a level closed in
+                                  column slices takes one) */
     uint32_t status;           /* 0, or the CFPQ_ERR_* that stopped the loop */
     uint32_t gpu_launches;     /* kernels launched by the call (graph nodes executed) */
     uint64_t edges_added;      /* nonterminal edges found, epsilon edges included */
     uint64_t closure_bits;     /* nnz(C3) at the fixpoint (counted on request, else 0) */
     uint64_t m3_bits;          /* nnz(M3) at the fixpoint (counted on request, else 0) */
-    uint64_t row_ors;          /* bit-packed source-row ORs issued by the closure */
-    uint64_t rows_changed;     /* output rows of C3 changed, summed over passes */
+    uint64_t row_ors;          /* bit-packed source-row ORs issued by the closure.  Column slices
+                                  (cyclic components of RSM states whose transitions all read
+                                  terminals; not with max_rounds) OR 64-bit words of rows: a
+                                  row's worth of them, rounded up per slice, counts as one.  Reads
+                                  of rows that are expanded from the graph's edges do not count */
+    uint64_t rows_changed;     /* output rows of C3 changed, summed over passes (column slices:
+                                  words changed, a row's worth as one) */
     uint64_t row_bytes;        /* bytes of one bit-packed row (n rounded up to 128 bits, / 8) */
     uint64_t tile_mmas;        /* dense tensor-core tile products issued */
     uint64_t closure_blocks;   /* n x n state blocks of C3 held on the device */
@@ -168,7 +174,8 @@ typedef struct {
                                   128 x 256 x 128 tensor-core multiply-adds */
     /* profile = 1: the closure time of ms_closure split by kernel, from CUDA
      * events on the context's stream around each group of launches of a pass */
-    double ms_gather;          /* row-gather launches (k_gather, every row-width class) */
+    double ms_gather;          /* row-kernel launches: gathers of every row width, expanded
+                                  blocks, column slices */
     double ms_tile_operands;   /* tile jobs' dirty-row lists and 0/1 FP8 operand expansion */
     double ms_tile_products;   /* tcgen05 tile-product launches */
     uint32_t gather_launches;  /* row-gather launches timed */
@@ -286,9 +293,9 @@ int cfpq_set_start(cfpq_ctx *ctx, const uint64_t *bits, uint32_t n_boxes, uint32
  * device it runs a probe query -- Dyck-4 (S -> S S | o_i c_i | o_i S c_i)
  * on a seeded graph of 8192 vertices with Zipf(2.1) out-degrees (mean
  * about 3), 8 labels --
- * with the bit-packed closure and with each tile kernel, times their kernel
- * groups with CUDA events, times reads of an L2-sized and an HBM-sized
- * buffer, and derives: the fastest tile kernel (AUTO's default) and the
+ * with the bit-packed closure and times its kernel groups with CUDA events,
+ * times a dense product of two 8192 x 8192 0/1 matrices in each tile kernel and
+ * reads of an L2-sized and an HBM-sized buffer, and derives: the fastest tile kernel (AUTO's default) and the
  * cost-model ratio (new-edge tiles run while M * K < ratio x new edges),
  * searched around tile rate / (16 x gather rate) -- one new edge costs the
  * gather n/8 bytes, a tile product 2n multiply-adds per (row, column) of its
@@ -452,8 +459,9 @@ int cfpq_release(cfpq_server *srv, uint64_t ticket);
  * cfpq_get_closure_rows and cfpq_count_index describe those columns only.
  *
  * Errors: CFPQ_ERR_STATE (no graph/RSM, a start answer set, step/apply
- * without begin, or after a graph was loaded since), CFPQ_ERR_INVALID_ARG (columns, NULL buffers),
- * CFPQ_ERR_TIMEOUT (a cap of cfpq_options stopped the loop), CFPQ_ERR_CUDA. */
+ * without begin, or after a graph was loaded since), CFPQ_ERR_INVALID_ARG
+ * (columns, NULL buffers), CFPQ_ERR_TIMEOUT (a cap of cfpq_options stopped
+ * the loop), CFPQ_ERR_CUDA. */
 int cfpq_shard_begin(cfpq_ctx *ctx, uint32_t col0, uint32_t col1);
 
 /* Run one iteration (closure passes and extraction) on the rank's columns and

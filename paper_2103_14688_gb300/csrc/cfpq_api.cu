@@ -111,7 +111,8 @@ int run_executor(cfpq_ctx *ctx, Executor &ex, std::vector<QCtl> *ctls, uint32_t 
     for (uint32_t k : ex.n_items) n_gather += k ? 1 : 0;
     for (uint32_t k : ex.n_xitems) n_extract += k ? 1 : 0;
     // tile jobs: new-edge columns, row list, A and B operands, the product kernel (two with uncompacted jobs)
-    const uint32_t per_pass = n_gather + n_extract + (ex.n_tcjobs ? (ex.any_uncompacted ? 6 : 5) : 0) + (n_extract ? 0 : 1);
+    const uint32_t per_tiles = ex.n_tcjobs ? (ex.any_uncompacted ? 6 : 5) : 0;
+    const uint32_t per_pass = n_gather + n_extract + per_tiles + (n_extract ? 0 : 1);
     if (ctx->opt.loop_mode == CFPQ_LOOP_HOST) {
         if (ex.enqueue_prologue(st, mi, mr, mp)) return fail(ctx, CFPQ_ERR_CUDA, "prologue launch failed");
         int running = 1;

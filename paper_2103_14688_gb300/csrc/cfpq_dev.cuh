@@ -116,10 +116,10 @@ struct SrcDesc {
     const uint32_t *pure_col;
     const uint64_t *pure_mask[2];  // per label: bit y set iff y has an edge of it (W words)
     // Tile source with a product job for the iteration's new edges
-    // (TcJob::covers_new): when that job runs in this pass (new_tiles_pay on its counts: tc_kcount, tagged with the pass, at
-    // most tc_kcap rows; tc_mcount; tc_ecount), the row gather leaves the new
-    // edges' row ORs to the tiles and keeps only the product edges
-    // themselves (ident).
+    // (TcJob::covers_new): when that job runs in this pass (new_tiles_pay on
+    // its counts: tc_kcount, tagged with the pass, at most tc_kcap rows;
+    // tc_mcount; tc_ecount), the row gather leaves the new edges' row ORs to
+    // the tiles and keeps only the product edges themselves (ident).
     uint32_t tile_new;
     uint32_t tc_kcap;
     uint32_t tc_ratio;         // new_tiles_pay's ratio for the job's tile format

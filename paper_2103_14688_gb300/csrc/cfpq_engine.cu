@@ -458,7 +458,8 @@ int QueryDev::plan(std::string *err) {
         }
         loop_mask = 0;
         for (size_t b = 0; b < blocks.size(); ++b)
-            if (reach[(size_t)blocks[b].first * Q + blocks[b].first] && blk_slice[b] < 0) loop_mask |= 1ull << blk_level[b];
+            if (reach[(size_t)blocks[b].first * Q + blocks[b].first] && blk_slice[b] < 0)
+                loop_mask |= 1ull << blk_level[b];
     }
     // Boxes read by some transition (bit 63: a box >= 63 is read).
     nt_read_mask = 0;
@@ -769,9 +770,10 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
         // Small graphs: items of that size would leave SMs without work (47
         // items of 64 rows for a block at n = 3001, each warp on eight rows in turn:
         // 27 us a pass; with items of 8 rows Dyck-4 went from 3.64 to 3.40 ms), so
-        // `blocks` blocks of a level are cut into four CTAs an SM's worth of items, a
-        // row per group at the least.  Not on levels that repeat: fewer, larger items see more of the rows that
-        // changed earlier in the same pass, which saves passes.
+        // `blocks` blocks of a level are cut into four CTAs' worth of items for each of
+        // the 152 SMs, a row per group at the least.  Not on levels that repeat: fewer,
+        // larger items see more of the rows that changed earlier in the same pass,
+        // which saves passes.
         auto rows_for = [&](uint32_t blocks, bool repeats) -> uint32_t {
             if (item_scale > 1u || repeats || blocks == 0u) return rpi;
             const uint64_t want = (uint64_t)q.n * blocks * nq / (4u * 152u);
@@ -854,8 +856,9 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
                 // multiple-source runs are few and far between: 1024-row items
                 const uint32_t rows_item =
                     q.restricted ? 1024u
-                    : (has_nt && !expand && q.W >= 256u) ? std::min<uint32_t>(1024u, std::max<uint32_t>(rpi, 128u * item_scale))
-                                                         : rpl;
+                    : (has_nt && !expand && q.W >= 256u)
+                        ? std::min<uint32_t>(1024u, std::max<uint32_t>(rpi, 128u * item_scale))
+                        : rpl;
                 // the gather lists an item's rows in 1024 entries of shared memory
                 if (rows_item == 0u || rows_item > 1024u) {
                     *err = "gather items: at most 1024 rows per item";

@@ -246,13 +246,16 @@ __device__ __forceinline__ bool row_has_work(const SrcDesc &d, uint32_t chans, u
 // variant (nonterminal adjacency rows, pure-terminal blocks); without it the
 // kernel holds only the CSR paths, which keeps its registers for the rows.
 // --------------------------------------------------------------------------
-// Occupancy target per row width: narrow rows keep 4 CTAs (32 warps) per SM.
+// Occupancy target per row width: narrow rows keep 4 CTAs (32 warps) per SM, for
+// which the general variants of widths 1 and 2 spill 184 and 248 bytes and the CSR
+// ones 68 and 116.
 template <int VPL>
 struct GatherOcc {
     static constexpr int value = VPL <= 2 ? 4 : (VPL == 4 ? 2 : 1);
 };
 // CSR variant of wide rows: one source row in registers beside the output row
-// leaves room for two CTAs (it was one CTA with two source rows in flight).
+// leaves room for two CTAs (it was one CTA with two source rows in flight); at
+// width 16 it spills 112 bytes.
 template <int VPL, bool NT>
 struct GatherCtas {
     static constexpr int value = !NT && VPL >= 8 ? 2 : GatherOcc<VPL>::value;
@@ -808,7 +811,11 @@ __global__ void __launch_bounds__(256, GatherCtas<VPL, NT>::value)
 // 8 warps per SM beside the closure-row ring) this took 110 of the 190 ms of
 // gather of Dyck-4 at n = 65536; the query went from 303 to 233 ms.
 // --------------------------------------------------------------------------
-constexpr int kExpandOcc = 6;  // CTAs per SM (40 registers a thread; 32 would spill)
+// CTAs per SM.  48 warps leave 40 registers a thread, where the wide and the narrow
+// variant spill 44 and 48 bytes (the heaviest launch of Dyck-4 at n = 16384, 0.24 ms:
+// 1.35 million spill instructions of warps, 67% of warps active).  Fewer CTAs without
+// spills have not been timed.
+constexpr int kExpandOcc = 6;
 constexpr uint32_t kExpandParts = 4;
 template <bool WIDE>
 __global__ void __launch_bounds__(256, kExpandOcc)
@@ -1341,7 +1348,8 @@ __global__ void __launch_bounds__(256) k_extract(const XItem *__restrict__ items
     __syncthreads();
     }
     if (FC.enabled) {
-        for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < FC.zero_words; i += (size_t)gridDim.x * blockDim.x)
+        for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < FC.zero_words;
+             i += (size_t)gridDim.x * blockDim.x)
             FC.zero[i] = 0ull;
         // Control rewrites what every CTA of this launch reads (x_total, the live
         // lists, the queries' state), so the CTA that finishes last runs it, in a pass
@@ -1446,7 +1454,7 @@ __device__ __forceinline__ void advance_query(QCtl &c) {
 // state is read once, changed in registers and written twice; a single query's
 // lists are written by one thread a class, without the scans over queries.
 // (extraction and control, Dyck-4 n = 3001, average over its passes with cold caches:
-// 16.3 -> 10.9 us.)
+// 16.3 -> 10.3 us.)
 __device__ void control_body(QCtl *const *ctls, uint32_t nq, QCtl *mirror, cudaGraphConditionalHandle handle,
                              int use_handle, int *running_out, const ExecTables &T, int advance) {
     constexpr int K = kClasses + kXClasses + 1;

@@ -781,6 +781,17 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
             while (rows > rows_per_step && rows > want) rows >>= 1;
             return rows;
         };
+        // Multiple-source runs: how many rows are reached is known only on the device,
+        // often few of many, so items grow (to 1024 rows) while a level keeps four
+        // CTAs' worth of them for each of the 152 SMs.  (ab)*c|a*b*, items of 1024 rows at
+        // any n -> these: n = 2000, 6 edges a vertex 4.0 -> 2.1 ms, n = 8192, 8 edges 7.0 ->
+        // 2.7, n = 20000, 6 edges 13.9 -> 7.7; few rows reached at n = 65536, 2 edges: 0.9
+        // either way, and 1.06 with the usual items.
+        auto rows_restricted = [&](uint32_t blocks) -> uint32_t {
+            uint32_t rows = rpi;
+            while (rows < 1024u && (uint64_t)q.n * blocks / (2u * rows) >= 4u * 152u) rows <<= 1;
+            return rows;
+        };
         // product jobs: tcgen05 tiles of 128 rows x 256 columns
         const uint32_t tiles_m = (q.n + 127u) / 128u, tiles_n = (q.n + 255u) / 256u;
         for (uint32_t L = 0; L <= q.n_levels; ++L) {
@@ -852,10 +863,9 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
                 uint32_t n_slices = sliceable ? 4u : 1u;
                 if (q.gather_slices) n_slices = sliceable ? std::min<uint32_t>(q.gather_slices, 16u) : 1u;
                 // nonterminal blocks of wide rows: 128-row items (measured on
-                // Dyck-4; the CSR blocks of the RPQ bench prefer 64); rows of
-                // multiple-source runs are few and far between: 1024-row items
+                // Dyck-4; the CSR blocks of the RPQ bench prefer 64)
                 const uint32_t rows_item =
-                    q.restricted ? 1024u
+                    q.restricted ? rows_restricted(lvl_blocks)
                     : (has_nt && !expand && q.W >= 256u)
                         ? std::min<uint32_t>(1024u, std::max<uint32_t>(rpi, 128u * item_scale))
                         : rpl;

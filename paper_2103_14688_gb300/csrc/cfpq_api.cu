@@ -215,7 +215,7 @@ int ensure_query(cfpq_ctx *ctx, bool restricted = false) {
         bool moved = false;
         ctx->exec_dirty = true;  // (also when it fails: a buffer may have moved before)
         if (int rc = q.refresh_graph_caches(&ctx->A, ctx->stream, &e, &moved)) return fail(ctx, rc, e);
-        ctx->exec_dirty = moved;
+        ctx->exec_dirty = moved || q.slice_choices_stale();
     }
     if (!q.prepared || q.graph_generation != ctx->graph.generation || ctx->exec_dirty) {
         std::string e;
@@ -968,6 +968,7 @@ extern "C" int cfpq_batch_run(cfpq_ctx *ctx, uint32_t n_queries, const cfpq_quer
         set_tiles(*q, ctx->opt, ctx->stream, max_n);
         q->gather_slices = ctx->opt.gather_slices;
         q->use_slices = ctx->opt.max_rounds == 0;
+        q->shares_device = n_queries > 1;
         rc = copy_rsm(qq.rsm, &q->rsm, &e);
         if (rc) return fail(ctx, rc, "query " + std::to_string(i) + ": " + e);
         q->g = g.get();

@@ -241,7 +241,8 @@ int stage_graph(GraphDev *g, Allocator *A, cudaStream_t st, uint32_t n, uint32_t
     if (!g->csr_off.ensure(A, (rows + 1) * 4, err) || !g->csr_col.ensure(A, mm * 4, err) ||
         !g->cnt.ensure(A, rows * 4, err) || !g->off.ensure(A, (rows + 1) * 4, err) || !g->col.ensure(A, mm * 4, err) ||
         !g->ucnt.ensure(A, rows * 4, err) || !g->scan_tmp.ensure(A, nb * 4, err) ||
-        !g->label_map.ensure(A, (size_t)n_term * 4, err) || !g->err.ensure(A, 16, err))
+        !g->label_map.ensure(A, (size_t)n_term * 4, err) ||
+        !g->err.ensure(A, (2 + GraphDev::kCountedLabels) * 4, err))
         return CFPQ_ERR_OUT_OF_MEMORY;
     const uint32_t *s = src, *l = lbl, *d = dst;
     if (!device_ptrs && m) {
@@ -262,25 +263,27 @@ int stage_graph(GraphDev *g, Allocator *A, cudaStream_t st, uint32_t n, uint32_t
     }
     uint32_t *cnt = g->cnt.as<uint32_t>(), *off = g->off.as<uint32_t>(), *col = g->col.as<uint32_t>();
     uint32_t *ucnt = g->ucnt.as<uint32_t>(), *tmp = g->scan_tmp.as<uint32_t>();
-    int *errf = g->err.as<int>();
+    uint32_t *res = g->err.as<uint32_t>();
+    const uint32_t counted = g->counted_labels(n_term);
     if (stage_small_bytes(n, n_term, m)) {
-        ENG_CK(launch_stage_small(s, l, d, m, n, n_term, g->csr_off.as<uint32_t>(), g->csr_col.as<uint32_t>(), errf, st));
+        ENG_CK(launch_stage_small(s, l, d, m, n, n_term, counted, g->csr_off.as<uint32_t>(), g->csr_col.as<uint32_t>(),
+                                  res, st));
     } else {
         ENG_CK(cudaMemsetAsync(cnt, 0, rows * 4, st));
-        ENG_CK(cudaMemsetAsync(errf, 0, 16, st));
-        ENG_CK(launch_stage_count(s, l, d, m, n, n_term, g->label_map.as<int32_t>(), cnt, errf, st));
+        ENG_CK(cudaMemsetAsync(res, 0, 16, st));
+        ENG_CK(launch_stage_count(s, l, d, m, n, n_term, g->label_map.as<int32_t>(), cnt, reinterpret_cast<int *>(res),
+                                  st));
         ENG_CK(scan_exclusive(cnt, off, rows, tmp, st));
         ENG_CK(cudaMemsetAsync(ucnt, 0, rows * 4, st));
         ENG_CK(launch_stage_fill(s, l, d, m, n, n_term, g->label_map.as<int32_t>(), off, ucnt, col, st));
         ENG_CK(launch_stage_unique(off, col, ucnt, rows, st));
         ENG_CK(scan_exclusive(ucnt, g->csr_off.as<uint32_t>(), rows, tmp, st));
-        ENG_CK(launch_stage_compact(off, col, g->csr_off.as<uint32_t>(), g->csr_col.as<uint32_t>(), rows,
-                                    reinterpret_cast<uint32_t *>(errf + 1), st));
+        ENG_CK(launch_stage_compact(off, col, g->csr_off.as<uint32_t>(), g->csr_col.as<uint32_t>(), rows, n, counted,
+                                    res, st));
     }
-    int result[2] = {0, 0};  // an edge out of range; edges kept
-    ENG_CK(cudaMemcpyAsync(result, errf, sizeof(result), cudaMemcpyDeviceToHost, st));
+    uint32_t result[2 + GraphDev::kCountedLabels];
+    ENG_CK(cudaMemcpyAsync(result, res, (2 + counted) * 4, cudaMemcpyDeviceToHost, st));
     ENG_CK(cudaStreamSynchronize(st));
-    const uint32_t total = (uint32_t)result[1];
     if (result[0]) {
         *err = "an edge names a vertex >= n_vertices or a label >= n_terminals";
         g->n = 0;
@@ -294,7 +297,7 @@ int stage_graph(GraphDev *g, Allocator *A, cudaStream_t st, uint32_t n, uint32_t
     g->W = W;
     g->n_term = n_term;
     g->m_in = m;
-    g->m_unique = total;
+    g->set_counts(result, n_term);
     g->host_valid = false;
     return CFPQ_OK;
 }
@@ -434,23 +437,28 @@ int QueryDev::plan(std::string *err) {
     // component's column word fits an SM.
     blk_slice.assign(blocks.size(), -1);
     n_slice_groups = 0;
+    slice_choices.clear();
     loop_mask = cyclic_mask;
     if (use_slices && !restricted && !closure_all_tiles(closure_mode)) {
         for (uint32_t c = 0; c < Q; ++c) {
             if (comp[c] != c || !reach[(size_t)c * Q + c]) continue;
-            uint32_t members = 0;
+            SliceChoice ch{0u, 0u, {}, false};
             bool ok = true;
             for (uint32_t s = 0; s < Q; ++s) {
                 if (comp[s] != c) continue;
-                ++members;
+                ++ch.members;
                 for (const auto &tr : rsm.tr) ok &= tr.from != s || tr.kind == 0;
             }
-            ok = ok && (uint64_t)members * n * 9u <= kSliceMaxBytes;
-            for (uint32_t t = 0; t < Q && ok; ++t) {
-                uint32_t same = 0;  // sources of the group's blocks that read its own blocks
-                for (const auto &tr : rsm.tr)
-                    same += (comp[tr.from] == c && comp[tr.to] == c) ? 1u : 0u;
-                if (same > kSliceMaxSrc || blk_of[(size_t)c * Q + t] < 0) continue;
+            if (!ok || (uint64_t)ch.members * n * 9u > kSliceMaxBytes) continue;
+            for (const auto &tr : rsm.tr)  // sources of a group's blocks that read its own blocks
+                if (comp[tr.from] == c && comp[tr.to] == c) ch.labels.push_back(tr.sym);
+            if (ch.labels.size() > kSliceMaxSrc) continue;
+            for (uint32_t t = 0; t < Q; ++t) ch.groups += blk_of[(size_t)c * Q + t] >= 0 ? 1u : 0u;
+            ch.sliced = slice_edges(ch) <= slice_edges_max(ch);
+            slice_choices.push_back(ch);
+            if (!ch.sliced) continue;
+            for (uint32_t t = 0; t < Q; ++t) {
+                if (blk_of[(size_t)c * Q + t] < 0) continue;
                 for (uint32_t s = 0; s < Q; ++s)
                     if (comp[s] == c) blk_slice[(size_t)blk_of[(size_t)s * Q + t]] = (int32_t)n_slice_groups;
                 ++n_slice_groups;
@@ -515,6 +523,35 @@ int QueryDev::plan(std::string *err) {
     n_eps = 0;
     for (uint32_t b = 0; b < B; ++b) n_eps += rsm.final_[rsm.box_start[b]] ? 1u : 0u;
     return CFPQ_OK;
+}
+
+// Edges a sweep of the component's slices visits, and up to how many slices beat the
+// row gather.  A slice visits every edge in every sweep while the gather reads only the
+// rows that changed, with all SMs and a launch's latency a pass: slices win where a row
+// has few edges, and on denser labels, whose paths are short, the gather does.
+// Measured on random graphs (run time, gather / slices): one wave of slices (a+) n = 4000,
+// 16 edges a row 1.16, 24 1.00, 32 0.83; n = 8192 1.17, 1.02, 0.88; more than the SMs
+// hold: a+ n = 15000, 3 edges 1.26, 4 1.03, 6 0.84; n = 22700, 4 edges 1.08, 6 0.96;
+// (ab)*c|a*b* n = 8192, 4 edges a row of (ab)* 1.26, 6 1.00, 8 0.82, 33 0.46.  Few edges in
+// all never lose: n = 2000, 48 K edges 1.15 (a+), 1.38 (three labels).
+uint64_t QueryDev::slice_edges(const SliceChoice &c) const {
+    uint64_t e = 0;
+    for (uint32_t l : c.labels) e += g->edges_of(l);
+    return e;
+}
+
+uint64_t QueryDev::slice_edges_max(const SliceChoice &c) const {
+    const bool one_wave = !shares_device && (uint64_t)c.groups * W <= 152u;
+    return std::max<uint64_t>(48u << 10, (uint64_t)c.members * n * (one_wave ? 24u : 5u));
+}
+
+// (with a margin, so that graphs near the limit do not set the query up again in turn)
+bool QueryDev::slice_choices_stale() const {
+    for (const auto &c : slice_choices) {
+        const uint64_t e = slice_edges(c), lim = slice_edges_max(c);
+        if (c.sliced ? e * 4u > lim * 5u : e * 5u < lim * 4u) return true;
+    }
+    return false;
 }
 
 uint64_t QueryDev::tc_slot_bytes() const {

@@ -79,10 +79,11 @@ cudaError_t launch_stage_fill(const uint32_t *src, const uint32_t *lbl, const ui
                               uint32_t *col, cudaStream_t st);
 cudaError_t launch_stage_unique(const uint32_t *off, uint32_t *col, uint32_t *ucnt, size_t rows, cudaStream_t st);
 cudaError_t launch_stage_compact(const uint32_t *off, const uint32_t *col, const uint32_t *uoff, uint32_t *ucol,
-                                 size_t rows, uint32_t *total_out, cudaStream_t st);
+                                 size_t rows, uint32_t n, uint32_t counted, uint32_t *result, cudaStream_t st);
 size_t stage_small_bytes(uint32_t n, uint32_t n_term, size_t m);
 cudaError_t launch_stage_small(const uint32_t *src, const uint32_t *lbl, const uint32_t *dst, size_t m, uint32_t n,
-                               uint32_t n_term, uint32_t *csr_off, uint32_t *csr_col, int *result, cudaStream_t st);
+                               uint32_t n_term, uint32_t counted, uint32_t *csr_off, uint32_t *csr_col,
+                               uint32_t *result, cudaStream_t st);
 cudaError_t launch_popcount(const uint64_t *p, size_t nwords, unsigned long long *out, cudaStream_t st);
 cudaError_t launch_csr_to_coo(const uint32_t *off, const uint32_t *col, size_t rows, uint32_t n, uint32_t *coo,
                               cudaStream_t st);
@@ -188,6 +189,22 @@ int copy_rsm(const cfpq_rsm *r, HostRSM *out, std::string *err);
 struct GraphDev {
     uint32_t n = 0, n_pad = 0, W = 0, n_term = 0;
     size_t m_in = 0, m_unique = 0;
+    // What staging reports: an edge out of range, edges kept, and for the first
+    // kCountedLabels labels the edges kept of the labels before.
+    static constexpr uint32_t kCountedLabels = 62;  // (256 bytes in all)
+    std::vector<uint32_t> label_start;
+    uint32_t counted_labels(uint32_t nt) const { return nt < kCountedLabels ? nt : kCountedLabels; }
+    void set_counts(const uint32_t *result, uint32_t nt) {
+        m_unique = result[1];
+        label_start.assign(result + 2, result + 2 + counted_labels(nt));
+        label_start.push_back(result[1]);
+    }
+    // edges kept of label l; past the counted labels, the mean of the rest
+    uint64_t edges_of(uint32_t l) const {
+        const uint32_t c = (uint32_t)label_start.size() - 1u;
+        if (l + 1u < c || n_term == c) return label_start[l + 1u] - label_start[l];
+        return (label_start[c] - label_start[c - 1u]) / (n_term - c + 1u);
+    }
     DBuf csr_off;  // [n_term * n + 1]
     DBuf csr_col;  // [m_unique]
     // Row bitmaps derived from the CSR, rebuilt when `content` moves on:
@@ -286,6 +303,18 @@ struct QueryDev {
     std::vector<int32_t> blk_slice;
     uint32_t n_slice_groups = 0;
     uint64_t loop_mask = 0;
+    // Components that could be sliced, and whether they are: by the edges that a
+    // sweep visits (slice_edges_max).  A graph loaded since may decide otherwise.
+    struct SliceChoice {
+        uint32_t members, groups;
+        std::vector<uint32_t> labels;  // one per transition within the component
+        bool sliced;
+    };
+    std::vector<SliceChoice> slice_choices;
+    bool shares_device = false;  // other queries run in the same passes (batch, server)
+    uint64_t slice_edges(const SliceChoice &c) const;
+    uint64_t slice_edges_max(const SliceChoice &c) const;
+    bool slice_choices_stale() const;
     unsigned long long nt_read_mask = 0;  // boxes read by some transition (bit 63: some box >= 63)
     std::vector<Src> srcs;
     std::vector<uint32_t> box_f0, box_nf;

@@ -1752,8 +1752,12 @@ __global__ void k_stage_unique(const uint32_t *__restrict__ off, uint32_t *col, 
 }
 
 __global__ void k_stage_compact(const uint32_t *__restrict__ off, const uint32_t *__restrict__ col,
-                                const uint32_t *__restrict__ uoff, uint32_t *ucol, size_t rows, uint32_t *total_out) {
-    if (total_out && blockIdx.x == 0 && threadIdx.x == 0) *total_out = uoff[rows];
+                                const uint32_t *__restrict__ uoff, uint32_t *ucol, size_t rows, uint32_t n,
+                                uint32_t counted, uint32_t *result) {
+    if (blockIdx.x == 0) {
+        if (threadIdx.x == 0) result[1] = uoff[rows];
+        for (uint32_t l = threadIdx.x; l < counted; l += blockDim.x) result[2u + l] = uoff[(size_t)l * n];
+    }
     for (size_t r = (size_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += (size_t)gridDim.x * blockDim.x) {
         const uint32_t a = off[r], u0 = uoff[r], k = uoff[r + 1] - u0;
         for (uint32_t i = 0; i < k; ++i) ucol[u0 + i] = col[a + i];
@@ -1833,11 +1837,13 @@ __global__ void k_scan_add(uint32_t *out, const uint32_t *__restrict__ block_sum
 // shared memory (rows = n_term * n counters, m columns): a load of a small graph is a
 // chain of launches otherwise, 62 us at n = 200 and 72 at n = 1000 with eleven, 21 and
 // 29 with this one.  The CSR is the same (rows sorted, repeated edges dropped up
-// to kUniqueMax).  result[0] = 1 on an edge out of range, result[1] = edges kept.
+// to kUniqueMax).  result[0] = 1 on an edge out of range, result[1] = edges kept,
+// result[2 + l] = edges kept of the labels before l (l < counted).
 constexpr uint32_t kStageThreads = 1024;
 __global__ void __launch_bounds__(kStageThreads, 1)
     k_stage_small(const uint32_t *__restrict__ src, const uint32_t *__restrict__ lbl, const uint32_t *__restrict__ dst,
-                  uint32_t m, uint32_t n, uint32_t n_term, uint32_t *csr_off, uint32_t *csr_col, int *result) {
+                  uint32_t m, uint32_t n, uint32_t n_term, uint32_t counted, uint32_t *csr_off, uint32_t *csr_col,
+                  uint32_t *result) {
     extern __shared__ uint32_t s_stage[];  // [rows] counters, then [m] columns
     const uint32_t tid = threadIdx.x, rows = n * n_term;
     uint32_t *const cnt = s_stage, *const col = s_stage + rows;
@@ -1898,6 +1904,7 @@ __global__ void __launch_bounds__(kStageThreads, 1)
     for (uint32_t r = r0; r < r1; ++r) {
         const uint32_t k = cnt[r] & 0xFFFFu, len = cnt[r] >> 16;
         csr_off[r] = out;
+        if (r % n == 0u && r / n < counted) result[2u + r / n] = out;
         if (k == len)
             for (uint32_t i = 0; i < len; ++i) csr_col[out + i] = col[a + i];
         else
@@ -1908,8 +1915,8 @@ __global__ void __launch_bounds__(kStageThreads, 1)
     }
     if (tid == 0) {
         csr_off[rows] = total;
-        result[0] = bad;
-        result[1] = (int)total;
+        result[0] = (uint32_t)bad;
+        result[1] = total;
     }
 }
 
@@ -2216,17 +2223,19 @@ size_t stage_small_bytes(uint32_t n, uint32_t n_term, size_t m) {
     return m <= 16384u && (uint64_t)n * n_term <= 12288u && bytes <= (160u << 10) ? (size_t)std::max<uint64_t>(bytes, 16u) : 0;
 }
 cudaError_t launch_stage_small(const uint32_t *src, const uint32_t *lbl, const uint32_t *dst, size_t m, uint32_t n,
-                               uint32_t n_term, uint32_t *csr_off, uint32_t *csr_col, int *result, cudaStream_t st) {
+                               uint32_t n_term, uint32_t counted, uint32_t *csr_off, uint32_t *csr_col,
+                               uint32_t *result, cudaStream_t st) {
     const size_t smem = stage_small_bytes(n, n_term, m);
     const cudaError_t e = cudaFuncSetAttribute(k_stage_small, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 << 10);
     if (e != cudaSuccess) return e;
-    k_stage_small<<<1, kStageThreads, smem, st>>>(src, lbl, dst, (uint32_t)m, n, n_term, csr_off, csr_col, result);
+    k_stage_small<<<1, kStageThreads, smem, st>>>(src, lbl, dst, (uint32_t)m, n, n_term, counted, csr_off, csr_col,
+                                                  result);
     return cudaGetLastError();
 }
 cudaError_t launch_stage_compact(const uint32_t *off, const uint32_t *col, const uint32_t *uoff, uint32_t *ucol,
-                                 size_t rows, uint32_t *total_out, cudaStream_t st) {
+                                 size_t rows, uint32_t n, uint32_t counted, uint32_t *result, cudaStream_t st) {
     if (rows == 0) return cudaSuccess;
-    k_stage_compact<<<grid_for(rows, 128), 128, 0, st>>>(off, col, uoff, ucol, rows, total_out);
+    k_stage_compact<<<grid_for(rows, 128), 128, 0, st>>>(off, col, uoff, ucol, rows, n, counted, result);
     return cudaGetLastError();
 }
 cudaError_t launch_csr_to_bits(const uint32_t *off, const uint32_t *col, size_t rows, uint32_t W, uint64_t *bits,

@@ -40,6 +40,7 @@ constexpr size_t kNaCol = kNaUcnt + rup(kNaMaxRows);
 constexpr size_t kNaTmp = kNaCol + rup(kNaMaxEdges);
 constexpr size_t kNaMap = kNaTmp + rup(kNaMaxRows / 4096 + 2);
 constexpr size_t kNaErr = kNaMap + rup(kNaMaxRows);
+static_assert(2 + GraphDev::kCountedLabels <= kNaAlign, "what staging reports fits its part");
 constexpr size_t kNaWords = kNaErr + kNaAlign;  // 4 * 2^19 + 2^21 words + padding: about 16 MiB
 
 __device__ __align__(256) uint32_t g_na_scratch[kNaWords];
@@ -106,7 +107,8 @@ extern "C" int cfpq_load_graph_device_noalloc(cfpq_ctx *ctx, uint32_t n, uint32_
         uint32_t *cnt = base + kNaCnt, *off = base + kNaOff, *ucnt = base + kNaUcnt, *col = base + kNaCol;
         uint32_t *tmp = base + kNaTmp;
         int32_t *map = reinterpret_cast<int32_t *>(base + kNaMap);
-        int *errf = reinterpret_cast<int *>(base + kNaErr);
+        uint32_t *res = base + kNaErr;
+        const uint32_t counted = g.counted_labels(n_term);
         const cudaStream_t st = ctx->stream;
         ctx->has_result = false;
         ++ctx->result_gen;
@@ -120,21 +122,20 @@ extern "C" int cfpq_load_graph_device_noalloc(cfpq_ctx *ctx, uint32_t n, uint32_
         k_na_identity<<<(n_term + 255) / 256, 256, 0, st>>>(map, n_term);
         NA_CK(cudaGetLastError());
         NA_CK(cudaMemsetAsync(cnt, 0, rows * 4, st));
-        NA_CK(cudaMemsetAsync(errf, 0, 16, st));
-        NA_CK(launch_stage_count(d_src, d_label, d_dst, m, n, n_term, map, cnt, errf, st));
+        NA_CK(cudaMemsetAsync(res, 0, 16, st));
+        NA_CK(launch_stage_count(d_src, d_label, d_dst, m, n, n_term, map, cnt, reinterpret_cast<int *>(res), st));
         NA_CK(scan_exclusive(cnt, off, rows, tmp, st));
         NA_CK(cudaMemsetAsync(ucnt, 0, rows * 4, st));
         NA_CK(launch_stage_fill(d_src, d_label, d_dst, m, n, n_term, map, off, ucnt, col, st));
         NA_CK(launch_stage_unique(off, col, ucnt, rows, st));
         NA_CK(scan_exclusive(ucnt, g.csr_off.as<uint32_t>(), rows, tmp, st));
-        NA_CK(launch_stage_compact(off, col, g.csr_off.as<uint32_t>(), g.csr_col.as<uint32_t>(), rows, nullptr, st));
-        int herr = 0;
-        uint32_t total = 0;
-        NA_CK(cudaMemcpyAsync(&herr, errf, 4, cudaMemcpyDeviceToHost, st));
-        NA_CK(cudaMemcpyAsync(&total, g.csr_off.as<uint32_t>() + rows, 4, cudaMemcpyDeviceToHost, st));
+        NA_CK(launch_stage_compact(off, col, g.csr_off.as<uint32_t>(), g.csr_col.as<uint32_t>(), rows, n, counted,
+                                   res, st));
+        uint32_t result[2 + GraphDev::kCountedLabels];
+        NA_CK(cudaMemcpyAsync(result, res, (2 + counted) * 4, cudaMemcpyDeviceToHost, st));
         NA_CK(cudaStreamSynchronize(st));
 #undef NA_CK
-        if (herr) {
+        if (result[0]) {
             g.n = 0;
             return fail(CFPQ_ERR_INVALID_ARG, "an edge names a vertex >= n_vertices or a label >= n_terminals");
         }
@@ -145,7 +146,7 @@ extern "C" int cfpq_load_graph_device_noalloc(cfpq_ctx *ctx, uint32_t n, uint32_
         g.W = W;
         g.n_term = n_term;
         g.m_in = m;
-        g.m_unique = total;
+        g.set_counts(result, n_term);
         g.host_valid = false;
         ctx->has_graph = true;
         // an RSM reading more terminals than this graph has is reported by

@@ -133,6 +133,7 @@ int cfpq_submit(cfpq_server *s, const cfpq_rsm *rsm, uint64_t *ticket) {
         }
         j.q->gather_slices = s->opt.gather_slices;
         j.q->use_slices = s->opt.max_rounds == 0;
+        j.q->shares_device = true;
         std::string e;
         int rc = copy_rsm(rsm, &j.q->rsm, &e);
         if (rc) return sfail(s, rc, e);

@@ -247,18 +247,21 @@ __device__ __forceinline__ bool row_has_work(const SrcDesc &d, uint32_t chans, u
 // kernel holds only the CSR paths, which keeps its registers for the rows.
 // --------------------------------------------------------------------------
 // Occupancy target per row width: narrow rows keep 4 CTAs (32 warps) per SM, for
-// which the general variants of widths 1 and 2 spill 184 and 248 bytes and the CSR
-// ones 68 and 116.
+// which the general variants of widths 1 and 2 spill 160 and 224 bytes and the CSR
+// one of width 1 spills 48.
 template <int VPL>
 struct GatherOcc {
     static constexpr int value = VPL <= 2 ? 4 : (VPL == 4 ? 2 : 1);
 };
 // CSR variant of wide rows: one source row in registers beside the output row
 // leaves room for two CTAs (it was one CTA with two source rows in flight); at
-// width 16 it spills 112 bytes.
+// width 16 it spills 72 bytes.  Width 2 takes three CTAs (80 registers): four spilled
+// 116 bytes in its inner loop.  With them and the item's channels in shared memory
+// (ab)*c|a*b* on the gather alone, n = 8192, went from 1.43 to 1.28 ms with 48 edges a
+// vertex, from 2.03 to 1.78 with 100.
 template <int VPL, bool NT>
 struct GatherCtas {
-    static constexpr int value = !NT && VPL >= 8 ? 2 : GatherOcc<VPL>::value;
+    static constexpr int value = NT ? GatherOcc<VPL>::value : VPL >= 8 ? 2 : VPL == 2 ? 3 : GatherOcc<VPL>::value;
 };
 
 // Scheduling.  Narrow rows: one CTA per live item (the grid covers every
@@ -289,6 +292,7 @@ __global__ void __launch_bounds__(256, GatherCtas<VPL, NT>::value)
     // rows of the item with work: their bits, then the list (an item has at most 1024 rows)
     __shared__ uint32_t s_rowbits[32];
     __shared__ uint16_t s_rows[1024];
+    __shared__ uint8_t s_chans[16];  // channels of the item's first sources (one CTA per item)
     // general variant: per-warp ring of source rows loaded with cp.async
     extern __shared__ uint4 s_ring[];
     constexpr int P = GatherRing<VPL>::depth;
@@ -329,6 +333,8 @@ __global__ void __launch_bounds__(256, GatherCtas<VPL, NT>::value)
             act |= src_channels<NT>(srcs[it.src0 + k], mode, iter, g, g0, dmask) != 0u;
         if (!__syncthreads_or(act)) continue;
 
+        for (uint32_t k = threadIdx.x; k < it.nsrc && k < 16u; k += blockDim.x)
+            s_chans[k] = (uint8_t)src_channels<NT>(srcs[it.src0 + k], mode, iter, g, g0, dmask);
         if (threadIdx.x == 0) { s_changed = 0; s_ors = 0; }
         if (threadIdx.x < 32u) s_rowbits[threadIdx.x] = 0u;
         __syncthreads();
@@ -361,14 +367,15 @@ __global__ void __launch_bounds__(256, GatherCtas<VPL, NT>::value)
     }
     const bool sliced = slices_on && (sv0 != 0u || sv1 < nvec);
     uint32_t my_changed = 0, my_ors = 0;
-    // channels of the item's first 16 sources in this pass (4 bits each): the
-    // same for every row of the unit
+    // channels of the item's first 16 sources in this pass: the same for every row.
+    // A warp unit packs them into a register pair (4 bits each), a CTA has them in s_chans.
     unsigned long long chpack = 0ull;
-    for (uint32_t k = 0; k < it.nsrc && k < 16u; ++k)
-        chpack |= (unsigned long long)src_channels<NT>(srcs[it.src0 + k], mode, iter, g, g0, dmask) << (4u * k);
+    if constexpr (kDyn)
+        for (uint32_t k = 0; k < it.nsrc && k < 16u; ++k)
+            chpack |= (unsigned long long)src_channels<NT>(srcs[it.src0 + k], mode, iter, g, g0, dmask) << (4u * k);
     auto chans_of = [&](uint32_t k) -> uint32_t {
-        return k < 16u ? (uint32_t)(chpack >> (4u * k)) & 15u
-                       : src_channels<NT>(srcs[it.src0 + k], mode, iter, g, g0, dmask);
+        if (k >= 16u) return src_channels<NT>(srcs[it.src0 + k], mode, iter, g, g0, dmask);
+        return kDyn ? (uint32_t)(chpack >> (4u * k)) & 15u : (uint32_t)s_chans[k];
     };
     auto wanted = [&](uint32_t r) { return !it.rmask || ((it.rmask[r >> 6] >> (r & 63u)) & 1ull) != 0ull; };
 

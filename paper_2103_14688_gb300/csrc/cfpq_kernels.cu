@@ -222,6 +222,11 @@ __device__ __forceinline__ uint32_t src_channels(const SrcDesc &d, uint32_t mode
 // warp that owns a row finds that out behind four dependent loads.  Loop time, visiting
 // every row -> only these: regular query n = 30011 7.27 -> 3.05 ms, Dyck-4 n = 3001
 // 4.84 -> 4.07, n = 65536 209 -> 186, 16 sources at n = 65536 5.0 -> 2.8.
+// A row of more than kTestEdges edges is taken untested: its lane would walk it alone, two
+// dependent loads an edge, where the gather reads the row with a warp.  a+ over a path of
+// 200 vertices and four vertices with edges to all others, on the gather: n = 8000 37.9 ->
+// 26.9 ms, n = 16000 78.3 -> 53.0, n = 30000 169 -> 108.
+constexpr uint32_t kTestEdges = 32;
 template <bool NT>
 __device__ __forceinline__ bool row_has_work(const SrcDesc &d, uint32_t chans, uint32_t x, uint32_t iter, uint32_t g,
                                              uint32_t g0) {
@@ -229,7 +234,7 @@ __device__ __forceinline__ bool row_has_work(const SrcDesc &d, uint32_t chans, u
         const uint32_t e1 = d.csr_off[x + 1];
         uint32_t e = d.csr_off[x];
         if (e >= e1) return false;
-        if (chans & 1u) return true;
+        if ((chans & 1u) || e1 - e > kTestEdges) return true;
         const uint32_t thr = (chans & 2u) ? g0 : g - 1u;
         for (; e < e1; ++e)
             if (d.rstamp[d.csr_col[e]] >= thr) return true;

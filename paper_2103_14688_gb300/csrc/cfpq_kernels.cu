@@ -1009,7 +1009,10 @@ __global__ void __launch_bounds__(256, kExpandOcc)
 // the one before read their words.  Slices of up to 2048 rows (R > 0) are bound by
 // latency instead: a thread owns R rows for all sweeps and holds the places of their
 // first four edges in registers, so that a row costs five independent loads and no
-// atomics (further edges are listed and applied edge by edge).  Regular query:
+// atomics (further edges are listed and applied edge by edge; when they are more than a
+// quarter of the rows, the slice is swept over edges instead: with a thread walking the rest
+// of its row, a+ at n = 2000, a path of 200 vertices and 20 vertices with edges to all others,
+// took 24.8 ms, with edge sweeps 1.25).  Regular query:
 // n = 1000 1785 -> 385 us with edge sweeps (241 us of run time), 183 us of run time with
 // owned rows; n = 8192 2119 -> 1369 us (owned rows: no gain, 1.07 ms of run time against
 // 1.04).  Above 200 KB a slice (n = 22755 for one state) the component stays on
@@ -1029,7 +1032,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
     extern __shared__ uint64_t s_col[];  // [nmem][n] words, then [nmem][n] bytes
     __shared__ uint32_t s_e0[kSliceMaxSrc], s_e1[kSliceMaxSrc], s_to[kSliceMaxSrc], s_from[kSliceMaxSrc], s_n;
     __shared__ const uint32_t *s_off[kSliceMaxSrc], *s_adj;
-    __shared__ uint32_t s_rest_n;
+    __shared__ uint32_t s_past, s_rest_n;
     __shared__ unsigned long long s_changed, s_ors;
     const uint32_t tid = threadIdx.x, NT = blockDim.x, total = T.g_total[cls];
     for (uint32_t li = blockIdx.x; li < total; li += gridDim.x) {
@@ -1071,6 +1074,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
                 }
             }
             s_n = k2;
+            s_past = 0u;
             s_rest_n = 0u;
         }
         for (uint32_t m = 0; m < G.nmem; ++m) {
@@ -1104,18 +1108,33 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
         }
         __syncthreads();
         const uint32_t ns = s_n;
+        bool owned = false;
         if constexpr (R > 0) {
+            uint32_t *const s_rest = reinterpret_cast<uint32_t *>(s_col + rows);  // edges past the fourth
+            uint32_t past = 0u;
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                const uint32_t row = tid + (uint32_t)i * NT;
+                if (row >= rows) continue;
+                const uint32_t m0 = row / n * n, x = row - m0;
+                uint32_t deg = 0u;
+                for (uint32_t k = 0; k < ns; ++k)
+                    if (s_to[k] == m0) deg += s_off[k][x + 1] - s_off[k][x];
+                past += deg > 4u ? deg - 4u : 0u;
+            }
+            past = __reduce_add_sync(FULLMASK, past);
+            if ((tid & 31u) == 0u && past) atomicAdd(&s_past, past);
+            __syncthreads();
+            owned = s_past <= rows / 4u;
             // this thread's rows tid, tid + NT, ...: places of their first four
             // edges (where there are fewer, the row's own: four plain loads beat
-            // four branches, 100 instructions a row), and whether there are more
-            uint32_t place[R][2], more = 0u;
-            uint32_t *const s_rest = reinterpret_cast<uint32_t *>(s_col + rows);  // edges past the fourth
-            const uint32_t rest_cap = rows / 4u;
+            // four branches, 100 instructions a row)
+            uint32_t place[R][2];
 #pragma unroll
             for (int i = 0; i < R; ++i) {
                 const uint32_t row = tid + (uint32_t)i * NT;
                 place[i][0] = place[i][1] = row < rows ? row | (row << 16) : 0u;
-                if (row >= rows) continue;
+                if (!owned || row >= rows) continue;
                 const uint32_t m0 = row / n * n, x = row - m0;
                 uint32_t got = 0u;
                 for (uint32_t k = 0; k < ns; ++k) {
@@ -1127,17 +1146,13 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
                         else if (got == 1u) place[i][0] = (place[i][0] & 0xFFFFu) | (at << 16);
                         else if (got == 2u) place[i][1] = (place[i][1] & 0xFFFF0000u) | at;
                         else if (got == 3u) place[i][1] = (place[i][1] & 0xFFFFu) | (at << 16);
-                        else {
-                            const uint32_t j = atomicAdd(&s_rest_n, 1u);
-                            if (j < rest_cap) s_rest[j] = (row << 16) | at;
-                            else more |= 1u << i;  // no room: the row walks its edges in the CSR
-                        }
+                        else s_rest[atomicAdd(&s_rest_n, 1u)] = (row << 16) | at;
                     }
                 }
             }
             __syncthreads();
-            const uint32_t rest = min(s_rest_n, rest_cap);
-            bool ch = true;
+            const uint32_t rest = s_rest_n;
+            bool ch = owned;
             while (__syncthreads_or(ch)) {
                 ch = false;
                 // (a row's owner may overwrite bits set here; the next sweep, which
@@ -1157,16 +1172,6 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
                     const uint64_t old = s_col[row < rows ? row : 0u];
                     uint64_t v = s_col[place[i][0] & 0xFFFFu] | s_col[place[i][0] >> 16] | s_col[place[i][1] & 0xFFFFu] |
                                  s_col[place[i][1] >> 16];
-                    if ((more >> i) & 1u) {
-                        const uint32_t m0 = row / n * n, x = row - m0;
-                        uint32_t got = 0u;
-                        for (uint32_t k = 0; k < ns; ++k) {
-                            if (s_to[k] != m0) continue;
-                            const uint32_t e1 = s_off[k][x + 1];
-                            for (uint32_t e = s_off[k][x]; e < e1; ++e, ++got)
-                                if (got >= 4u) v |= s_col[s_from[k] + s_adj[e]];
-                        }
-                    }
                     // (a thread past the last row read row 0's word five times: it may have
                     // grown in between, and there is no row to store)
                     if (row < rows && (v & ~old)) {
@@ -1176,7 +1181,8 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
                     }
                 }
             }
-        } else {
+        }
+        if (!owned) {
         // mark: the low byte of the sweep that last changed the row (rows with bits start as
         // changed in sweep 0; 128 is no sweep within reach of the first ones)
         for (uint32_t x = tid; x < rows; x += NT) s_mark[x] = s_col[x] ? 0u : 128u;

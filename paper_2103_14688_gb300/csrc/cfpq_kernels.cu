@@ -253,14 +253,14 @@ __device__ __forceinline__ bool row_has_work(const SrcDesc &d, uint32_t chans, u
 // --------------------------------------------------------------------------
 // Occupancy target per row width: narrow rows keep 4 CTAs (32 warps) per SM, for
 // which the general variants of widths 1 and 2 spill 160 and 224 bytes and the CSR
-// one of width 1 spills 48.
+// one of width 1 spills 52.
 template <int VPL>
 struct GatherOcc {
     static constexpr int value = VPL <= 2 ? 4 : (VPL == 4 ? 2 : 1);
 };
 // CSR variant of wide rows: one source row in registers beside the output row
 // leaves room for two CTAs (it was one CTA with two source rows in flight); at
-// width 16 it spills 72 bytes.  Width 2 takes three CTAs (80 registers): four spilled
+// width 16 it spills 80 bytes.  Width 2 takes three CTAs (80 registers): four spilled
 // 116 bytes in its inner loop.  With them and the item's channels in shared memory
 // (ab)*c|a*b* on the gather alone, n = 8192, went from 1.43 to 1.28 ms with 48 edges a
 // vertex, from 2.03 to 1.78 with 100.
@@ -289,6 +289,93 @@ struct GatherDyn {
 constexpr uint32_t kGatherParts = 8;
 constexpr uint32_t kStrideWaves = 8;  // launch_gather: waves of resident CTAs at most
 
+// Row `at` of a CSR item, source k of more than kHubEdges edges, by the whole CTA: its warps
+// take 32 edges in turn and merge what they found with atomics.  Such a row's one warp was
+// the pass, bound by the latency of a source row after another, and the widest rows, which
+// gave up half their loads in flight for a second CTA, took 2.5 times what they had taken before.
+// a+ on the gather, a path of 200 vertices and four with edges to all others: n = 8000 26.7 ->
+// 6.6 ms, 30000 105 -> 21, 60000 463 -> 63.  Not inlined, and the main loop only leaves the
+// row's source out: inlined, or listed before the loop, sparse graphs lost up to 7% to
+// spills and extra loads; as it is they lose 1%.
+constexpr uint32_t kHubEdges = 512, kHubs = 64;  // (kHubs: listed by an item at most)
+template <int VPL>
+__device__ __noinline__ void gather_hub(const GItem *__restrict__ item, const SrcDesc *__restrict__ srcs, uint32_t at,
+                                        uint32_t k, unsigned long long *s_changed, unsigned long long *s_ors) {
+    const GItem &it = *item;
+    const QCtl *c = it.ctl;
+    const uint32_t row = it.row0 + at;
+    const uint32_t g = c->g, iter = c->iter, mode = c->mode, g0 = c->g_iter_start, dmask = c->dense_mask;
+    const int lane = threadIdx.x & 31, lpr = (int)it.lpr, grp = lane / lpr, gl = lane % lpr;
+    const unsigned gmask = (lpr == 32 ? FULLMASK : ((1u << lpr) - 1u)) << (grp * lpr);
+    const uint32_t W = it.W, cv0 = c->col_v0, cv1 = min(c->col_v1, W / 2u);
+    uint64_t *const out = it.out + (size_t)row * W;
+    uint4 acc[VPL];
+#pragma unroll
+    for (int j = 0; j < VPL; ++j) acc[j] = make_uint4(0, 0, 0, 0);
+    uint32_t ors = 0u;
+    bool ch = false;
+    const SrcDesc &d = srcs[it.src0 + k];
+    const uint32_t chans = src_channels<false>(d, mode, iter, g, g0, dmask);
+    const uint32_t *const col = d.csr_col, *const rstamp = d.rstamp;
+    const uint64_t *const rblk = d.rblk;
+    const uint32_t e1 = d.csr_off[row + 1];
+    const bool ident = (chans & 1u) && d.ident;
+    // (one channel a pass: new edges only in iteration 1, whole rows then)
+    const uint32_t thr = (chans & 1u) ? 0u : (chans & 2u) ? g0 : g - 1u;
+    for (uint32_t b = d.csr_off[row] + (threadIdx.x & ~31u); b < e1; b += 256u) {
+        const bool has = b + (uint32_t)lane < e1;
+        const uint32_t yl = has ? col[b + (uint32_t)lane] : 0u;
+        if (ident && has && (yl >> 7) >= cv0 && (yl >> 7) < cv1) {
+            unsigned int *const w = reinterpret_cast<unsigned int *>(out) + (yl >> 5);
+            const unsigned int bit = 1u << (yl & 31u);
+            if (!(*w & bit) && !(atomicOr(w, bit) & bit)) ch = true;
+        }
+        if (!rblk) continue;
+        const unsigned bal = __ballot_sync(FULLMASK, has && (thr == 0u || rstamp[yl] >= thr));
+        unsigned mine = (bal & gmask) >> (grp * lpr);
+        constexpr int U = VPL >= 8 ? 1 : VPL == 4 ? 2 : 4, J = VPL < 8 ? VPL : 8;
+        while (__any_sync(FULLMASK, mine != 0u)) {
+            const uint4 *r[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const bool h = mine != 0u;
+                const uint32_t y = __shfl_sync(FULLMASK, yl, h ? __ffs(mine) - 1 : 0, lpr);
+                r[u] = h ? reinterpret_cast<const uint4 *>(rblk + (size_t)y * W) : nullptr;
+                if (h && gl == 0) ++ors;
+                mine &= mine - 1u;
+            }
+#pragma unroll
+            for (int j0 = 0; j0 < VPL; j0 += J) {
+                uint4 a[U][J];
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+#pragma unroll
+                    for (int j = 0; j < J; ++j) {
+                        const uint32_t v = (uint32_t)gl + (uint32_t)(j0 + j) * lpr;
+                        a[u][j] = r[u] && v >= cv0 && v < cv1 ? r[u][v] : make_uint4(0, 0, 0, 0);
+                    }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+#pragma unroll
+                    for (int j = 0; j < J; ++j) or4(acc[j0 + j], a[u][j]);
+            }
+        }
+    }
+    unsigned long long *const o = reinterpret_cast<unsigned long long *>(out);
+#pragma unroll
+    for (int j = 0; j < VPL; ++j) {
+        if (!nz4(acc[j])) continue;
+        const uint32_t v = (uint32_t)gl + (uint32_t)j * lpr;
+        const unsigned long long lo = ((unsigned long long)acc[j].y << 32) | acc[j].x;
+        const unsigned long long hi = ((unsigned long long)acc[j].w << 32) | acc[j].z;
+        if ((lo & ~o[2u * v]) && (lo & ~atomicOr(o + 2u * v, lo))) ch = true;
+        if ((hi & ~o[2u * v + 1u]) && (hi & ~atomicOr(o + 2u * v + 1u, hi))) ch = true;
+    }
+    // (a pass counts the row once)
+    if (__any_sync(FULLMASK, ch) && lane == 0 && atomicExch(it.out_stamp + row, g) != g) atomicAdd(s_changed, 1ull);
+    if (ors) atomicAdd(s_ors, (unsigned long long)ors);
+}
+
 template <int VPL, bool NT>
 __global__ void __launch_bounds__(256, GatherCtas<VPL, NT>::value)
     k_gather(const GItem *__restrict__ items, const SrcDesc *__restrict__ srcs, ExecTables T, int cls) {
@@ -298,6 +385,7 @@ __global__ void __launch_bounds__(256, GatherCtas<VPL, NT>::value)
     __shared__ uint32_t s_rowbits[32];
     __shared__ uint16_t s_rows[1024];
     __shared__ uint8_t s_chans[16];  // channels of the item's first sources (one CTA per item)
+    __shared__ uint32_t s_hubs[kHubs], s_nhubs;  // CSR variant: rows (k << 10 | row) left to gather_hub
     // general variant: per-warp ring of source rows loaded with cp.async
     extern __shared__ uint4 s_ring[];
     constexpr int P = GatherRing<VPL>::depth;
@@ -340,7 +428,7 @@ __global__ void __launch_bounds__(256, GatherCtas<VPL, NT>::value)
 
         for (uint32_t k = threadIdx.x; k < it.nsrc && k < 16u; k += blockDim.x)
             s_chans[k] = (uint8_t)src_channels<NT>(srcs[it.src0 + k], mode, iter, g, g0, dmask);
-        if (threadIdx.x == 0) { s_changed = 0; s_ors = 0; }
+        if (threadIdx.x == 0) { s_changed = 0; s_ors = 0; s_nhubs = 0u; }
         if (threadIdx.x < 32u) s_rowbits[threadIdx.x] = 0u;
         __syncthreads();
     }
@@ -607,9 +695,20 @@ __global__ void __launch_bounds__(256, GatherCtas<VPL, NT>::value)
 
                 if (d.csr_off) {
                     if (sv0 != 0u) continue;  // CSR sources belong to the first slice
-                    const uint32_t e0 = valid ? d.csr_off[row] : 0u, e1 = valid ? d.csr_off[row + 1] : 0u;
-                    const uint32_t cnt = e1 - e0;
-                    const uint32_t maxcnt = __reduce_max_sync(FULLMASK, cnt);
+                    const uint32_t e0 = valid ? d.csr_off[row] : 0u;
+                    uint32_t e1 = valid ? d.csr_off[row + 1] : 0u;
+                    uint32_t cnt = e1 - e0, maxcnt = __reduce_max_sync(FULLMASK, cnt);
+                    if (!NT && maxcnt > kHubEdges) {  // (uniform over the warp)
+                        bool listed = false;
+                        if (cnt > kHubEdges && gl == 0) {
+                            const uint32_t h = atomicAdd(&s_nhubs, 1u);
+                            listed = h < kHubs;
+                            if (listed) s_hubs[h] = (k << 10) | (row - it.row0);
+                        }
+                        if (__shfl_sync(FULLMASK, (int)listed, 0, lpr)) e1 = e0;
+                        cnt = e1 - e0;
+                        maxcnt = __reduce_max_sync(FULLMASK, cnt);
+                    }
                     if (maxcnt <= 8u && (!NT || !d.pure_n)) {
                         // short adjacency rows (the common case on sparse
                         // graphs): no ballot; edges two at a time so that the
@@ -791,6 +890,12 @@ __global__ void __launch_bounds__(256, GatherCtas<VPL, NT>::value)
         if (my_changed) atomicAdd(&s_changed, (unsigned long long)my_changed);
         if (my_ors) atomicAdd(&s_ors, (unsigned long long)my_ors);
         __syncthreads();
+        if (!NT && s_nhubs) {
+            for (uint32_t h = 0; h < min(s_nhubs, kHubs); ++h)
+                gather_hub<VPL>(items + live_item(T.g_pre[cls], T.g_beg[cls], T.nq, li), srcs, s_hubs[h] & 1023u,
+                                s_hubs[h] >> 10, &s_changed, &s_ors);
+            __syncthreads();
+        }
         if (threadIdx.x == 0) {
             QCtl *cw = it.ctl;
             if (s_changed) {

@@ -215,7 +215,8 @@ int ensure_query(cfpq_ctx *ctx, bool restricted = false) {
         bool moved = false;
         ctx->exec_dirty = true;  // (also when it fails: a buffer may have moved before)
         if (int rc = q.refresh_graph_caches(&ctx->A, ctx->stream, &e, &moved)) return fail(ctx, rc, e);
-        ctx->exec_dirty = moved || q.slice_choices_stale();
+        // (rows to share: the other variant would be right, but slow)
+        ctx->exec_dirty = moved || q.slice_choices_stale() || (ctx->graph.hub_rows && !ctx->exec.hub_rows);
     }
     if (!q.prepared || q.graph_generation != ctx->graph.generation || ctx->exec_dirty) {
         std::string e;

@@ -284,7 +284,7 @@ int stage_graph(GraphDev *g, Allocator *A, cudaStream_t st, uint32_t n, uint32_t
     uint32_t result[2 + GraphDev::kCountedLabels];
     ENG_CK(cudaMemcpyAsync(result, res, (2 + counted) * 4, cudaMemcpyDeviceToHost, st));
     ENG_CK(cudaStreamSynchronize(st));
-    if (result[0]) {
+    if (result[0] & 1u) {
         *err = "an edge names a vertex >= n_vertices or a label >= n_terminals";
         g->n = 0;
         return CFPQ_ERR_INVALID_ARG;
@@ -1078,6 +1078,8 @@ int Executor::assemble(Allocator *A, cudaStream_t st, std::string *err) {
     if ((rc = upload(fds, hf.data(), hf.size() * sizeof(FDesc)))) return rc;
     if ((rc = upload(tcjobs, hj.data(), hj.size() * sizeof(TcJob)))) return rc;
     n_tcjobs = (uint32_t)hj.size();
+    hub_rows = false;
+    for (const QueryDev *q : qs) hub_rows |= q->g->hub_rows;
     any_uncompacted = false;
     for (const auto &j : hj) any_uncompacted |= !j.covers_new && j.kcap < j.n;
     // TMA descriptors of the jobs' FP8 operands (a8, b8 per job)
@@ -1213,8 +1215,8 @@ int Executor::enqueue_pass(cudaStream_t st, cudaGraphConditionalHandle h, int us
     for (int c = kExpandNarrow; c <= kExpandWide; ++c)
         ENG_CK(launch_expand(c == kExpandWide, items[c].as<GItem>(), live(c), srcs.as<SrcDesc>(), max_expand_w, T, c, sa));
     for (int c = 0; c < kExpandNarrow; ++c)
-        ENG_CK(launch_gather(kVplOf[c / 2], (c & 1) != 0, items[c].as<GItem>(), live(c), srcs.as<SrcDesc>(), T, c,
-                             (c & 1) ? st : sb));
+        ENG_CK(launch_gather(kVplOf[c / 2], (c & 1) != 0, hub_rows, items[c].as<GItem>(), live(c), srcs.as<SrcDesc>(),
+                             T, c, (c & 1) ? st : sb));
     if (ev) ENG_CK(cudaEventRecord(ev[2], st));
     if (tiles) {
         if (any_uncompacted) ENG_CK(launch_tc_product(false, tcjobs.as<TcJob>(), tiles, T, tc_err.as<int>(), st));

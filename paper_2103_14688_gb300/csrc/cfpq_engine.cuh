@@ -24,7 +24,7 @@ namespace cfpq {
 
 // ---- kernel launchers (cfpq_kernels.cu) ----
 int vpl_for_words(uint32_t W);
-cudaError_t launch_gather(int vpl, bool nt, const GItem *items, uint32_t n_items, const SrcDesc *srcs,
+cudaError_t launch_gather(int vpl, bool nt, bool hubs, const GItem *items, uint32_t n_items, const SrcDesc *srcs,
                           const ExecTables &T, int cls, cudaStream_t st);
 cudaError_t launch_expand(bool wide, const GItem *items, uint32_t n_items, const SrcDesc *srcs, uint32_t max_w,
                           const ExecTables &T, int cls, cudaStream_t st);
@@ -189,12 +189,15 @@ int copy_rsm(const cfpq_rsm *r, HostRSM *out, std::string *err);
 struct GraphDev {
     uint32_t n = 0, n_pad = 0, W = 0, n_term = 0;
     size_t m_in = 0, m_unique = 0;
-    // What staging reports: an edge out of range, edges kept, and for the first
-    // kCountedLabels labels the edges kept of the labels before.
+    // What staging reports: an edge out of range (1) and a row of more than kHubEdges
+    // edges (2), edges kept, and for the first kCountedLabels labels the edges kept of
+    // the labels before.
     static constexpr uint32_t kCountedLabels = 62;  // (256 bytes in all)
     std::vector<uint32_t> label_start;
+    bool hub_rows = false;
     uint32_t counted_labels(uint32_t nt) const { return nt < kCountedLabels ? nt : kCountedLabels; }
     void set_counts(const uint32_t *result, uint32_t nt) {
+        hub_rows = (result[0] & 2u) != 0u;
         m_unique = result[1];
         label_start.assign(result + 2, result + 2 + counted_labels(nt));
         label_start.push_back(result[1]);
@@ -407,6 +410,7 @@ struct Executor {
     static constexpr int kBranches = 2;
     cudaStream_t side[kBranches] = {nullptr, nullptr};
     cudaEvent_t fork_ev = nullptr, join_ev[kBranches] = {nullptr, nullptr};
+    bool hub_rows = false;         // some graph has rows that the CSR gather shares (gather_hub)
     bool any_uncompacted = false;  // some tile job's list may exceed its operands' room (k_tc_product)
     bool built = false;
     ~Executor() {

@@ -253,14 +253,14 @@ __device__ __forceinline__ bool row_has_work(const SrcDesc &d, uint32_t chans, u
 // --------------------------------------------------------------------------
 // Occupancy target per row width: narrow rows keep 4 CTAs (32 warps) per SM, for
 // which the general variants of widths 1 and 2 spill 160 and 224 bytes and the CSR
-// one of width 1 spills 52.
+// one of width 1 spills 48.
 template <int VPL>
 struct GatherOcc {
     static constexpr int value = VPL <= 2 ? 4 : (VPL == 4 ? 2 : 1);
 };
 // CSR variant of wide rows: one source row in registers beside the output row
 // leaves room for two CTAs (it was one CTA with two source rows in flight); at
-// width 16 it spills 80 bytes.  Width 2 takes three CTAs (80 registers): four spilled
+// width 16 it spills 72 bytes.  Width 2 takes three CTAs (80 registers): four spilled
 // 116 bytes in its inner loop.  With them and the item's channels in shared memory
 // (ab)*c|a*b* on the gather alone, n = 8192, went from 1.43 to 1.28 ms with 48 edges a
 // vertex, from 2.03 to 1.78 with 100.
@@ -296,7 +296,8 @@ constexpr uint32_t kStrideWaves = 8;  // launch_gather: waves of resident CTAs a
 // a+ on the gather, a path of 200 vertices and four with edges to all others: n = 8000 26.7 ->
 // 6.6 ms, 30000 105 -> 21, 60000 463 -> 63.  Not inlined, and the main loop only leaves the
 // row's source out: inlined, or listed before the loop, sparse graphs lost up to 7% to
-// spills and extra loads; as it is they lose 1%.
+// spills and extra loads.  As it is they lost 1.5% (the regular query at n = 30011), so graphs
+// without such rows take a variant without it (GraphDev::hub_rows).
 constexpr uint32_t kHubEdges = 512, kHubs = 64;  // (kHubs: listed by an item at most)
 template <int VPL>
 __device__ __noinline__ void gather_hub(const GItem *__restrict__ item, const SrcDesc *__restrict__ srcs, uint32_t at,
@@ -376,7 +377,7 @@ __device__ __noinline__ void gather_hub(const GItem *__restrict__ item, const Sr
     if (ors) atomicAdd(s_ors, (unsigned long long)ors);
 }
 
-template <int VPL, bool NT>
+template <int VPL, bool NT, bool HUB>
 __global__ void __launch_bounds__(256, GatherCtas<VPL, NT>::value)
     k_gather(const GItem *__restrict__ items, const SrcDesc *__restrict__ srcs, ExecTables T, int cls) {
     constexpr bool kDyn = GatherDyn<VPL, NT>::on;
@@ -385,7 +386,7 @@ __global__ void __launch_bounds__(256, GatherCtas<VPL, NT>::value)
     __shared__ uint32_t s_rowbits[32];
     __shared__ uint16_t s_rows[1024];
     __shared__ uint8_t s_chans[16];  // channels of the item's first sources (one CTA per item)
-    __shared__ uint32_t s_hubs[kHubs], s_nhubs;  // CSR variant: rows (k << 10 | row) left to gather_hub
+    __shared__ uint32_t s_hubs[kHubs], s_nhubs;  // HUB: rows (k << 10 | row) left to gather_hub
     // general variant: per-warp ring of source rows loaded with cp.async
     extern __shared__ uint4 s_ring[];
     constexpr int P = GatherRing<VPL>::depth;
@@ -695,20 +696,8 @@ __global__ void __launch_bounds__(256, GatherCtas<VPL, NT>::value)
 
                 if (d.csr_off) {
                     if (sv0 != 0u) continue;  // CSR sources belong to the first slice
-                    const uint32_t e0 = valid ? d.csr_off[row] : 0u;
-                    uint32_t e1 = valid ? d.csr_off[row + 1] : 0u;
+                    const uint32_t e0 = valid ? d.csr_off[row] : 0u, e1 = valid ? d.csr_off[row + 1] : 0u;
                     uint32_t cnt = e1 - e0, maxcnt = __reduce_max_sync(FULLMASK, cnt);
-                    if (!NT && maxcnt > kHubEdges) {  // (uniform over the warp)
-                        bool listed = false;
-                        if (cnt > kHubEdges && gl == 0) {
-                            const uint32_t h = atomicAdd(&s_nhubs, 1u);
-                            listed = h < kHubs;
-                            if (listed) s_hubs[h] = (k << 10) | (row - it.row0);
-                        }
-                        if (__shfl_sync(FULLMASK, (int)listed, 0, lpr)) e1 = e0;
-                        cnt = e1 - e0;
-                        maxcnt = __reduce_max_sync(FULLMASK, cnt);
-                    }
                     if (maxcnt <= 8u && (!NT || !d.pure_n)) {
                         // short adjacency rows (the common case on sparse
                         // graphs): no ballot; edges two at a time so that the
@@ -771,6 +760,16 @@ __global__ void __launch_bounds__(256, GatherCtas<VPL, NT>::value)
                             }
                         }
                     } else {
+                        if (HUB && maxcnt > kHubEdges) {  // (uniform over the warp)
+                            bool listed = false;
+                            if (cnt > kHubEdges && gl == 0) {
+                                const uint32_t h = atomicAdd(&s_nhubs, 1u);
+                                listed = h < kHubs;
+                                if (listed) s_hubs[h] = (k << 10) | (row - it.row0);
+                            }
+                            if (__shfl_sync(FULLMASK, (int)listed, 0, lpr)) cnt = 0u;
+                            maxcnt = __reduce_max_sync(FULLMASK, cnt);
+                        }
                         for (uint32_t base = 0; base < maxcnt; base += (uint32_t)lpr) {
                             const uint32_t k2 = base + (uint32_t)gl;
                             const bool has = k2 < cnt;
@@ -890,7 +889,7 @@ __global__ void __launch_bounds__(256, GatherCtas<VPL, NT>::value)
         if (my_changed) atomicAdd(&s_changed, (unsigned long long)my_changed);
         if (my_ors) atomicAdd(&s_ors, (unsigned long long)my_ors);
         __syncthreads();
-        if (!NT && s_nhubs) {
+        if (HUB && s_nhubs) {
             for (uint32_t h = 0; h < min(s_nhubs, kHubs); ++h)
                 gather_hub<VPL>(items + live_item(T.g_pre[cls], T.g_beg[cls], T.nq, li), srcs, s_hubs[h] & 1023u,
                                 s_hubs[h] >> 10, &s_changed, &s_ors);
@@ -1874,6 +1873,7 @@ __global__ void k_stage_unique(const uint32_t *__restrict__ off, uint32_t *col, 
     }
 }
 
+// result[0] bit 1: a row of more than kHubEdges edges is kept.
 __global__ void k_stage_compact(const uint32_t *__restrict__ off, const uint32_t *__restrict__ col,
                                 const uint32_t *__restrict__ uoff, uint32_t *ucol, size_t rows, uint32_t n,
                                 uint32_t counted, uint32_t *result) {
@@ -1883,6 +1883,7 @@ __global__ void k_stage_compact(const uint32_t *__restrict__ off, const uint32_t
     }
     for (size_t r = (size_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += (size_t)gridDim.x * blockDim.x) {
         const uint32_t a = off[r], u0 = uoff[r], k = uoff[r + 1] - u0;
+        if (k > kHubEdges) atomicOr(result, 2u);
         for (uint32_t i = 0; i < k; ++i) ucol[u0 + i] = col[a + i];
     }
 }
@@ -1960,7 +1961,8 @@ __global__ void k_scan_add(uint32_t *out, const uint32_t *__restrict__ block_sum
 // shared memory (rows = n_term * n counters, m columns): a load of a small graph is a
 // chain of launches otherwise, 62 us at n = 200 and 72 at n = 1000 with eleven, 21 and
 // 29 with this one.  The CSR is the same (rows sorted, repeated edges dropped up
-// to kUniqueMax).  result[0] = 1 on an edge out of range, result[1] = edges kept,
+// to kUniqueMax).  result[0] = 1 on an edge out of range, | 2 on a row
+// of more than kHubEdges edges, result[1] = edges kept,
 // result[2 + l] = edges kept of the labels before l (l < counted).
 constexpr uint32_t kStageThreads = 1024;
 __global__ void __launch_bounds__(kStageThreads, 1)
@@ -2024,9 +2026,11 @@ __global__ void __launch_bounds__(kStageThreads, 1)
     uint32_t sum = 0u, total;
     for (uint32_t r = r0; r < r1; ++r) sum += cnt[r] & 0xFFFFu;
     uint32_t out = block_exclusive_scan(sum, &total), a = first;
+    bool hub = false;
     for (uint32_t r = r0; r < r1; ++r) {
         const uint32_t k = cnt[r] & 0xFFFFu, len = cnt[r] >> 16;
         csr_off[r] = out;
+        hub |= k > kHubEdges;
         if (r % n == 0u && r / n < counted) result[2u + r / n] = out;
         if (k == len)
             for (uint32_t i = 0; i < len; ++i) csr_col[out + i] = col[a + i];
@@ -2036,9 +2040,10 @@ __global__ void __launch_bounds__(kStageThreads, 1)
         out += k;
         a += len;
     }
+    hub = __syncthreads_or(hub) != 0;
     if (tid == 0) {
         csr_off[rows] = total;
-        result[0] = (uint32_t)bad;
+        result[0] = (bad ? 1u : 0u) | (hub ? 2u : 0u);
         result[1] = total;
     }
 }
@@ -2130,7 +2135,7 @@ int vpl_for_words(uint32_t W) {
 static int g_gather_sms[64];
 static int g_extract_ctas[64][kXClasses];  // CTAs of k_extract that a device holds at once, per row width
 
-cudaError_t launch_gather(int vpl, bool nt, const GItem *items, uint32_t n_items, const SrcDesc *srcs,
+cudaError_t launch_gather(int vpl, bool nt, bool hubs, const GItem *items, uint32_t n_items, const SrcDesc *srcs,
                           const ExecTables &T, int cls, cudaStream_t st) {
     if (n_items == 0) return cudaSuccess;
     int dev = 0;
@@ -2148,9 +2153,11 @@ cudaError_t launch_gather(int vpl, bool nt, const GItem *items, uint32_t n_items
         return std::max<uint32_t>(1u, std::min<uint32_t>(want, sms * (uint32_t)occ));
     };
 #define CFPQ_GATHER(V)                                                                                          \
-    if (nt) k_gather<V, true><<<grid_of(GatherDyn<V, true>::on, GatherCtas<V, true>::value), 256, GatherRing<V>::bytes, \
+    if (nt) k_gather<V, true, false><<<grid_of(GatherDyn<V, true>::on, GatherCtas<V, true>::value), 256, GatherRing<V>::bytes, \
                                 st>>>(items, srcs, T, cls);                                                     \
-    else k_gather<V, false><<<grid_of(false, GatherCtas<V, false>::value), 256, 0, st>>>(items, srcs, T, cls);
+    else if (hubs) k_gather<V, false, true><<<grid_of(false, GatherCtas<V, false>::value), 256, 0, st>>>(       \
+        items, srcs, T, cls);                                                                                   \
+    else k_gather<V, false, false><<<grid_of(false, GatherCtas<V, false>::value), 256, 0, st>>>(items, srcs, T, cls);
     switch (vpl) {
         case 1: CFPQ_GATHER(1) break;
         case 2: CFPQ_GATHER(2) break;
@@ -2208,7 +2215,7 @@ cudaError_t prepare_gather_launch() {
     }
 #define CFPQ_RING(V)                                                                                      \
     {                                                                                                     \
-        const cudaError_t e = cudaFuncSetAttribute(k_gather<V, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+        const cudaError_t e = cudaFuncSetAttribute(k_gather<V, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                                    (int)GatherRing<V>::bytes);                            \
         if (e != cudaSuccess) return e;                                                                   \
     }

@@ -135,7 +135,7 @@ extern "C" int cfpq_load_graph_device_noalloc(cfpq_ctx *ctx, uint32_t n, uint32_
         NA_CK(cudaMemcpyAsync(result, res, (2 + counted) * 4, cudaMemcpyDeviceToHost, st));
         NA_CK(cudaStreamSynchronize(st));
 #undef NA_CK
-        if (result[0]) {
+        if (result[0] & 1u) {
             g.n = 0;
             return fail(CFPQ_ERR_INVALID_ARG, "an edge names a vertex >= n_vertices or a label >= n_terminals");
         }

@@ -56,3 +56,23 @@ def test_shared_hubs(C, n, hubs, degs):
             assert (got == want[src]).all()
             ctx.run_sources(src)
             assert (ctx.reachable_words(0)[src] == full[src]).all()
+
+
+@pytest.mark.parametrize("n", [1030, 5000])
+def test_reloads_change_the_variant(C, n):
+    """One context, graphs of one shape with and without such rows in turn."""
+    import torch
+    few, src = _graph(n, 2, [400, 3], 1)
+    many, src2 = _graph(n, 2, [1000, 3], 2)
+    src = sorted(set(src) | set(src2))
+    with C.Context(no_single_cta=1, max_rounds=1 << 19) as ctx:
+        ctx.load_rsm(RSM)
+        for i, g in enumerate((few, many, few, many, many)):
+            if i % 2:
+                e = [torch.from_numpy(a.view(np.int32)).cuda() for a in (g.src, g.lbl, g.dst)]
+                ctx.load_graph_device(g.n, g.n_terminals, *e)
+            else:
+                ctx.load_graph(g)
+            ctx.run()
+            got = np.unpackbits(ctx.reachable_words(0)[src].view(np.uint8), axis=1, bitorder="little")[:, :n]
+            assert (got.astype(bool) == oracle.worklist(g, RSM, sources=src)[0][src]).all()

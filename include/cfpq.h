@@ -292,10 +292,10 @@ int cfpq_set_start(cfpq_ctx *ctx, const uint64_t *bits, uint32_t n_boxes, uint32
  * whose closure runs on a CPU Boolean-matrix library).  On the context's
  * device it runs a probe query -- Dyck-4 (S -> S S | o_i c_i | o_i S c_i)
  * on a seeded graph of 8192 vertices with Zipf(2.1) out-degrees (mean
- * about 3), 8 labels --
- * with the bit-packed closure and times its kernel groups with CUDA events,
- * times a dense product of two 8192 x 8192 0/1 matrices in each tile kernel and
- * reads of an L2-sized and an HBM-sized buffer, and derives: the fastest tile kernel (AUTO's default) and the
+ * about 3), 8 labels -- with the bit-packed closure and times its kernel
+ * groups with CUDA events, times a dense product of two 8192 x 8192 0/1
+ * matrices in each tile kernel and reads of an L2-sized and an HBM-sized
+ * buffer, and derives: the fastest tile kernel (AUTO's default) and the
  * cost-model ratio (new-edge tiles run while M * K < ratio x new edges),
  * searched around tile rate / (16 x gather rate) -- one new edge costs the
  * gather n/8 bytes, a tile product 2n multiply-adds per (row, column) of its

@@ -533,7 +533,7 @@ int QueryDev::plan(std::string *err) {
 // 16 edges a row 1.16, 24 1.00, 32 0.83; n = 8192 1.17, 1.02, 0.88; more than the SMs
 // hold: a+ n = 15000, 3 edges 1.26, 4 1.03, 6 0.84; n = 22700, 4 edges 1.08, 6 0.96;
 // (ab)*c|a*b* n = 8192, 4 edges a row of (ab)* 1.26, 6 1.00, 8 0.82, 33 0.46.  Few edges in
-// all never lose: n = 2000, 48 K edges 1.15 (a+), 1.38 (three labels).
+// all never lose: n = 2000, 48 K edges 1.20 (a+), 1.42 (three labels).
 uint64_t QueryDev::slice_edges(const SliceChoice &c) const {
     uint64_t e = 0;
     for (uint32_t l : c.labels) e += g->edges_of(l);
